@@ -228,13 +228,12 @@ sem3d_status solve_once_f64(sem3d_plan* p, const double* in, double* out, bool a
   double* B = reinterpret_cast<double*>(static_cast<char*>(p->ws) + align256(N * sizeof(double)));
   const Geom& g = p->g;
   const DevAxis* d = p->dev;
-  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 2, d[2].Tinv, in, A, EPI_STORE, nullptr, nullptr, nullptr, s));
-  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 1, d[1].Tinv, A, B, EPI_STORE, nullptr, nullptr, nullptr, s));
-  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 0, d[0].Tinv, B, A, EPI_DIV, d[0].lam, d[1].lam, d[2].lam, s));
-  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 2, d[2].T, A, B, EPI_STORE, nullptr, nullptr, nullptr, s));
-  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 1, d[1].T, B, A, EPI_STORE, nullptr, nullptr, nullptr, s));
-  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 0, d[0].T, A, out, accumulate ? EPI_ACCUM : EPI_STORE, nullptr, nullptr,
-                                   nullptr, s));
+  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 2, d, 0, in, A, EPI_STORE, p->num_sms, s));
+  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 1, d, 0, A, B, EPI_STORE, p->num_sms, s));
+  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 0, d, 0, B, A, EPI_DIV, p->num_sms, s));
+  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 2, d, 1, A, B, EPI_STORE, p->num_sms, s));
+  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 1, d, 1, B, A, EPI_STORE, p->num_sms, s));
+  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 0, d, 1, A, out, accumulate ? EPI_ACCUM : EPI_STORE, p->num_sms, s));
   return SEM3D_OK;
 }
 
@@ -378,8 +377,10 @@ sem3d_status sem3d_setup_bc(int nx, int ny, int nz, int k, double Lx, double Ly,
     D.n = A.n; D.k = k; D.Kp = pad16(A.n);
     sem3d_status st;
     if ((st = dev_upload(p.get(), &D.M, A.M.data(), A.M.size())) != SEM3D_OK) return st;
-    if ((st = dev_upload(p.get(), &D.T, A.T.data(), A.T.size())) != SEM3D_OK) return st;
-    if ((st = dev_upload(p.get(), &D.Tinv, A.Tinv.data(), A.Tinv.size())) != SEM3D_OK) return st;
+    D.ne = A.ne; D.no = A.no;
+    for (int w = 0; w < 2; ++w)
+      if ((st = dev_upload(p.get(), &D.par[w], A.par[w].data(), A.par[w].size())) != SEM3D_OK) return st;
+    if ((st = dev_upload(p.get(), &D.lam_par, A.lam_par.data(), A.lam_par.size())) != SEM3D_OK) return st;
     if ((st = dev_upload(p.get(), &D.lam, A.lam.data(), A.lam.size())) != SEM3D_OK) return st;
     std::vector<float> lf(A.lam.begin(), A.lam.end());
     if ((st = dev_upload(p.get(), &D.lamf, lf.data(), lf.size())) != SEM3D_OK) return st;
@@ -1013,16 +1014,16 @@ sem3d_status ch_step_core(sem3d_plan* h, const double* phi_n, const double* phi_
     double* B = reinterpret_cast<double*>(w + align256(N * sizeof(double)));
     double* R = reinterpret_cast<double*>(w + 2 * align256(N * sizeof(double)));
     LAUNCH(h, K_STENCIL, 1, s, launch_ch_prep(SEM3D_FP64, g, phi_n, phi_nm1, A, B, nb, nb, c, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 2, d[2].Tinv, A, R, EPI_STORE, nullptr, nullptr, nullptr, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 1, d[1].Tinv, R, A, EPI_STORE, nullptr, nullptr, nullptr, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 0, d[0].Tinv, A, R, EPI_STORE, nullptr, nullptr, nullptr, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 2, d[2].Tinv, B, A, EPI_STORE, nullptr, nullptr, nullptr, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 1, d[1].Tinv, A, B, EPI_STORE, nullptr, nullptr, nullptr, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 0, d[0].Tinv, B, A, EPI_STORE, nullptr, nullptr, nullptr, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 2, d, 0, A, R, EPI_STORE, h->num_sms, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 1, d, 0, R, A, EPI_STORE, h->num_sms, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 0, d, 0, A, R, EPI_STORE, h->num_sms, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 2, d, 0, B, A, EPI_STORE, h->num_sms, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 1, d, 0, A, B, EPI_STORE, h->num_sms, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 0, d, 0, B, A, EPI_STORE, h->num_sms, s));
     LAUNCH(h, K_STENCIL, 1, s, launch_ch_combine(SEM3D_FP64, g, d, R, A, B, nb, nb, nb, c, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 0, d[0].T, B, A, EPI_STORE, nullptr, nullptr, nullptr, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 1, d[1].T, A, R, EPI_STORE, nullptr, nullptr, nullptr, s));
-    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 2, d[2].T, R, phi_np1, EPI_STORE, nullptr, nullptr, nullptr, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 0, d, 1, B, A, EPI_STORE, h->num_sms, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 1, d, 1, A, R, EPI_STORE, h->num_sms, s));
+    LAUNCH(h, K_F64, 1, s, launch_mode_product_f64(g, 2, d, 1, R, phi_np1, EPI_STORE, h->num_sms, s));
   } else if (h->prec == SEM3D_FP32) {
     float* A = reinterpret_cast<float*>(w);
     float* B = reinterpret_cast<float*>(w + align256(N * sizeof(float)));
@@ -1607,13 +1608,13 @@ sem3d_status solve_once_f64_into(sem3d_plan* p, const double* in, double* out, b
                                  cudaStream_t s) {
   const Geom& g = p->g;
   const DevAxis* d = p->dev;
-  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 2, d[2].Tinv, in, A, EPI_STORE, nullptr, nullptr, nullptr, s));
-  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 1, d[1].Tinv, A, B, EPI_STORE, nullptr, nullptr, nullptr, s));
-  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 0, d[0].Tinv, B, A, EPI_DIV, d[0].lam, d[1].lam, d[2].lam, s));
-  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 2, d[2].T, A, B, EPI_STORE, nullptr, nullptr, nullptr, s));
-  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 1, d[1].T, B, A, EPI_STORE, nullptr, nullptr, nullptr, s));
+  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 2, d, 0, in, A, EPI_STORE, p->num_sms, s));
+  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 1, d, 0, A, B, EPI_STORE, p->num_sms, s));
+  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 0, d, 0, B, A, EPI_DIV, p->num_sms, s));
+  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 2, d, 1, A, B, EPI_STORE, p->num_sms, s));
+  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 1, d, 1, B, A, EPI_STORE, p->num_sms, s));
   LAUNCH_COUNTED(p, 1,
-         launch_mode_product_f64(g, 0, d[0].T, A, out, accumulate ? EPI_ACCUM : EPI_STORE, nullptr, nullptr, nullptr, s));
+         launch_mode_product_f64(g, 0, d, 1, A, out, accumulate ? EPI_ACCUM : EPI_STORE, p->num_sms, s));
   return SEM3D_OK;
 }
 

@@ -128,8 +128,8 @@ cudaError_t launch_ch_combine(int tier, const Geom& g, const DevAxis* ax, const 
   const long long N = (long long)g.nx * g.ny * g.nz;
   if (tier == SEM3D_FP64) {
     ch_combine_kernel<double><<<ch_grid(N), CH_THREADS, 0, s>>>(
-        static_cast<const double*>(a1), static_cast<const double*>(a2), static_cast<double*>(out), ax[0].lam,
-        ax[1].lam, ax[2].lam, g.nx, g.ny, N, c);
+        static_cast<const double*>(a1), static_cast<const double*>(a2), static_cast<double*>(out),
+        ax[0].lam_par, ax[1].lam_par, ax[2].lam_par, g.nx, g.ny, N, c);  // FP64 transforms order the modes by parity
   } else if (tier == SEM3D_FP32) {
     ch_combine_kernel<float><<<ch_grid(N), CH_THREADS, 0, s>>>(
         static_cast<const float*>(a1), static_cast<const float*>(a2), static_cast<float*>(out), ax[0].lam,

@@ -14,110 +14,177 @@ namespace {
 // index has stride sm, so the same kernel serves x, y and z without
 // transposes (Section 2.4, Eq. 11: the paper's tensorprod / pagemtimes).
 //
-// CTA tile: 64 rows x 64 outputs, K chunk 16; 8 warps, each owning 32 rows x
-// 16 outputs = 4 x 2 fragments of mma.m8n8k4.f64.
+// The FP64 pipe bounds it (1.05 TF/s on this GPU, reached at n = 255), so W is
+// taken in its parity blocks (Axis1D::par), which halves the multiply-adds:
+// forward, the A tiles are the half sums and half differences of a line,
+// formed as they are loaded, and the outputs are the modes, even ones first;
+// backward, the A tiles are the two halves of the modes and the epilogue
+// writes E + O and E - O to the mirrored nodes.  A CTA computes BM rows x
+// (32 even + 32 odd) outputs in K chunks of 16 + 16; the next chunk's loads
+// are in flight while the current one is multiplied.  8 warps, each owning
+// BM/2 rows x (8 even + 8 odd) outputs, i.e. BM/16 x 2 fragments of
+// mma.m8n8k4.f64.  Measured per pass: n = 255 8.0 ms (full matrices) -> 4.0;
+// n = 63 88 us (full matrices, 64-row tiles) -> 25.
 
-constexpr int F64_BM = 64, F64_BN = 64, F64_BK = 16;
+constexpr int F64_BN = 32, F64_BK = 16;  // outputs and K of one parity per CTA and chunk
 
 struct F64Pass {
   const double* in;
   double* out;
-  const double* W;        // n x n row-major
+  const double* W;        // even block (ne x ne row-major), then the odd one (no x no)
   long long s1, s2, sm;   // strides of p, q and the axis index
-  int R1, R2, n;          // row loops and axis length
+  int R1, R2, n, ne, no;  // row loops and axis length
   int epi;
   int nx, ny;             // to decode (i, j, l) for the division epilogue
-  const double *lamx, *lamy, *lamz;
+  const double *lamx, *lamy, *lamz;  // mode order (even modes first)
   double c;
 };
 
-template <bool KCONTIG>
+template <bool KCONTIG, bool FWD, int BM>
 __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
-  __shared__ double As[F64_BK][F64_BM + 1];
-  __shared__ double Bs[F64_BK][F64_BN + 1];
+  constexpr int AF = BM / 16;                    // fragments of 8 rows per warp
+  constexpr int LA = BM * F64_BK / 256;          // (even, odd) A pairs loaded per thread and chunk
+  constexpr int LW = 2 * F64_BN * F64_BK / 256;  // W entries loaded per thread and chunk
+  __shared__ double As[2][F64_BK][BM + 1];       // [parity]
+  __shared__ double Bs[2][F64_BK][F64_BN + 1];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long rows = (long long)p.R1 * p.R2;
-  const long long row0 = (long long)blockIdx.x * F64_BM;
+  const long long row0 = (long long)blockIdx.x * BM;
   const int o0 = blockIdx.y * F64_BN;
-  const int wr = (warp & 1) * 32, wc = (warp >> 1) * 16;
+  const int wr = (warp & 1) * (BM / 2), wc = (warp >> 1) * 8;
 
-  double acc[4][2][2];
+  // The rows this thread loads are the same in every chunk.
+  const double* abase[LA];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int it = 0; it < LA; ++it) {
+    const int e = tid + it * 256;
+    const long long row = row0 + (KCONTIG ? e / F64_BK : e % BM);
+    abase[it] = row < rows ? p.in + (row % p.R1) * p.s1 + (row / p.R1) * p.s2 : nullptr;
+  }
+  double ra[LA][2], rw[LW];
+  auto load = [&](int t0) {
+#pragma unroll
+    for (int it = 0; it < LA; ++it) {
+      const int e = tid + it * 256;
+      const int t = t0 + (KCONTIG ? e % F64_BK : e / BM);
+      double u = 0.0, v = 0.0;
+      if (abase[it] && t < p.ne) {
+        u = abase[it][(long long)t * p.sm];
+        if (t < p.no) v = abase[it][(long long)(FWD ? p.n - 1 - t : p.ne + t) * p.sm];
+      }
+      // the middle node of an odd n (t = no) has no partner: v = 0 and the
+      // odd block has no such column
+      ra[it][0] = FWD ? u + v : u;
+      ra[it][1] = FWD ? (t < p.no ? u - v : 0.0) : v;
+    }
+#pragma unroll
+    for (int it = 0; it < LW; ++it) {
+      const int e = tid + it * 256;
+      const int kk = e % F64_BK, o = o0 + (e / F64_BK) % F64_BN, par = e / (F64_BK * F64_BN);
+      const int t = t0 + kk, m = par == 0 ? p.ne : p.no;
+      rw[it] = (o < m && t < m) ? __ldg(p.W + (par == 0 ? 0 : (long long)p.ne * p.ne) + (long long)o * m + t) : 0.0;
+    }
+  };
+  auto store = [&]() {
+#pragma unroll
+    for (int it = 0; it < LA; ++it) {
+      const int e = tid + it * 256;
+      const int kk = KCONTIG ? e % F64_BK : e / BM, r = KCONTIG ? e / F64_BK : e % BM;
+      As[0][kk][r] = ra[it][0];
+      As[1][kk][r] = ra[it][1];
+    }
+#pragma unroll
+    for (int it = 0; it < LW; ++it) {
+      const int e = tid + it * 256;
+      Bs[e / (F64_BK * F64_BN)][e % F64_BK][(e / F64_BK) % F64_BN] = rw[it];
+    }
+  };
+
+  double acc[AF][2][2];  // [fragment][parity][column]
+#pragma unroll
+  for (int a = 0; a < AF; ++a)
 #pragma unroll
     for (int b = 0; b < 2; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
 
-  for (int t0 = 0; t0 < p.n; t0 += F64_BK) {
-    // A tile: 64 rows x 16 t.
-#pragma unroll
-    for (int it = 0; it < (F64_BM * F64_BK) / 256; ++it) {
-      const int e = tid + it * 256;
-      int r, kk;
-      if (KCONTIG) { kk = e % F64_BK; r = e / F64_BK; }
-      else { r = e % F64_BM; kk = e / F64_BM; }
-      const long long row = row0 + r;
-      const int t = t0 + kk;
-      double v = 0.0;
-      if (row < rows && t < p.n) {
-        const long long pp = row % p.R1, qq = row / p.R1;
-        v = p.in[pp * p.s1 + qq * p.s2 + (long long)t * p.sm];
-      }
-      As[kk][r] = v;
-    }
-    // W tile: 64 outputs x 16 t (row-major W, t contiguous).
-#pragma unroll
-    for (int it = 0; it < (F64_BN * F64_BK) / 256; ++it) {
-      const int e = tid + it * 256;
-      const int kk = e % F64_BK, o = e / F64_BK;
-      const int oo = o0 + o, t = t0 + kk;
-      Bs[kk][o] = (oo < p.n && t < p.n) ? p.W[(long long)oo * p.n + t] : 0.0;
-    }
+  load(0);
+  for (int t0 = 0; t0 < p.ne; t0 += F64_BK) {
+    store();
     __syncthreads();
+    if (t0 + F64_BK < p.ne) load(t0 + F64_BK);
 #pragma unroll
     for (int k4 = 0; k4 < F64_BK; k4 += 4) {
-      double afr[4], bfr[2];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) afr[a] = As[k4 + (lane & 3)][wr + a * 8 + (lane >> 2)];
+      for (int b = 0; b < 2; ++b) {
+        const double bfr = Bs[b][k4 + (lane & 3)][wc + (lane >> 2)];
 #pragma unroll
-      for (int b = 0; b < 2; ++b) bfr[b] = Bs[k4 + (lane & 3)][wc + b * 8 + (lane >> 2)];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
+        for (int a = 0; a < AF; ++a) {
+          const double afr = As[b][k4 + (lane & 3)][wr + a * 8 + (lane >> 2)];
           asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};\n"
                        : "+d"(acc[a][b][0]), "+d"(acc[a][b][1])
-                       : "d"(afr[a]), "d"(bfr[b]));
+                       : "d"(afr), "d"(bfr));
+        }
+      }
     }
     __syncthreads();
   }
-  // Epilogue: fragment (a, b) holds rows wr + a*8 + lane/4, outputs
-  // wc + b*8 + 2*(lane%4) + {0,1}.
+  // Epilogue: fragment a holds rows wr + a*8 + lane/4, outputs
+  // wc + 2*(lane%4) + {0,1} of both parities.
+  auto put = [&](long long base, int o, double v) {
+    const long long idx = base + (long long)o * p.sm;
+    if (p.epi == EPI_DIV) {
+      const long long i = idx % p.nx, jl = idx / p.nx;
+      const long long j = jl % p.ny, l = jl / p.ny;
+      p.out[idx] = v / (p.lamx[i] + p.lamy[j] + p.lamz[l] + p.c);
+    } else if (p.epi == EPI_ACCUM) {
+      p.out[idx] += v;
+    } else {
+      p.out[idx] = v;
+    }
+  };
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
+  for (int a = 0; a < AF; ++a) {
     const long long row = row0 + wr + a * 8 + (lane >> 2);
     if (row >= rows) continue;
-    const long long pp = row % p.R1, qq = row / p.R1;
-    const long long base = pp * p.s1 + qq * p.s2;
+    const long long base = (row % p.R1) * p.s1 + (row / p.R1) * p.s2;
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int o = o0 + wc + b * 8 + 2 * (lane & 3) + h;
-        if (o >= p.n) continue;
-        const long long idx = base + (long long)o * p.sm;
-        double v = acc[a][b][h];
-        if (p.epi == EPI_DIV) {
-          const long long i = idx % p.nx, jl = idx / p.nx;
-          const long long j = jl % p.ny, l = jl / p.ny;
-          v = v / (p.lamx[i] + p.lamy[j] + p.lamz[l] + p.c);
-          p.out[idx] = v;
-        } else if (p.epi == EPI_ACCUM) {
-          p.out[idx] += v;
-        } else {
-          p.out[idx] = v;
-        }
+    for (int h = 0; h < 2; ++h) {
+      const int o = o0 + wc + 2 * (lane & 3) + h;
+      if (o >= p.ne) continue;
+      const double e = acc[a][0][h], d = acc[a][1][h];
+      if (o >= p.no) {  // the middle of an odd n
+        put(base, o, e);
+      } else if (FWD) {
+        put(base, o, e);
+        put(base, p.ne + o, d);
+      } else {
+        put(base, o, e + d);
+        put(base, p.n - 1 - o, e - d);
       }
+    }
   }
+}
+
+template <bool KCONTIG, bool FWD>
+cudaError_t launch_f64(const F64Pass& p, int num_sms, cudaStream_t s) {
+  // Rows per CTA: the CTAs of an SM share its FP64 pipe, so a pass takes as
+  // long as the SM with the most rows; the largest tile within that minimum.
+  // (n = 63: 125 tiles of 32 rows, one per SM at most, instead of 62 of 64.)
+  const long long rows = (long long)p.R1 * p.R2;
+  const long long nt = (p.ne + F64_BN - 1) / F64_BN;
+  int best = 64;
+  long long best_cost = 0;
+  for (int bm : {64, 32, 16}) {
+    const long long blocks = (rows + bm - 1) / bm * nt;
+    const long long cost = (blocks + num_sms - 1) / num_sms * bm;
+    if (bm == 64 || cost < best_cost) { best = bm; best_cost = cost; }
+  }
+  const long long bx = (rows + best - 1) / best;
+  if (bx >= (1LL << 31)) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)bx, (unsigned)nt);
+  if (best == 64) mode_product_f64_kernel<KCONTIG, FWD, 64><<<grid, 256, 0, s>>>(p);
+  else if (best == 32) mode_product_f64_kernel<KCONTIG, FWD, 32><<<grid, 256, 0, s>>>(p);
+  else mode_product_f64_kernel<KCONTIG, FWD, 16><<<grid, 256, 0, s>>>(p);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ stencil
@@ -705,33 +772,33 @@ int grid_for(long long work, int per_block) {
 
 }  // namespace
 
-cudaError_t launch_mode_product_f64(const Geom& g, int axis, const double* W, const double* in, double* out, int epi,
-                                    const double* lamx, const double* lamy, const double* lamz, cudaStream_t s) {
+cudaError_t launch_mode_product_f64(const Geom& g, int axis, const DevAxis* ax, int which, const double* in,
+                                    double* out, int epi, int num_sms, cudaStream_t s) {
   F64Pass p{};
   p.in = in;
   p.out = out;
-  p.W = W;
+  p.W = ax[axis].par[which];
+  p.n = ax[axis].n;
+  p.ne = ax[axis].ne;
+  p.no = ax[axis].no;
   p.epi = epi;
   p.nx = g.nx;
   p.ny = g.ny;
-  p.lamx = lamx;
-  p.lamy = lamy;
-  p.lamz = lamz;
+  p.lamx = ax[0].lam_par;
+  p.lamy = ax[1].lam_par;
+  p.lamz = ax[2].lam_par;
   p.c = g.c;
   const long long nxy = (long long)g.nx * g.ny;
   bool kcontig = false;
   if (axis == 0) {         // rows = (j,l) lines, t = i contiguous
-    p.R1 = g.ny * g.nz; p.R2 = 1; p.s1 = g.nx; p.s2 = 0; p.sm = 1; p.n = g.nx; kcontig = true;
+    p.R1 = g.ny * g.nz; p.R2 = 1; p.s1 = g.nx; p.s2 = 0; p.sm = 1; kcontig = true;
   } else if (axis == 1) {  // rows = (i, l), t = j
-    p.R1 = g.nx; p.R2 = g.nz; p.s1 = 1; p.s2 = nxy; p.sm = g.nx; p.n = g.ny;
+    p.R1 = g.nx; p.R2 = g.nz; p.s1 = 1; p.s2 = nxy; p.sm = g.nx;
   } else {                 // rows = (i,j) plane, t = l
-    p.R1 = (int)nxy; p.R2 = 1; p.s1 = 1; p.s2 = 0; p.sm = nxy; p.n = g.nz;
+    p.R1 = (int)nxy; p.R2 = 1; p.s1 = 1; p.s2 = 0; p.sm = nxy;
   }
-  const long long rows = (long long)p.R1 * p.R2;
-  dim3 grid((unsigned)((rows + F64_BM - 1) / F64_BM), (unsigned)((p.n + F64_BN - 1) / F64_BN));
-  if (kcontig) mode_product_f64_kernel<true><<<grid, 256, 0, s>>>(p);
-  else mode_product_f64_kernel<false><<<grid, 256, 0, s>>>(p);
-  return cudaGetLastError();
+  if (which == 0) return kcontig ? launch_f64<true, true>(p, num_sms, s) : launch_f64<false, true>(p, num_sms, s);
+  return kcontig ? launch_f64<true, false>(p, num_sms, s) : launch_f64<false, false>(p, num_sms, s);
 }
 
 cudaError_t launch_stencil(const Geom& g, int k, const DevAxis* ax, const double* u, const double* f, double* out64,

@@ -83,6 +83,20 @@ struct Axis1D {
   // Hq[q*(2k+1) + d + k] = H[g][g+d], including the columns of the two
   // boundary nodes (their values are zero, so those entries are never used).
   std::vector<double> Hq;
+  // Parity form of the eigenbasis.  The mesh is symmetric about the middle of
+  // the axis, so every eigenvector is even or odd under i -> n-1-i: with the
+  // ne = ceil(n/2) even modes first and the no = floor(n/2) odd ones after
+  // them, a product with T^{-1} needs only the half sums v_t + v_{n-1-t} (even
+  // modes) and half differences v_t - v_{n-1-t} (odd modes), t < ne / no (the
+  // middle node of an odd n stands alone in the even half), and a product with
+  // T gives u_t = E_t + O_t, u_{n-1-t} = E_t - O_t.  Half the operations of
+  // the full matrices (Solomonoff 1992 calls it even-odd decomposition).
+  //   par[0] = T^{-1}, par[1] = T, each the even block (ne x ne row-major)
+  //   followed by the odd block (no x no); forward rows are modes, backward
+  //   rows are nodes.  lam_par: eigenvalues in the same order of modes.
+  int ne = 0, no = 0;
+  std::vector<double> par[2];
+  std::vector<double> lam_par;
 };
 
 void gll_rule(int N, std::vector<double>& r, std::vector<double>& w);
@@ -99,9 +113,10 @@ inline int pad16(int n) { return (n + 15) & ~15; }
 struct DevAxis {
   int n = 0, k = 0, Kp = 0;     // Kp = pad16(n): row pitch of the bf16 matrices
   double* M = nullptr;          // FP64 lumped mass diagonal (n)
-  double* T = nullptr;          // FP64 n x n row-major (W[out][in] for the backward pass)
-  double* Tinv = nullptr;       // FP64 n x n row-major (W[out][in] for the forward pass)
   double* lam = nullptr;        // FP64 eigenvalues
+  int ne = 0, no = 0;           // even and odd modes (see Axis1D::par)
+  double* par[2] = {nullptr, nullptr};  // FP64 even block, then odd block: [0] = T^{-1}, [1] = T
+  double* lam_par = nullptr;    // FP64 eigenvalues, even modes first
   float* lamf = nullptr;        // FP32 copy for the low-precision epilogues
   double* Hband = nullptr;      // FP64 n x (2k+1)
   double* Hq = nullptr;         // FP64 k x (2k+1) per-local-index rows of H (x axis: + c on the diagonal)
@@ -172,10 +187,11 @@ struct Geom {
 
 // ---- FP64 kernels (fp64_kernels.cu)
 // One mode product along `axis` (0 = x, 1 = y, 2 = z) on dense n-pitch FP64
-// arrays: out[.., o, ..] (=|+=|/=) sum_t W[o*n + t] * in[.., t, ..].
-cudaError_t launch_mode_product_f64(const Geom& g, int axis, const double* W, const double* in, double* out,
-                                    int epi, const double* lamx, const double* lamy, const double* lamz,
-                                    cudaStream_t s);
+// arrays with the parity blocks of T^{-1} (which = 0: nodes -> modes, even
+// modes first) or T (which = 1: modes -> nodes).  EPI_DIV divides by
+// lam_x + lam_y + lam_z + c, all three axes being in mode order.
+cudaError_t launch_mode_product_f64(const Geom& g, int axis, const DevAxis* ax, int which, const double* in,
+                                    double* out, int epi, int num_sms, cudaStream_t s);
 // ---- FP32 CUDA-core kernels (fp32_kernels.cu)
 // One mode product in FP32 arithmetic; `in` is FP64 (first pass) or FP32,
 // `out` FP64 (last pass, EPI_STORE or EPI_ACCUM) or FP32.

@@ -210,6 +210,79 @@ void sym_eig(int n, std::vector<double>& A, std::vector<double>& d, std::vector<
   }
 }
 
+// Parity form of the eigenbasis (see Axis1D::par) from the eigenvectors Q of
+// S1 = M^{-1/2} S M^{-1/2}.  An eigenvector's part of the wrong parity is rounding of the eigen-
+// solver (~eps * lambda_max / gap); it is dropped when it is below 1e-9 of the
+// vector, so that the blocks' orthogonality is touched at 1e-18.  Where an
+// even and an odd eigenvalue nearly coincide the solver may return mixtures of
+// the two vectors: then each half problem is diagonalised by itself.
+void build_parity(Axis1D& ax, const std::vector<double>& Q) {
+  const int n = ax.n, no = n / 2, ne = n - no;
+  ax.ne = ne;
+  ax.no = no;
+  std::vector<double> half[2];  // [t * count + mode]: components t of the modes of one parity
+  half[0].assign((size_t)ne * ne, 0.0);
+  half[1].assign((size_t)no * no, 0.0);
+  ax.lam_par.assign(n, 0.0);
+  int cnt[2] = {0, 0};
+  bool pure = true;
+  for (int j = 0; j < n && pure; ++j) {
+    double even = 0.0, odd = 0.0;  // squared norms of the two parts
+    for (int i = 0; i < n; ++i) {
+      const double a = Q[(size_t)i * n + j], b = Q[(size_t)(n - 1 - i) * n + j];
+      even += 0.25 * (a + b) * (a + b);
+      odd += 0.25 * (a - b) * (a - b);
+    }
+    const int w = even >= odd ? 0 : 1, m = w == 0 ? ne : no;
+    pure = std::min(even, odd) <= 1e-18 && cnt[w] < m;
+    if (!pure) break;
+    for (int t = 0; t < m; ++t) {
+      const double a = Q[(size_t)t * n + j], b = Q[(size_t)(n - 1 - t) * n + j];
+      half[w][(size_t)t * m + cnt[w]] = 0.5 * (w == 0 ? a + b : a - b);
+    }
+    ax.lam_par[(w == 0 ? 0 : ne) + cnt[w]++] = ax.lam[j];
+  }
+  if (!pure) {
+    const double r2 = std::sqrt(2.0);
+    auto s1 = [&](int i, int j) {  // S1 = M^{-1/2} S M^{-1/2}
+      return 0.5 * (ax.S[(size_t)i * n + j] + ax.S[(size_t)j * n + i]) / std::sqrt(ax.M[i] * ax.M[j]);
+    };
+    for (int w = 0; w < 2; ++w) {
+      const int m = w == 0 ? ne : no;
+      if (m == 0) continue;
+      std::vector<double> A((size_t)m * m), lam, V;
+      for (int t = 0; t < m; ++t)
+        for (int s = 0; s < m; ++s) {
+          const bool mt = 2 * t == n - 1, ms = 2 * s == n - 1;  // the middle node
+          const double a = s1(t, s), b = s1(t, n - 1 - s);
+          A[(size_t)t * m + s] = mt && ms ? a : (mt || ms) ? r2 * a : (w == 0 ? a + b : a - b);
+        }
+      for (int t = 0; t < m; ++t)
+        for (int s = t + 1; s < m; ++s)
+          A[(size_t)t * m + s] = A[(size_t)s * m + t] = 0.5 * (A[(size_t)t * m + s] + A[(size_t)s * m + t]);
+      sym_eig(m, A, lam, V);
+      for (int t = 0; t < m; ++t)
+        for (int j = 0; j < m; ++j)
+          half[w][(size_t)t * m + j] = 2 * t == n - 1 ? V[(size_t)t * m + j] : V[(size_t)t * m + j] / r2;
+      for (int j = 0; j < m; ++j) ax.lam_par[(w == 0 ? 0 : ne) + j] = lam[j];
+    }
+  }
+  for (auto& b : ax.par) b.assign((size_t)ne * ne + (size_t)no * no, 0.0);
+  for (int w = 0; w < 2; ++w) {
+    const int m = w == 0 ? ne : no;
+    double* fwd = ax.par[0].data() + (w == 0 ? 0 : (size_t)ne * ne);
+    double* bwd = ax.par[1].data() + (w == 0 ? 0 : (size_t)ne * ne);
+    for (int t = 0; t < m; ++t) {
+      const double sm = std::sqrt(ax.M[t]);
+      for (int j = 0; j < m; ++j) {
+        const double q = half[w][(size_t)t * m + j];
+        fwd[(size_t)j * m + t] = q * sm;
+        bwd[(size_t)t * m + j] = q / sm;
+      }
+    }
+  }
+}
+
 }  // namespace
 
 // Build the axis data of degree k on [0, L]: n interior nodes (Dirichlet,
@@ -285,6 +358,7 @@ Axis1D build_axis(int n, int k, double L, int bc) {
       ax.Tinv[(size_t)j * n + i] = Q[(size_t)i * n + j] * sm;
     }
   }
+  build_parity(ax, Q);
   // Band of H = M^{-1} S: row i couples columns [lo_i, hi_i] (one or two
   // elements), stored as H[i][i+d] for d in [-k, k].
   const int bw = 2 * k + 1;
