@@ -57,6 +57,7 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
 struct TcArgs {
   int m_tiles, n_tiles, batches, k_blocks;
   int kc;              // K blocks per TMEM accumulation chunk (see the kernel)
+  int bn;              // outputs per tile of the pair kernel: a multiple of 32, <= BN (see tile_outputs)
   int rows;            // valid tile rows per batch (x: ny*nz, y: Px, z: Px*ny)
   int nout;            // valid outputs (length of the output axis)
   int nx, ny, nz, Px;
@@ -81,8 +82,24 @@ struct TcGroupEntry {
   CUtensorMap A_hi, A_lo, B_hi, B_lo;  // 64-byte aligned (CUtensorMap's alignment)
   TcArgs a;
   int tile0;            // first pair tile of this problem in the launch
-  int tiles_per_batch;  // pair tiles per batch (page) of this problem
 };
+
+// Outputs per pair tile for an output axis of n: the fewest tiles of at most
+// BN outputs, each no wider than it has to be.  The MMA's time goes with its
+// N, so n = 383 runs as 2 x 192 instead of 2 x 256, n = 127 as 128.  With the
+// flattened M tiles below: 16 uneven problems (n = 63..511, refined) 58.3 ->
+// 55.0 ms, a 383^3 PCG solve 53.8 -> 51.4 ms, 449x320x383 7.25 -> 6.99 ms.
+inline int tile_outputs(int n) {
+  const int tiles = (n + BN - 1) / BN;
+  return ((n + tiles - 1) / tiles + 31) & ~31;
+}
+
+// Pair tiles of a pass.  The two CTAs of a pair take consecutive 128-row
+// tiles of the flattened (batch, M tile) sequence, so a page of the y pass
+// with an odd number of M tiles shares its last pair with the next page.
+inline long long pair_tiles(const TcArgs& a) {
+  return ((long long)a.m_tiles * a.batches + 1) / 2 * a.n_tiles;
+}
 
 // Output modes of the epilogue.  The DF modes (y and z passes only) keep the
 // solution as a double-FP32 pair u = hi + lo between refinement sweeps:

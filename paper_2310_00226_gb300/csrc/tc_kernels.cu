@@ -537,10 +537,10 @@ cudaError_t prepare_pass(const Geom& g, int axis, const DevAxis& W, int which, T
   }
   {
     // W: dims {t: n, o: n}, row pitch Kp*2 B; box {BK (K), BN/CLUSTER rows}
-    // (pair kernel: BN/2 rows, each CTA of the pair stages half of the tile)
+    // (pair kernel: bn/2 rows, each CTA of the pair stages half of the tile)
     const uint64_t dims[2] = {(uint64_t)W.n, (uint64_t)W.n};
     const uint64_t str[1] = {(uint64_t)W.Kp * 2};
-    const uint32_t box[2] = {BK, (uint32_t)(pair ? BN / 2 : BN / CLUSTER)};
+    const uint32_t box[2] = {BK, (uint32_t)(pair ? tile_outputs(W.n) / 2 : BN / CLUSTER)};
     const void* wh = fmt ? (const void*)W.W16_hi[which] : (const void*)W.W_hi[which];
     const void* wl = fmt ? (const void*)W.W16_lo[which] : (const void*)W.W_lo[which];
     ok = ok && make_map(&ps.mBh, wh, 2, dims, str, box, SWZ_K) && make_map(&ps.mBl, wl, 2, dims, str, box, SWZ_K);
@@ -548,7 +548,8 @@ cudaError_t prepare_pass(const Geom& g, int axis, const DevAxis& W, int which, T
   if (!ok) return cudaErrorInvalidValue;
   a.nout = W.n;
   a.m_tiles = (a.rows + BM - 1) / BM;
-  a.n_tiles = (W.n + BN - 1) / BN;
+  a.bn = pair ? tile_outputs(W.n) : BN;
+  a.n_tiles = (W.n + a.bn - 1) / a.bn;
   a.k_blocks = (nin + BK - 1) / BK;
   a.kc = (fmt == 1 && SEM3D_TC_CHUNK_KBLOCKS > 0) ? SEM3D_TC_CHUNK_KBLOCKS : a.k_blocks;
   return cudaSuccess;
@@ -569,7 +570,7 @@ cudaError_t launch_mode_product_bf16x3(const Geom& g, int axis, const DevAxis& W
   TcArgs& a = ps.a;
   a.stall = tc_take_stall();
   if (pair) {
-    const long long work = (long long)((a.m_tiles + 1) / 2) * a.n_tiles * a.batches;
+    const long long work = pair_tiles(a);
     if (work >= (1LL << 31)) return cudaErrorInvalidValue;
     return launch_pair_pass(axis, nprod, ps, work, num_sms, s);
   }

@@ -17,10 +17,11 @@ using namespace tcx;
 // ---------------------------------------------------------------- CTA-pair kernel
 //
 // The same mode product with one MMA per pair of SMs (tcgen05 cta_group::2):
-// a cluster of 2 CTAs owns a 256-row x 256-output tile.  CTA r of the pair
-// stages rows [128 r, 128 r + 128) of the A tile and rows [128 r, 128 r + 128)
-// of the W tile, so a stage holds 32 KB per CTA instead of 48 KB (6 stages fit
-// where 4 did) and each SM loads half of W without multicast.  The leader CTA
+// a cluster of 2 CTAs owns a 256-row x bn-output tile (bn <= 256, see
+// tile_outputs).  CTA r of the pair stages its own 128 rows of A and rows
+// [r bn/2, (r + 1) bn/2) of the W tile, so a stage holds 32 KB per CTA instead
+// of 48 KB (6 stages fit where 4 did) and each SM loads half of W without
+// multicast.  The leader CTA
 // (rank 0) issues M = 256 MMAs that read A and W from both CTAs' shared memory
 // at the same offsets and accumulate rows 128 r .. 128 r + 127 of the tile in
 // CTA r's tensor memory.  Both CTAs' TMA loads complete on the leader's "full"
@@ -46,24 +47,22 @@ __device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, u
 }
 
 // One pair tile handed to the kernel body: the problem's arguments and tensor
-// maps, and the tile's (batch, M pair, N tile) within that problem.
+// maps, and the tile's (pair of flattened M tiles, N tile) within that problem.
 struct PairTile {
   const TcArgs* a;
   const CUtensorMap *Ah, *Al, *Bh, *Bl;
-  int b, mp, nt;
+  int mp, nt;
 };
 
 // Tile source of a launch for one problem: the kernel's own parameters.
 struct OneProblem {
   const CUtensorMap *Ah, *Al, *Bh, *Bl;
   const TcArgs* a;
-  int tiles_per_batch, total;
+  int total;
   __device__ __forceinline__ void at(int pt, int& /*cursor*/, PairTile& t) const {
     t.a = a; t.Ah = Ah; t.Al = Al; t.Bh = Bh; t.Bl = Bl;
-    t.b = pt / tiles_per_batch;
-    const int rem = pt - t.b * tiles_per_batch;
-    t.mp = rem / a->n_tiles;
-    t.nt = rem - t.mp * a->n_tiles;
+    t.mp = pt / a->n_tiles;
+    t.nt = pt - t.mp * a->n_tiles;
   }
 };
 
@@ -78,10 +77,8 @@ struct ProblemGroup {
     const TcGroupEntry& e = tab[cursor];
     t.a = &e.a; t.Ah = &e.A_hi; t.Al = &e.A_lo; t.Bh = &e.B_hi; t.Bl = &e.B_lo;
     const int local = pt - e.tile0;
-    t.b = local / e.tiles_per_batch;
-    const int rem = local - t.b * e.tiles_per_batch;
-    t.mp = rem / e.a.n_tiles;
-    t.nt = rem - t.mp * e.a.n_tiles;
+    t.mp = local / e.a.n_tiles;
+    t.nt = local - t.mp * e.a.n_tiles;
   }
 };
 
@@ -99,7 +96,6 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
   auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * P_STAGES + 2 + b); };
   const uint32_t drain_bar = bar0 + 8u * (2 * P_STAGES + 4);
   constexpr uint16_t kPair = 3;  // both CTAs of the pair
-  constexpr int ROWS_B = BN / 2;  // rows of the W tile this CTA stages
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr bool a_mn = (PASS != 0);
@@ -124,9 +120,9 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
 
-  // Pair tile pt -> (problem, batch b, M pair mp, N tile nt); this CTA's M
-  // tile is 2 mp + rank (past the problem's last M tile, TMA reads zeros and
-  // nothing is stored).
+  // Pair tile pt -> (problem, M pair mp, N tile nt); this CTA's flattened M
+  // tile is 2 mp + rank, i.e. M tile mt of batch b (past the problem's last
+  // one, TMA reads zeros and nothing is stored).
   const int total_pt = src.total;
   PairTile t;
   if (warp == 0 && lane == 0) {
@@ -136,7 +132,9 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
     bool ok = true;
     for (int pt = pid; pt < total_pt && ok && !stall; pt += npairs) {
       src.at(pt, cursor, t);
-      const int m0 = (2 * t.mp + rank) * BM, n0 = t.nt * BN + rank * ROWS_B;
+      const int mf = 2 * t.mp + rank;
+      const int b = PASS == 1 ? mf / t.a->m_tiles : 0;
+      const int m0 = (mf - b * t.a->m_tiles) * BM, bn = t.a->bn, n0 = t.nt * bn + rank * (bn / 2);
       const int k_blocks = t.a->k_blocks;
       for (int kb = 0; kb < k_blocks; ++kb, ++it) {
         const int s = it % P_STAGES;
@@ -147,17 +145,17 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
         const uint32_t b_hi = st + 2 * A_TILE_BYTES, b_lo = b_hi + P_B_TILE_BYTES;
         const uint32_t fb = full_leader0 + 8u * s;  // the leader's full barrier of stage s
         if (rank == 0)
-          mbar_arrive_expect_tx(full_bar(s), 2 * (NP == 3 ? P_STAGE_BYTES : A_TILE_BYTES + P_B_TILE_BYTES));
+          mbar_arrive_expect_tx(full_bar(s), (NP == 3 ? 4 : 2) * A_TILE_BYTES + (NP == 3 ? 2 : 1) * bn * (BK * 2));
         const int k0 = kb * BK;
         if (PASS == 0) {
           tma_load_2d_pair(a_hi, t.Ah, fb, k0, m0);
           if (NP == 3) tma_load_2d_pair(a_lo, t.Al, fb, k0, m0);
         } else if (PASS == 1) {
-          tma_load_3d_pair(a_hi, t.Ah, fb, m0, k0, t.b);
-          tma_load_3d_pair(a_hi + A_TILE_BYTES / 2, t.Ah, fb, m0 + 64, k0, t.b);
+          tma_load_3d_pair(a_hi, t.Ah, fb, m0, k0, b);
+          tma_load_3d_pair(a_hi + A_TILE_BYTES / 2, t.Ah, fb, m0 + 64, k0, b);
           if (NP == 3) {
-            tma_load_3d_pair(a_lo, t.Al, fb, m0, k0, t.b);
-            tma_load_3d_pair(a_lo + A_TILE_BYTES / 2, t.Al, fb, m0 + 64, k0, t.b);
+            tma_load_3d_pair(a_lo, t.Al, fb, m0, k0, b);
+            tma_load_3d_pair(a_lo + A_TILE_BYTES / 2, t.Al, fb, m0 + 64, k0, b);
           }
         } else {
           tma_load_2d_pair(a_hi, t.Ah, fb, m0, k0);
@@ -182,7 +180,6 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
     }
   } else if (warp == 1 && lane == 0 && rank == 0) {
     // ------------------------------------------------ MMA issuer (leader CTA only)
-    constexpr uint32_t idesc = make_idesc(2 * BM, BN, a_mn, 0);
     constexpr uint32_t a_lbo = a_mn ? 4096u : 16u, a_sbo = a_mn ? 1024u : 512u, a_kstep = a_mn ? 2048u : 32u;
     constexpr uint32_t a_layout = a_mn ? LAYOUT_SW128 : LAYOUT_SW64;
     int it = 0, cc = 0, cursor = 0;
@@ -190,6 +187,7 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
     for (int pt = pid; pt < total_pt && ok; pt += npairs, ++cc) {
       src.at(pt, cursor, t);
       const int k_blocks = t.a->k_blocks;
+      const uint32_t idesc = make_idesc(2 * BM, t.a->bn, a_mn, 0);
       const int buf = cc & 1;
       if (!mbar_wait_cluster(tempty_bar(buf), ((cc >> 1) & 1) ^ 1, err, KERN_SPLIT_PAIR | WAIT_MMA_TMEM)) {
         ok = false;
@@ -229,26 +227,28 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
     const int quad = warp & 3;
     const int slice = (warp - 2) >> 2;
     uint8_t* xstage = PASS == 0 ? smem + P_STAGES * P_STAGE_BYTES + 256 + (warp - 2) * XSTAGE_BYTES : nullptr;
-    constexpr int COLS = BN / (epi_warps(MODE) / 4);
+    constexpr int SLICES = epi_warps(MODE) / 4;  // warps per lane quadrant; they take 32-output chunks in turn
     const uint32_t tempty_leader0 = mapa_shared(tempty_bar(0), 0);
     float vmax = 0.f;
     int cc = 0, cursor = 0;
     for (int pt = pid; pt < total_pt; pt += npairs, ++cc) {
       src.at(pt, cursor, t);
       const TcArgs& a = *t.a;
-      const int mt = 2 * t.mp + rank;
-      const int row = mt * BM + quad * 32 + lane;
-      const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(slice * COLS);
+      const int mf = 2 * t.mp + rank;
+      const int b = PASS == 1 ? mf / a.m_tiles : 0;
+      const int row = (mf - b * a.m_tiles) * BM + quad * 32 + lane;
+      const bool any = mf < a.m_tiles * a.batches;
+      const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
       const int buf = cc & 1;
       if (!mbar_wait(tfull_bar(buf), (cc >> 1) & 1, err, KERN_SPLIT_PAIR | WAIT_EPILOGUE)) break;
       tc_fence_after();
 #pragma unroll 1
-      for (int ch = 0; ch < COLS / 32; ++ch) {
-        const int col0 = t.nt * BN + slice * COLS + ch * 32;
-        if (col0 >= a.nout || mt >= a.m_tiles) break;  // warp-uniform
+      for (int ch = slice; ch * 32 < a.bn; ch += SLICES) {
+        const int col0 = t.nt * a.bn + ch * 32;
+        if (col0 >= a.nout || !any) break;  // warp-uniform
         float v[32];
         tmem_ld32(lane_addr + (uint32_t)(buf * BN + ch * 32), v);
-        epilogue_chunk<PASS, MODE, NP, 0>(a, row, col0, t.b, v, 1.f, 1.f, vmax, xstage);
+        epilogue_chunk<PASS, MODE, NP, 0>(a, row, col0, b, v, 1.f, 1.f, vmax, xstage);
       }
       tc_fence_before();
       __syncwarp();
@@ -271,8 +271,7 @@ __global__ void __launch_bounds__(num_threads(MODE), 1)
                                     const __grid_constant__ CUtensorMap tmA_lo,
                                     const __grid_constant__ CUtensorMap tmB_hi,
                                     const __grid_constant__ CUtensorMap tmB_lo, const __grid_constant__ TcArgs a) {
-  const int m_pairs = (a.m_tiles + 1) / 2;
-  const OneProblem src{&tmA_hi, &tmA_lo, &tmB_hi, &tmB_lo, &a, m_pairs * a.n_tiles, m_pairs * a.n_tiles * a.batches};
+  const OneProblem src{&tmA_hi, &tmA_lo, &tmB_hi, &tmB_lo, &a, (a.m_tiles * a.batches + 1) / 2 * a.n_tiles};
   pair_body<PASS, MODE, NP>(src, a.err, a.stall);
 }
 
@@ -434,9 +433,8 @@ cudaError_t launch_mode_product_bf16x3_grouped(int count, const TcGroupItem* ite
     TcGroupEntry& en = tab[q];
     en.A_hi = ps.mAh; en.A_lo = ps.mAl; en.B_hi = ps.mBh; en.B_lo = ps.mBl;
     en.a = ps.a;
-    en.tiles_per_batch = ((ps.a.m_tiles + 1) / 2) * ps.a.n_tiles;
     en.tile0 = (int)total;
-    total += (long long)en.tiles_per_batch * ps.a.batches;
+    total += pair_tiles(ps.a);
     if (total >= (1LL << 31)) return cudaErrorInvalidValue;
   }
   cudaError_t e = cudaMemcpyAsync(dev_table, host_table, (size_t)count * sizeof(TcGroupEntry), cudaMemcpyHostToDevice, s);
