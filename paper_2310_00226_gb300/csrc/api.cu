@@ -121,17 +121,17 @@ sem3d_status dev_upload(sem3d_plan* p, T** dst, const T* src, size_t count) {
   return SEM3D_OK;
 }
 
-// Split W (n x n row-major FP64) into bf16 hi + lo with row pitch Kp.
-void split_matrix(const std::vector<double>& W, int n, int Kp, std::vector<__nv_bfloat16>& hi,
-                  std::vector<__nv_bfloat16>& lo) {
-  hi.assign((size_t)n * Kp, __float2bfloat16_rn(0.f));
-  lo.assign((size_t)n * Kp, __float2bfloat16_rn(0.f));
+// Append W (n x n row-major FP64) split into bf16 hi + lo with row pitch Kp.
+void split_matrix(const double* W, int n, int Kp, std::vector<__nv_bfloat16>& hi, std::vector<__nv_bfloat16>& lo) {
+  const size_t at = hi.size();
+  hi.resize(at + (size_t)n * Kp, __float2bfloat16_rn(0.f));
+  lo.resize(at + (size_t)n * Kp, __float2bfloat16_rn(0.f));
   for (int o = 0; o < n; ++o)
     for (int t = 0; t < n; ++t) {
       const float x = (float)W[(size_t)o * n + t];
       const __nv_bfloat16 h = __float2bfloat16_rn(x);
-      hi[(size_t)o * Kp + t] = h;
-      lo[(size_t)o * Kp + t] = __float2bfloat16_rn(x - __bfloat162float(h));
+      hi[at + (size_t)o * Kp + t] = h;
+      lo[at + (size_t)o * Kp + t] = __float2bfloat16_rn(x - __bfloat162float(h));
     }
 }
 
@@ -324,6 +324,113 @@ sem3d_status solve_once_bf16x3(sem3d_plan* p, TcBuffers S0, TcBuffers S1, double
   return SEM3D_OK;
 }
 
+// ---- BF16x3 path in parity order (fold_kernels.cu).
+//
+// Where it is used: split-bf16 solves with at least two refinement sweeps,
+// whose result no longer depends on how the correction solves round (a bare
+// solve's 1e-5 and one sweep's 1e-8 do, and keep the node-order passes), on
+// grids of at least 255 nodes along every axis.  Below, the passes are bound
+// by memory and latency instead of the tensor cores and the folding kernels
+// cost what is saved.  Refined solves, node order -> parity order: n = 127
+// 377 -> 421 us, 255 1647 -> 1644 (a group of 16 problems, most of them 255
+// and larger, 52.0 -> 51.3 ms), 383 5455 -> 5160, 511 12.6 -> 11.5 ms, 767
+// 49.7 -> 42.7 ms, 999 133.8 ->
+// 102.8 ms; 511x63x255 978 -> 1007 us.
+constexpr int kFoldMin = 255;
+bool use_fold(const sem3d_plan* h) {
+  return h->prec == SEM3D_BF16X3 && h->sweeps >= 2 && std::min(h->g.nx, std::min(h->g.ny, h->g.nz)) >= kFoldMin;
+}
+
+// Its workspace, inside the node-order path's: two split arrays at the parity
+// pitch (at most 30 entries longer than the node pitch, so that the four bf16
+// parts fit in the six of the workspace for every n >= kFoldMin) and the double-FP32
+// solution.  The first split array also takes the correction in FP32 (written
+// by the last pass, which reads the second), the second the FP32 residual.
+struct FoldBuffers {
+  FoldGeom g;
+  TcBuffers S0, S1;
+  float *delta, *r32;
+  DfBuffers D;
+};
+
+FoldBuffers fold_buffers(const sem3d_plan* h) {
+  FoldBuffers b{};
+  b.g = fold_geom(h->g);
+  const size_t lines = (size_t)h->g.ny * h->g.nz;
+  const size_t Nf = align256((size_t)b.g.Px * lines * sizeof(__nv_bfloat16));
+  const size_t Ns = align256((size_t)h->g.Px * lines * sizeof(__nv_bfloat16));
+  char* w = static_cast<char*>(h->ws);
+  b.S0 = TcBuffers{reinterpret_cast<__nv_bfloat16*>(w), reinterpret_cast<__nv_bfloat16*>(w + Nf)};
+  b.S1 = TcBuffers{reinterpret_cast<__nv_bfloat16*>(w + 2 * Nf), reinterpret_cast<__nv_bfloat16*>(w + 3 * Nf)};
+  b.delta = reinterpret_cast<float*>(b.S0.hi);
+  b.r32 = reinterpret_cast<float*>(b.S1.hi);
+  b.D = DfBuffers{reinterpret_cast<float*>(w + 6 * Ns),
+                  reinterpret_cast<float*>(w + 6 * Ns + align256((size_t)h->g.Px * lines * sizeof(float)))};
+  return b;
+}
+
+// The six passes: S0 (folded right-hand side) -> delta.
+sem3d_status solve_once_fold(sem3d_plan* p, const FoldBuffers& b, cudaStream_t s) {
+  const DevAxis* d = p->dev;
+  const float c = (float)p->g.c;
+  const TcBuffers nb{nullptr, nullptr};
+  int* e = p->d_err;
+  const int sms = p->num_sms;
+  LAUNCH_SUB(p, K_TC, K_TC_Z, 1, s, launch_mode_product_fold(b.g, c, 2, d, 0, b.S0, b.S1, nullptr, EPI_STORE, e, sms, s));
+  LAUNCH_SUB(p, K_TC, K_TC_Y, 1, s, launch_mode_product_fold(b.g, c, 1, d, 0, b.S1, b.S0, nullptr, EPI_STORE, e, sms, s));
+  LAUNCH_SUB(p, K_TC, K_TC_X, 1, s, launch_mode_product_fold(b.g, c, 0, d, 0, b.S0, b.S1, nullptr, EPI_DIV, e, sms, s));
+  LAUNCH_SUB(p, K_TC, K_TC_X, 1, s, launch_mode_product_fold(b.g, c, 0, d, 1, b.S1, b.S0, nullptr, EPI_STORE, e, sms, s));
+  LAUNCH_SUB(p, K_TC, K_TC_Y, 1, s, launch_mode_product_fold(b.g, c, 1, d, 1, b.S0, b.S1, nullptr, EPI_STORE, e, sms, s));
+  LAUNCH_SUB(p, K_TC, K_TC_F64OUT, 1, s, launch_mode_product_fold(b.g, c, 2, d, 1, b.S1, nb, b.delta, EPI_STORE, e, sms, s));
+  return SEM3D_OK;
+}
+
+int df_sweeps(const sem3d_plan* h);                // double-FP32 sweeps of a split-tier solve (defined below)
+bool use_fixed_residual(const sem3d_plan* h);      // FP64-accurate residuals in fixed point (defined below)
+
+// f -> S0, with f's exponent for the fixed-point residuals.
+sem3d_status fold_rhs(sem3d_plan* h, const FoldBuffers& b, const double* f, cudaStream_t s) {
+  const bool fixed = use_fixed_residual(h);
+  if (fixed) CUDA_TRY(cudaMemsetAsync(h->d_fix + 1, 0, sizeof(int), s));
+  LAUNCH(h, K_SPLIT, 1, s, launch_fold(b.g, f, nullptr, h->g.nx, b.S0, fixed ? h->d_fix + 1 : nullptr, s));
+  return SEM3D_OK;
+}
+
+// After solve `sw` (0 = the first): delta into the solution, which is held in
+// double-FP32 until the last of the ndf double-FP32 sweeps.
+sem3d_status fold_update(sem3d_plan* h, const FoldBuffers& b, double* u, int sw, cudaStream_t s) {
+  const int ndf = df_sweeps(h);
+  const bool in_df = sw < ndf;
+  const int epi = sw == 0 ? (in_df ? EPI_DF_STORE : EPI_STORE)
+                          : in_df ? EPI_DF_ACCUM : sw == ndf ? EPI_DF_ACCUM_F64 : EPI_ACCUM;
+  // the vector double-FP32 residuals know that the first solution has no low parts
+  const bool vec = h->k == 1 || h->k == 2 || h->k == 4;
+  const DfBuffers D{b.D.hi, epi == EPI_DF_STORE && vec ? nullptr : b.D.lo};
+  const bool emax = !in_df && sw < h->sweeps && use_fixed_residual(h);  // a fixed-point residual of u follows
+  if (emax) CUDA_TRY(cudaMemsetAsync(h->d_fix, 0, sizeof(int), s));
+  LAUNCH(h, K_SPLIT, 1, s, launch_unfold(b.g, b.delta, epi, sw == 1, u, D, h->g.Px, emax ? h->d_fix : nullptr, s));
+  return SEM3D_OK;
+}
+
+// Residual of sweep `sw` (1 .. sweeps) in FP32, folded into S0.
+sem3d_status fold_residual(sem3d_plan* h, const FoldBuffers& b, const double* f, const double* u, int sw,
+                           cudaStream_t s) {
+  if (sw <= df_sweeps(h)) {
+    // Every residual in double-FP32 (SEM3D_RESIDUAL_DF): the rows of H must then be exact
+    LAUNCH(h, K_STENCIL, 1, s,
+           launch_stencil_df(h->g, h->k, h->dev, b.D, f, nullptr, nullptr, s, b.r32, nullptr,
+                             h->residual == SEM3D_RESIDUAL_DF, sw == 1));
+  } else if (use_fixed_residual(h)) {
+    LAUNCH(h, K_STENCIL, 2, s,
+           launch_residual_fixed(h->g, h->k, h->fix, u, f, h->d_fix, true, reinterpret_cast<int*>(b.D.hi),
+                                 reinterpret_cast<int*>(b.D.lo), nullptr, nullptr, h->num_sms, s, nullptr, b.r32, true));
+  } else {
+    LAUNCH(h, K_STENCIL, 1, s, launch_stencil_f32out(h->g, h->k, h->dev, u, f, b.r32, nullptr, s));
+  }
+  LAUNCH(h, K_SPLIT, 1, s, launch_fold(b.g, nullptr, b.r32, h->g.Px, b.S0, nullptr, s));
+  return SEM3D_OK;
+}
+
 sem3d_status run_solve(sem3d_plan* h, const double* f, double* u, cudaStream_t s);
 
 }  // namespace
@@ -381,6 +488,10 @@ sem3d_status sem3d_setup_bc(int nx, int ny, int nz, int k, double Lx, double Ly,
     for (int w = 0; w < 2; ++w)
       if ((st = dev_upload(p.get(), &D.par[w], A.par[w].data(), A.par[w].size())) != SEM3D_OK) return st;
     if ((st = dev_upload(p.get(), &D.lam_par, A.lam_par.data(), A.lam_par.size())) != SEM3D_OK) return st;
+    {
+      std::vector<float> lp(A.lam_par.begin(), A.lam_par.end());
+      if ((st = dev_upload(p.get(), &D.lamf_par, lp.data(), lp.size())) != SEM3D_OK) return st;
+    }
     if ((st = dev_upload(p.get(), &D.lam, A.lam.data(), A.lam.size())) != SEM3D_OK) return st;
     std::vector<float> lf(A.lam.begin(), A.lam.end());
     if ((st = dev_upload(p.get(), &D.lamf, lf.data(), lf.size())) != SEM3D_OK) return st;
@@ -452,9 +563,17 @@ sem3d_status sem3d_setup_bc(int nx, int ny, int nz, int k, double Lx, double Ly,
     }
     std::vector<__nv_bfloat16> hi, lo;
     for (int w = 0; w < 2; ++w) {
-      split_matrix(w == 0 ? A.Tinv : A.T, A.n, D.Kp, hi, lo);
+      hi.clear();
+      lo.clear();
+      split_matrix((w == 0 ? A.Tinv : A.T).data(), A.n, D.Kp, hi, lo);
       if ((st = dev_upload(p.get(), &D.W_hi[w], hi.data(), hi.size())) != SEM3D_OK) return st;
       if ((st = dev_upload(p.get(), &D.W_lo[w], lo.data(), lo.size())) != SEM3D_OK) return st;
+      hi.clear();
+      lo.clear();
+      split_matrix(A.par[w].data(), A.ne, pad16(A.ne), hi, lo);
+      split_matrix(A.par[w].data() + (size_t)A.ne * A.ne, A.no, pad16(A.no), hi, lo);
+      if ((st = dev_upload(p.get(), &D.Wp_hi[w], hi.data(), hi.size())) != SEM3D_OK) return st;
+      if ((st = dev_upload(p.get(), &D.Wp_lo[w], lo.data(), lo.size())) != SEM3D_OK) return st;
     }
   }
   {
@@ -696,6 +815,14 @@ sem3d_status run_solve(sem3d_plan* h, const double* f, double* u, cudaStream_t s
         LAUNCH(h, K_STENCIL, 1, s, launch_stencil(h->g, h->k, h->dev, u, f, r, nullptr, nullptr, 1, s));
       if ((st = solve_once_tf32(h, r, u, true, s)) != SEM3D_OK) return st;
     }
+  } else if (use_fold(h)) {
+    const FoldBuffers b = fold_buffers(h);
+    if ((st = fold_rhs(h, b, f, s)) != SEM3D_OK) return st;
+    for (int sw = 0; sw <= h->sweeps; ++sw) {
+      if (sw > 0 && (st = fold_residual(h, b, f, u, sw, s)) != SEM3D_OK) return st;
+      if ((st = solve_once_fold(h, b, s)) != SEM3D_OK) return st;
+      if ((st = fold_update(h, b, u, sw, s)) != SEM3D_OK) return st;
+    }
   } else {
     const size_t Ns = align256((size_t)h->g.Px * h->g.ny * h->g.nz * sizeof(__nv_bfloat16));
     const size_t Nf = align256((size_t)h->g.Px * h->g.ny * h->g.nz * sizeof(float));  // double-FP32 u, pitch Px
@@ -708,10 +835,7 @@ sem3d_status run_solve(sem3d_plan* h, const double* f, double* u, cudaStream_t s
     // Double-FP32 sweeps (the solution held as a double-FP32 pair between
     // them): SEM3D_RESIDUAL_MIXED runs sweeps 1 .. sw-1 so and the last one in
     // FP64 on the FP64 solution; SEM3D_RESIDUAL_DF runs every sweep so.
-    const bool df_ok = h->k <= 8 && h->g.bc == 0 && (h->prec == SEM3D_BF16X3 || h->prec == SEM3D_F16X3);
-    const int ndf = !df_ok ? 0
-                           : (h->residual == SEM3D_RESIDUAL_MIXED && sw >= 2) ? sw - 1
-                           : (h->residual == SEM3D_RESIDUAL_DF) ? sw : 0;
+    const int ndf = df_sweeps(h);
     const bool mixed = ndf > 0;
     // Every residual in double-FP32: the operator's rows must then be exact
     // (three FP32 terms), or the sweeps converge to the 48-bit operator's
@@ -1179,7 +1303,7 @@ struct BatchState {
 };
 BatchState g_batch;
 
-constexpr size_t kStageTableBytes = 64 * 1024;  // per grouped launch (>= 64 problems)
+constexpr size_t kStageTableBytes = 128 * 1024;  // per grouped launch (>= 64 problems of two entries)
 
 sem3d_status batch_resources(int device, size_t stages) {
   if (g_batch.device != device) {
@@ -1344,15 +1468,26 @@ sem3d_status batched_tc(int count, const sem3d_handle* hs, const double* const* 
   const int sweeps = hs[0]->sweeps;
   const int ndf = df_sweeps(hs[0]);
   const int nprod = hs[0]->prec == SEM3D_BF16 ? 1 : 3;
-  sem3d_status st = batch_resources(hs[0]->device, 6 * (size_t)(1 + sweeps));
+  // 7 grouped launches per solve: the last pass of the node-order problems and
+  // that of the parity-order ones write different outputs
+  sem3d_status st = batch_resources(hs[0]->device, 7 * (size_t)(1 + sweeps));
   if (st != SEM3D_OK) return st;
   StagingRelease release{s};
   StreamFan fan;
   if ((st = fan.init(s, count)) != SEM3D_OK) return st;
   std::vector<TcBuffers> S0(count), S1(count);
   std::vector<DfBuffers> D(count);
+  std::vector<FoldBuffers> fb(count);
+  std::vector<char> fold(count);
   for (int q = 0; q < count; ++q) {
     sem3d_plan* h = hs[q];
+    fold[q] = use_fold(h);
+    if (fold[q]) {
+      fb[q] = fold_buffers(h);
+      S0[q] = fb[q].S0;
+      S1[q] = fb[q].S1;
+      continue;
+    }
     const size_t Ns = align256((size_t)h->g.Px * h->g.ny * h->g.nz * sizeof(__nv_bfloat16));
     const size_t Nf = align256((size_t)h->g.Px * h->g.ny * h->g.nz * sizeof(float));
     char* w = static_cast<char*>(h->ws);
@@ -1361,81 +1496,95 @@ sem3d_status batched_tc(int count, const sem3d_handle* hs, const double* const* 
     D[q] = DfBuffers{reinterpret_cast<float*>(w + 6 * Ns), reinterpret_cast<float*>(w + 6 * Ns + Nf)};
   }
   const DfBuffers none{nullptr, nullptr};
-  std::vector<TcGroupItem> items(count);
+  std::vector<TcGroupItem> items;
+  items.reserve(count);
   size_t stage = 0;
-  // One grouped pass: problem q reads in(q), writes out(q) / out64(q) / df(q).
-  auto pass = [&](int axis, int which, int epi, int sub, auto in_of, auto out_of, auto out64_of,
-                  bool use_df) -> sem3d_status {
+  // One grouped pass over the problems of `set` (0: node order, 1: parity
+  // order, 2: all): in -> out, the last pass with epi_last into u / D / delta.
+  auto pass = [&](int axis, int which, int epi, int sub, const std::vector<TcBuffers>& in,
+                  const std::vector<TcBuffers>& out, int set, bool last, bool out_u, bool use_df) -> sem3d_status {
+    items.clear();
     for (int q = 0; q < count; ++q) {
       const sem3d_plan* h = hs[q];
-      items[q] = TcGroupItem{&h->g, &h->dev[axis], in_of(q), out_of(q), out64_of(q), use_df ? D[q] : none,
-                             h->dev[0].lamf, h->dev[1].lamf, h->dev[2].lamf};
+      if (set != 2 && fold[q] != set) continue;
+      TcGroupItem it{&h->g, &h->dev[axis], in[q], last ? TcBuffers{nullptr, nullptr} : out[q], nullptr, none,
+                     h->dev[0].lamf, h->dev[1].lamf, h->dev[2].lamf, nullptr, nullptr, nullptr, 0.f};
+      if (fold[q]) {
+        it.fold = &fb[q].g;
+        it.ax = h->dev;
+        it.c = (float)h->g.c;
+        it.out32 = last ? fb[q].delta : nullptr;
+      } else if (last) {
+        it.out64 = out_u ? u[q] : nullptr;
+        it.df = use_df ? D[q] : none;
+      }
+      items.push_back(it);
     }
+    if (items.empty()) return SEM3D_OK;
     char* ht = static_cast<char*>(g_batch.host_table) + stage * kStageTableBytes;
     char* dt = static_cast<char*>(g_batch.dev_table) + stage * kStageTableBytes;
     ++stage;
     LAUNCH_SUB(hs[0], K_TC, sub, 1, s,
-               launch_mode_product_bf16x3_grouped(count, items.data(), axis, which, epi, nprod, hs[0]->d_err, dt, ht,
-                                                  kStageTableBytes, hs[0]->num_sms, s));
+               launch_mode_product_bf16x3_grouped((int)items.size(), items.data(), axis, which, epi, nprod,
+                                                  hs[0]->d_err, dt, ht, kStageTableBytes, hs[0]->num_sms, s));
     return SEM3D_OK;
   };
-  auto s0 = [&](int q) { return S0[q]; };
-  auto s1 = [&](int q) { return S1[q]; };
-  auto no64 = [&](int) -> double* { return nullptr; };
   // Forward z, y, x (division fused), backward x, y, then the last z pass with
-  // the epilogue epi_last into u / the double-FP32 solution.
+  // the epilogue epi_last into u / the double-FP32 solution (parity order:
+  // into the correction, which the updates below take in).
   auto solve_group = [&](int epi_last, bool out_u, bool use_df) -> sem3d_status {
     sem3d_status r;
-    if ((r = pass(2, 0, EPI_STORE, K_TC_Z, s0, s1, no64, false)) != SEM3D_OK) return r;
-    if ((r = pass(1, 0, EPI_STORE, K_TC_Y, s1, s0, no64, false)) != SEM3D_OK) return r;
-    if ((r = pass(0, 0, EPI_DIV, K_TC_X, s0, s1, no64, false)) != SEM3D_OK) return r;
-    if ((r = pass(0, 1, EPI_STORE, K_TC_X, s1, s0, no64, false)) != SEM3D_OK) return r;
-    if ((r = pass(1, 1, EPI_STORE, K_TC_Y, s0, s1, no64, false)) != SEM3D_OK) return r;
-    return pass(2, 1, epi_last, K_TC_F64OUT, s1, s0, [&](int q) -> double* { return out_u ? u[q] : nullptr; },
-                use_df);
+    if ((r = pass(2, 0, EPI_STORE, K_TC_Z, S0, S1, 2, false, false, false)) != SEM3D_OK) return r;
+    if ((r = pass(1, 0, EPI_STORE, K_TC_Y, S1, S0, 2, false, false, false)) != SEM3D_OK) return r;
+    if ((r = pass(0, 0, EPI_DIV, K_TC_X, S0, S1, 2, false, false, false)) != SEM3D_OK) return r;
+    if ((r = pass(0, 1, EPI_STORE, K_TC_X, S1, S0, 2, false, false, false)) != SEM3D_OK) return r;
+    if ((r = pass(1, 1, EPI_STORE, K_TC_Y, S0, S1, 2, false, false, false)) != SEM3D_OK) return r;
+    if ((r = pass(2, 1, EPI_STORE, K_TC_F64OUT, S1, S0, 1, true, false, false)) != SEM3D_OK) return r;
+    return pass(2, 1, epi_last, K_TC_F64OUT, S1, S0, 0, true, out_u, use_df);
   };
-  // f -> split input of every problem
-  if ((st = fan.begin()) != SEM3D_OK) return st;
-  for (int q = 0; q < count; ++q) {
-    int* fexp = use_fixed_residual(hs[q]) ? hs[q]->d_fix + 1 : nullptr;  // the fixed-point residuals' scale of f
-    if (fexp) CUDA_TRY(cudaMemsetAsync(fexp, 0, sizeof(int), fan.stream(q)));
-    LAUNCH(hs[q], K_SPLIT, 1, fan.stream(q), launch_split(hs[q]->g, f[q], S0[q].hi, S0[q].lo, fan.stream(q), fexp));
-  }
-  if ((st = fan.end()) != SEM3D_OK) return st;
-  if (ndf == 0) {
-    if ((st = solve_group(EPI_STORE, true, false)) != SEM3D_OK) return st;
-  } else {
-    if ((st = solve_group(EPI_DF_STORE, false, true)) != SEM3D_OK) return st;
-    const bool exact_coef = hs[0]->residual == SEM3D_RESIDUAL_DF;
-    for (int sw = 1; sw <= ndf; ++sw) {
-      if ((st = fan.begin()) != SEM3D_OK) return st;
-      for (int q = 0; q < count; ++q) {
-        sem3d_plan* h = hs[q];
-        const int launches = (h->k == 1 || h->k == 2 || h->k == 4 || h->g.Px == h->g.nx) ? 1 : 2;
-        LAUNCH(h, K_STENCIL, launches, fan.stream(q),
-               launch_stencil_df(h->g, h->k, h->dev, D[q], f[q], S0[q].hi, S0[q].lo, fan.stream(q), nullptr, nullptr,
-                                 exact_coef, sw == 1));
-      }
-      if ((st = fan.end()) != SEM3D_OK) return st;
-      const bool last_df = sw == ndf;
-      if ((st = solve_group(last_df ? EPI_DF_ACCUM_F64 : EPI_DF_ACCUM, last_df, true)) != SEM3D_OK) return st;
+  // Element-wise work of problem q before solve sw (on its stream of the fan):
+  // the update with the previous solve's correction, the residual, the split.
+  auto between = [&](int q, int sw, cudaStream_t qs) -> sem3d_status {
+    sem3d_plan* h = hs[q];
+    sem3d_status r;
+    if (fold[q]) {
+      if (sw == 0) return fold_rhs(h, fb[q], f[q], qs);
+      if ((r = fold_update(h, fb[q], u[q], sw - 1, qs)) != SEM3D_OK) return r;
+      return sw <= sweeps ? fold_residual(h, fb[q], f[q], u[q], sw, qs) : SEM3D_OK;
     }
-  }
-  for (int sw = ndf; sw < sweeps; ++sw) {
+    const bool fixed = use_fixed_residual(h);
+    if (sw == 0) {
+      int* fexp = fixed ? h->d_fix + 1 : nullptr;  // the fixed-point residuals' scale of f
+      if (fexp) CUDA_TRY(cudaMemsetAsync(fexp, 0, sizeof(int), qs));
+      LAUNCH(h, K_SPLIT, 1, qs, launch_split(h->g, f[q], S0[q].hi, S0[q].lo, qs, fexp));
+    } else if (sw > sweeps) {
+    } else if (sw <= ndf) {
+      const int launches = (h->k == 1 || h->k == 2 || h->k == 4 || h->g.Px == h->g.nx) ? 1 : 2;
+      LAUNCH(h, K_STENCIL, launches, qs,
+             launch_stencil_df(h->g, h->k, h->dev, D[q], f[q], S0[q].hi, S0[q].lo, qs, nullptr, nullptr,
+                               h->residual == SEM3D_RESIDUAL_DF, sw == 1));
+    } else if (fixed) {
+      LAUNCH(h, K_STENCIL, 3, qs,
+             launch_residual_fixed(h->g, h->k, h->fix, u[q], f[q], h->d_fix, true, reinterpret_cast<int*>(D[q].hi),
+                                   reinterpret_cast<int*>(D[q].lo), S0[q].hi, S0[q].lo, h->num_sms, qs));
+    } else {
+      LAUNCH(h, K_STENCIL, h->g.Px != h->g.nx ? 2 : 1, qs,
+             launch_stencil(h->g, h->k, h->dev, u[q], f[q], nullptr, S0[q].hi, S0[q].lo, 2, qs));
+    }
+    return SEM3D_OK;
+  };
+  const bool any_fold = std::find(fold.begin(), fold.end(), 1) != fold.end();
+  for (int sw = 0; sw <= sweeps + 1; ++sw) {
+    if (sw > sweeps && !any_fold) break;
     if ((st = fan.begin()) != SEM3D_OK) return st;
-    for (int q = 0; q < count; ++q) {
-      sem3d_plan* h = hs[q];
-      if (use_fixed_residual(h)) {
-        LAUNCH(h, K_STENCIL, 3, fan.stream(q),
-               launch_residual_fixed(h->g, h->k, h->fix, u[q], f[q], h->d_fix, true, reinterpret_cast<int*>(D[q].hi),
-                                     reinterpret_cast<int*>(D[q].lo), S0[q].hi, S0[q].lo, h->num_sms, fan.stream(q)));
-      } else {
-        LAUNCH(h, K_STENCIL, h->g.Px != h->g.nx ? 2 : 1, fan.stream(q),
-               launch_stencil(h->g, h->k, h->dev, u[q], f[q], nullptr, S0[q].hi, S0[q].lo, 2, fan.stream(q)));
-      }
-    }
+    for (int q = 0; q < count; ++q)
+      if ((st = between(q, sw, fan.stream(q))) != SEM3D_OK) return st;
     if ((st = fan.end()) != SEM3D_OK) return st;
-    if ((st = solve_group(EPI_ACCUM, true, false)) != SEM3D_OK) return st;
+    if (sw > sweeps) break;  // the last updates
+    const bool to_u = sw >= ndf, use_df = ndf > 0 && sw <= ndf;
+    const int epi = sw == 0 ? (ndf > 0 ? EPI_DF_STORE : EPI_STORE)
+                            : sw < ndf ? EPI_DF_ACCUM : sw == ndf ? EPI_DF_ACCUM_F64 : EPI_ACCUM;
+    if ((st = solve_group(epi, to_u, use_df)) != SEM3D_OK) return st;
   }
   return release.record();
 }

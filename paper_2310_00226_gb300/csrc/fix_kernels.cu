@@ -269,6 +269,10 @@ __global__ void __launch_bounds__(256, 4) stencil_fix4_kernel(FixArgs a, const _
       for (int p = 0; p < 4; ++p)  // pads stay zero
         r[p] = (i0 + p >= a.nx) ? 0.f : finite ? fixed_to_f32(R[p], X) : __int_as_float(0x7FC00000);
       const long long o = line * a.Px + i0;
+      if (a.out32) {
+        *reinterpret_cast<float4*>(a.out32 + o) = make_float4(r[0], r[1], r[2], r[3]);
+        continue;
+      }
       uint32_t hw[2], lw[2];
 #pragma unroll
       for (int p = 0; p < 4; p += 2) {
@@ -384,11 +388,15 @@ __global__ void __launch_bounds__(256) stencil_fix_elem_kernel(FixArgs a, const 
         continue;
       }
       const float r = finite ? fixed_to_f32(R, X) : __int_as_float(0x7FC00000);
+      if (a.out32) {
+        a.out32[row + i] = r;
+        continue;
+      }
       const __nv_bfloat16 h16 = __float2bfloat16_rn(r);
       a.hi[row + i] = h16;
       a.lo[row + i] = __float2bfloat16_rn(r - __bfloat162float(h16));
     }
-    if (ex == nex - 1 && !a.out64)
+    if (ex == nex - 1 && !a.out64 && !a.out32)
       for (int i = a.nx; i < a.Px; ++i) {
         a.hi[row + i] = __float2bfloat16_rn(0.f);
         a.lo[row + i] = __float2bfloat16_rn(0.f);
@@ -473,14 +481,17 @@ bool build_fix_coef(const double* const hq[3], int k, FixCoef& cf) {
 
 cudaError_t launch_residual_fixed(const Geom& g, int k, const FixCoef& cf, const double* u, const double* f,
                                   int* state, bool f_exponent_known, int* Uh, int* Ul, __nv_bfloat16* out_hi,
-                                  __nv_bfloat16* out_lo, int num_sms, cudaStream_t s, double* out64) {
+                                  __nv_bfloat16* out_lo, int num_sms, cudaStream_t s, double* out64, float* out32,
+                                  bool u_exponent_known) {
   if (g.bc != 0 || k < 1 || k > 8) return cudaErrorInvalidValue;
   const long long N = (long long)g.nx * g.ny * g.nz;
   const long long lines = (long long)g.ny * g.nz;
   const int red_grid = num_sms * 8;
-  cudaError_t e = cudaMemsetAsync(state, 0, f_exponent_known ? sizeof(int) : 2 * sizeof(int), s);
+  cudaError_t e = cudaSuccess;
+  if (!u_exponent_known) e = cudaMemsetAsync(state, 0, sizeof(int), s);
+  if (e == cudaSuccess && !f_exponent_known) e = cudaMemsetAsync(state + 1, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  max_exponent_kernel<<<red_grid, 256, 0, s>>>(u, N, state);
+  if (!u_exponent_known) max_exponent_kernel<<<red_grid, 256, 0, s>>>(u, N, state);
   if (!f_exponent_known) max_exponent_kernel<<<red_grid, 256, 0, s>>>(f, N, state + 1);
   const long long conv = lines * (g.Px / 4);
   long long cb = (conv + 255) / 256;
@@ -488,7 +499,7 @@ cudaError_t launch_residual_fixed(const Geom& g, int k, const FixCoef& cf, const
   to_fixed_kernel<<<(unsigned)(cb < 1 ? 1 : cb), 256, 0, s>>>(u, Uh, Ul, g.nx, g.Px, lines, state, cf.t);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   FixArgs a{};
-  a.Uh = Uh; a.Ul = Ul; a.f = f; a.hi = out_hi; a.lo = out_lo; a.state = state; a.out64 = out64;
+  a.Uh = Uh; a.Ul = Ul; a.f = f; a.hi = out_hi; a.lo = out_lo; a.state = state; a.out64 = out64; a.out32 = out32;
   a.nx = g.nx; a.ny = g.ny; a.nz = g.nz; a.Px = g.Px;
   switch (k) {
     case 1: return launch_fix4<1>(a, cf, s);  // 4 % k == 0: the vector layout

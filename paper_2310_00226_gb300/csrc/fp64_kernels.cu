@@ -203,7 +203,7 @@ struct StencilArgs {
   const int *lox, *hix, *loy, *hiy, *loz, *hiz;
   int nx, ny, nz, k, Px, mode;
   double c;
-  float* out32;        // MODE 3: FP32 residual at pitch Px, max |r| -> st slot 0
+  float* out32;        // mode 3: FP32 residual at pitch Px; with st, max |r| -> slot 0 (element kernels)
   F16State* st;
 };
 
@@ -248,6 +248,8 @@ __global__ void __launch_bounds__(256) stencil_kernel(StencilArgs a) {
       const double r = a.f[idx] - s;
       if (a.mode == 1) {
         a.out64[idx] = r;
+      } else if (a.mode == 3) {
+        a.out32[(long long)i + (long long)a.Px * jl] = (float)r;
       } else {
         const float rf = (float)r;
         const __nv_bfloat16 h16 = __float2bfloat16_rn(rf);
@@ -374,7 +376,7 @@ __global__ void __launch_bounds__(256) stencil_elem_kernel(StencilArgs a, const 
       }
     }
   }
-  if (MODE == 3) {  // every lane of the warp gets here (after the loop)
+  if (MODE == 3 && a.st) {  // every lane of the warp gets here (after the loop)
     rmax = warp_max(rmax);
     if ((threadIdx.x & 31) == 0 && rmax > 0.f) atomicMax(&a.st->maxbits[0], __float_as_uint(rmax));
   }
@@ -547,7 +549,7 @@ __global__ void __launch_bounds__(256) stencil_df_kernel(DfArgs a) {
       a.lo[o] = l16;
     }
   }
-  if (a.out32) {  // every lane of the warp gets here (after the loop)
+  if (a.out32 && a.st) {  // every lane of the warp gets here (after the loop)
     rmax = warp_max(rmax);
     if ((threadIdx.x & 31) == 0 && rmax > 0.f) atomicMax(&a.st->maxbits[0], __float_as_uint(rmax));
   }
@@ -666,7 +668,7 @@ __global__ void __launch_bounds__(256, 4) stencil_df4_kernel(DfArgs a, const __g
       }
     }
   }
-  if (a.out32) {  // every lane of the warp gets here
+  if (a.out32 && a.st) {  // every lane of the warp gets here
     rmax = warp_max(rmax);
     if ((threadIdx.x & 31) == 0 && rmax > 0.f) atomicMax(&a.st->maxbits[0], __float_as_uint(rmax));
   }
@@ -801,30 +803,43 @@ cudaError_t launch_mode_product_f64(const Geom& g, int axis, const DevAxis* ax, 
   return kcontig ? launch_f64<true, false>(p, num_sms, s) : launch_f64<false, false>(p, num_sms, s);
 }
 
-cudaError_t launch_stencil(const Geom& g, int k, const DevAxis* ax, const double* u, const double* f, double* out64,
-                           __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, int mode, cudaStream_t s) {
+namespace {
+
+StencilArgs stencil_args(const Geom& g, int k, const DevAxis* ax, const double* u, const double* f, int mode) {
   StencilArgs a{};
-  a.u = u; a.f = f; a.out64 = out64; a.hi = out_hi; a.lo = out_lo;
+  a.u = u; a.f = f;
   a.Hx = ax[0].Hband; a.Hy = ax[1].Hband; a.Hz = ax[2].Hband;
   a.lox = ax[0].band_lo; a.hix = ax[0].band_hi;
   a.loy = ax[1].band_lo; a.hiy = ax[1].band_hi;
   a.loz = ax[2].band_lo; a.hiz = ax[2].band_hi;
   a.nx = g.nx; a.ny = g.ny; a.nz = g.nz; a.k = k; a.Px = g.Px; a.mode = mode; a.c = g.c;
+  return a;
+}
+
+cudaError_t launch_stencil_any(const StencilArgs& a, const Geom& g, const DevAxis* ax, cudaStream_t s) {
   const long long N = (long long)g.nx * g.ny * g.nz;
-  cudaError_t e;
-  switch (g.bc == 0 ? k : 0) {  // the element-pattern kernels assume Dirichlet rows
-    case 1: e = launch_elem<1>(a, ax, mode, s); break;
-    case 2: e = launch_elem<2>(a, ax, mode, s); break;
-    case 3: e = launch_elem<3>(a, ax, mode, s); break;
-    case 4: e = launch_elem<4>(a, ax, mode, s); break;
-    case 5: e = launch_elem<5>(a, ax, mode, s); break;
-    case 6: e = launch_elem<6>(a, ax, mode, s); break;
-    case 7: e = launch_elem<7>(a, ax, mode, s); break;
-    case 8: e = launch_elem<8>(a, ax, mode, s); break;
+  switch (g.bc == 0 ? a.k : 0) {  // the element-pattern kernels assume Dirichlet rows
+    case 1: return launch_elem<1>(a, ax, a.mode, s);
+    case 2: return launch_elem<2>(a, ax, a.mode, s);
+    case 3: return launch_elem<3>(a, ax, a.mode, s);
+    case 4: return launch_elem<4>(a, ax, a.mode, s);
+    case 5: return launch_elem<5>(a, ax, a.mode, s);
+    case 6: return launch_elem<6>(a, ax, a.mode, s);
+    case 7: return launch_elem<7>(a, ax, a.mode, s);
+    case 8: return launch_elem<8>(a, ax, a.mode, s);
     default:  // higher degrees and Neumann data: one thread per node, per-row band ranges
       stencil_kernel<<<(int)((N + 255) / 256 < 0x7FFFFFFF ? (N + 255) / 256 : 0x7FFFFFFF), 256, 0, s>>>(a);
-      e = cudaGetLastError();
+      return cudaGetLastError();
   }
+}
+
+}  // namespace
+
+cudaError_t launch_stencil(const Geom& g, int k, const DevAxis* ax, const double* u, const double* f, double* out64,
+                           __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, int mode, cudaStream_t s) {
+  StencilArgs a = stencil_args(g, k, ax, u, f, mode);
+  a.out64 = out64; a.hi = out_hi; a.lo = out_lo;
+  const cudaError_t e = launch_stencil_any(a, g, ax, s);
   if (e != cudaSuccess || mode != 2 || g.Px == g.nx) return e;
   const long long lines = (long long)g.ny * g.nz;
   zero_pads_kernel<<<grid_for(lines * (g.Px - g.nx), 256), 256, 0, s>>>(out_hi, out_lo, g.nx, g.Px, lines);
@@ -864,20 +879,10 @@ cudaError_t launch_stencil_df(const Geom& g, int k, const DevAxis* ax, DfBuffers
 
 cudaError_t launch_stencil_f32out(const Geom& g, int k, const DevAxis* ax, const double* u, const double* f,
                                   float* out32, F16State* st, cudaStream_t s) {
-  if (k < 1 || k > 8 || g.bc != 0) return cudaErrorInvalidValue;
-  StencilArgs a{};
-  a.u = u; a.f = f; a.out32 = out32; a.st = st;
-  a.nx = g.nx; a.ny = g.ny; a.nz = g.nz; a.k = k; a.Px = g.Px; a.mode = 3; a.c = g.c;
-  switch (k) {
-    case 1: return launch_elem<1>(a, ax, 3, s);
-    case 2: return launch_elem<2>(a, ax, 3, s);
-    case 3: return launch_elem<3>(a, ax, 3, s);
-    case 4: return launch_elem<4>(a, ax, 3, s);
-    case 5: return launch_elem<5>(a, ax, 3, s);
-    case 6: return launch_elem<6>(a, ax, 3, s);
-    case 7: return launch_elem<7>(a, ax, 3, s);
-    default: return launch_elem<8>(a, ax, 3, s);
-  }
+  if (st && (k < 1 || k > 8 || g.bc != 0)) return cudaErrorInvalidValue;
+  StencilArgs a = stencil_args(g, k, ax, u, f, 3);
+  a.out32 = out32; a.st = st;
+  return launch_stencil_any(a, g, ax, s);
 }
 
 // ------------------------------------------------------------------ F16X3 split

@@ -21,19 +21,22 @@ namespace sem3d {
 // the FP64 pipe, 1/64 of the FP32 rate on this GPU).  Covers normal and
 // subnormal results, overflow to infinity, zeros, infinities and NaN (quieted).
 __device__ __forceinline__ float f64_to_f32_rn(double x) {
+  const unsigned int h = (unsigned int)__double2hiint(x), w = (unsigned int)__double2loint(x);
+  const unsigned int sign = h & 0x80000000u;
+  const int e = (int)((h >> 20) & 0x7FF) - 1023 + 127;  // biased FP32 exponent
+  if (e >= 1 && e < 255) {
+    // exponent and the leading 23 fraction bits, rebiased (the bits shifted
+    // out at the top drop out of the difference), then round to nearest even;
+    // a carry rounds into the exponent
+    unsigned int r = __funnelshift_l(w, h, 3) - (896u << 23);
+    r += ((w & 0x1FFFFFFFu) + 0x0FFFFFFFu + (r & 1u)) >> 29;
+    return __uint_as_float(sign | r);
+  }
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned int sign = (unsigned int)(b >> 63) << 31;
   const int ex = (int)((b >> 52) & 0x7FF);
   const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
   if (ex == 0x7FF) return __uint_as_float(sign | 0x7F800000u | (m ? 0x400000u | (unsigned int)(m >> 29) : 0u));
-  const int e = ex - 1023 + 127;  // biased FP32 exponent
   if (e >= 255) return __uint_as_float(sign | 0x7F800000u);
-  if (e >= 1) {
-    unsigned int r = ((unsigned int)e << 23) | (unsigned int)(m >> 29);  // truncated
-    const unsigned int rem = (unsigned int)(m & 0x1FFFFFFFull), half = 0x10000000u;
-    r += (rem > half || (rem == half && (r & 1u))) ? 1u : 0u;  // a carry rounds into the exponent
-    return __uint_as_float(sign | r);
-  }
   // Subnormal (or zero) result: significand 1.m (53 bits) scaled to units of
   // 2^-149, i.e. shifted right by s = 30 - e >= 30 bits, then rounded.
   if (ex == 0) return __uint_as_float(sign);  // FP64 zero or subnormal: below half of 2^-149
@@ -117,6 +120,10 @@ struct DevAxis {
   int ne = 0, no = 0;           // even and odd modes (see Axis1D::par)
   double* par[2] = {nullptr, nullptr};  // FP64 even block, then odd block: [0] = T^{-1}, [1] = T
   double* lam_par = nullptr;    // FP64 eigenvalues, even modes first
+  float* lamf_par = nullptr;    // FP32 copy
+  // the parity blocks split into bf16 hi + lo: ne rows x pad16(ne), then no rows x pad16(no)
+  __nv_bfloat16* Wp_hi[2] = {nullptr, nullptr};
+  __nv_bfloat16* Wp_lo[2] = {nullptr, nullptr};
   float* lamf = nullptr;        // FP32 copy for the low-precision epilogues
   double* Hband = nullptr;      // FP64 n x (2k+1)
   double* Hq = nullptr;         // FP64 k x (2k+1) per-local-index rows of H (x axis: + c on the diagonal)
@@ -185,6 +192,18 @@ struct Geom {
   int bc = 0;          // 0: Dirichlet (element-pattern stencils), 1: Neumann (per-row stencil)
 };
 
+// Grid of the split tier's working arrays in parity order (fold_kernels.cu):
+// along every axis the even part (ne entries) comes first, then the odd one
+// (no).  The x axis has pitch Px = Pe + Po, its odd part starting at Pe (both
+// multiples of 16, pad entries zero), so that either part of a line can be a
+// K-major TMA operand.
+struct FoldGeom {
+  int nx, ny, nz;
+  int ne[3], no[3];
+  int Pe, Po, Px;
+};
+FoldGeom fold_geom(const Geom& g);
+
 // ---- FP64 kernels (fp64_kernels.cu)
 // One mode product along `axis` (0 = x, 1 = y, 2 = z) on dense n-pitch FP64
 // arrays with the parity blocks of T^{-1} (which = 0: nodes -> modes, even
@@ -231,8 +250,8 @@ cudaError_t launch_stencil_df(const Geom& g, int k, const DevAxis* ax, DfBuffers
                               __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, cudaStream_t s,
                               float* out32 = nullptr, F16State* st = nullptr, bool exact_coef = false,
                               bool lo_zero = false);
-// FP64 residual written as FP32 at pitch Px with its max |r| in state slot 0
-// (the F16X3 tier then splits it with launch_split_f16).  1 <= k <= 8.
+// FP64 residual written as FP32 at pitch Px; with st, its max |r| goes to
+// state slot 0 (the F16X3 tier then splits it with launch_split_f16).
 cudaError_t launch_stencil_f32out(const Geom& g, int k, const DevAxis* ax, const double* u, const double* f,
                                   float* out32, F16State* st, cudaStream_t s);
 // ---- fixed-point residual (fix_kernels.cu)
@@ -267,6 +286,7 @@ struct FixArgs {
   __nv_bfloat16* lo;
   const int* state;  // [0]: max biased exponent of u, [1]: of f
   double* out64;     // if set: r in FP64 at pitch nx (hi / lo unused)
+  float* out32;      // if set: r in FP32 at pitch Px (hi / lo unused)
   int nx, ny, nz, Px;
 };
 // Build the tables from the FP64 rows hq[axis] (k x (2k+1), x with c on its
@@ -281,10 +301,12 @@ bool build_fix_coef(const double* const hq[3], int k, FixCoef& cf);
 // e.g. from launch_split's emax); Uh,
 // Ul: two int32 arrays of Px * ny * nz (the fixed-point u, 16-byte aligned).
 // With out64 set, r is written in FP64 at pitch nx instead (the TF32 tier's
-// refinement reads it so).
+// refinement reads it so); with out32 in FP32 at pitch Px (for launch_fold).
+// u_exponent_known: state[0] holds u's exponent already (launch_unfold's emax).
 cudaError_t launch_residual_fixed(const Geom& g, int k, const FixCoef& cf, const double* u, const double* f,
                                   int* state, bool f_exponent_known, int* Uh, int* Ul, __nv_bfloat16* out_hi,
-                                  __nv_bfloat16* out_lo, int num_sms, cudaStream_t s, double* out64 = nullptr);
+                                  __nv_bfloat16* out_lo, int num_sms, cudaStream_t s, double* out64 = nullptr,
+                                  float* out32 = nullptr, bool u_exponent_known = false);
 // FP64 dense n-pitch -> bf16 hi/lo at pitch Px with zero pads; with emax
 // set, also atomicMax(*emax, largest biased FP64 exponent of the input).
 cudaError_t launch_split(const Geom& g, const double* in, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t s,
@@ -295,6 +317,25 @@ struct TcBuffers {
   __nv_bfloat16* hi;
   __nv_bfloat16* lo;
 };
+// ---- parity form of the split arrays (fold_kernels.cu)
+// Right-hand side in node order (f64, pitch nx; or f32, rows of `pitch`) ->
+// split array in parity order.  emax (f64 only): as launch_split's.
+cudaError_t launch_fold(const FoldGeom& g, const double* f64, const float* f32, int pitch, TcBuffers out, int* emax,
+                        cudaStream_t s);
+// Add the correction delta (FP32, parity order) to the solution, as `epi`
+// says: EPI_STORE / EPI_ACCUM u, EPI_DF_STORE / EPI_DF_ACCUM the double-FP32
+// pair df (pitch PxDf; df.lo may be null for the store: then it is not
+// written, and the next update has to be told lo_zero), EPI_DF_ACCUM_F64 u
+// from the pair.  lo_zero: the pair's low parts are zero (not read).  emax: as
+// launch_split's, of the u written.
+cudaError_t launch_unfold(const FoldGeom& g, const float* delta, int epi, bool lo_zero, double* u, DfBuffers df,
+                          int PxDf, int* emax, cudaStream_t s);
+// One pass in parity order: both blocks of T^{-1} (which = 0) or T along
+// `axis` as one CTA-pair launch (tc_pair_kernels.cu).  Writes the split array
+// `out` (EPI_STORE, or EPI_DIV with lambdas in mode order) or, with out32 (the
+// z pass only), FP32.
+cudaError_t launch_mode_product_fold(const FoldGeom& g, float c, int axis, const DevAxis* ax, int which, TcBuffers in,
+                                     TcBuffers out, float* out32, int epi, int* err_flag, int num_sms, cudaStream_t s);
 // Tensor maps and launch data of one BF16x3 mode product, prepared on the host.
 struct TcPassPlan;
 // One BF16x3 mode product along `axis` reading the split array `in` and
@@ -331,6 +372,13 @@ struct TcGroupItem {
   double* out64;
   DfBuffers df;
   const float *lamx, *lamy, *lamz;
+  // parity-order problem (two queue entries): its grid, all three axes' data
+  // and, for the last pass, the FP32 output; the node-order fields g, W, out64,
+  // df and lam* are then unused
+  const FoldGeom* fold;
+  const DevAxis* ax;
+  float* out32;
+  float c;
 };
 // Bytes of the device (and pinned host) table of a grouped launch.
 size_t tc_group_table_bytes(int count);

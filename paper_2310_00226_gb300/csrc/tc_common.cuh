@@ -31,7 +31,7 @@ constexpr int TMEM_COLS = 2 * BN;  // 512
 // for the outputs that read and write FP64 / double-FP32 solution arrays
 // (12-16 more bytes per element), which need more loads in flight to keep up
 // with the MMAs.  Threads: producer warp, MMA warp, epilogue warps.
-__host__ __device__ constexpr int epi_warps(int mode) { return mode >= 2 ? 16 : 8; }
+__host__ __device__ constexpr int epi_warps(int mode) { return mode >= 2 && mode <= 6 ? 16 : 8; }
 __host__ __device__ constexpr int num_threads(int mode) { return 64 + 32 * epi_warps(mode); }
 
 // Instruction descriptor, kind::f16: FP32 accumulator (bits 4-5 = 1), A and
@@ -61,6 +61,8 @@ struct TcArgs {
   int rows;            // valid tile rows per batch (x: ny*nz, y: Px, z: Px*ny)
   int nout;            // valid outputs (length of the output axis)
   int nx, ny, nz, Px;
+  int xlim;            // x pass: columns of the output rows this pass may write (Px, or a parity block's share)
+  float* out32;        // OUT_F32
   __nv_bfloat16* out_hi;
   __nv_bfloat16* out_lo;
   double* out64;
@@ -108,7 +110,8 @@ inline long long pair_tiles(const TcArgs& a) {
 //   OUT_DF_ACCUM_F64 : out64 = (double)hi + (double)lo, (hi, lo) = (hi, lo) + acc
 enum : int {
   OUT_SPLIT = 0, OUT_DIV_SPLIT = 1, OUT_F64 = 2, OUT_F64_ACCUM = 3,
-  OUT_DF_STORE = 4, OUT_DF_ACCUM = 5, OUT_DF_ACCUM_F64 = 6
+  OUT_DF_STORE = 4, OUT_DF_ACCUM = 5, OUT_DF_ACCUM_F64 = 6,
+  OUT_F32 = 7  // the accumulator itself (z pass of a parity-order solve)
 };
 
 // Split two FP32 values into bf16 hi + lo pairs (packed bf16x2: element 0 in
@@ -234,7 +237,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcArgs& a, int row, int col
         for (int k = 0; k < 4; ++k) {
           const int r = 8 * k + (lane >> 2), seg = lane & 3;
           const uint4 val = *reinterpret_cast<const uint4*>(xstage + r * XSTAGE_ROW + 16 * seg);
-          if (row0 + r < a.rows && col0 + 8 * seg + 8 <= a.Px)  // Px is a multiple of 16
+          if (row0 + r < a.rows && col0 + 8 * seg + 8 <= a.xlim)  // a multiple of 16
             *reinterpret_cast<uint4*>(dst + (size_t)(row0 + r) * a.Px + col0 + 8 * seg) = val;
         }
         __syncwarp();
@@ -273,7 +276,14 @@ __device__ __forceinline__ void epilogue_chunk(const TcArgs& a, int row, int col
       v[q] *= sc_out;
     }
   }
-  if (MODE == OUT_DF_STORE || MODE == OUT_DF_ACCUM || MODE == OUT_DF_ACCUM_F64) {
+  if (MODE == OUT_F32) {
+    float* p = a.out32 + rowoff + (size_t)col0 * cs;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) {
+      if (full || col0 + q < a.nout) *p = v[q];
+      p += cs;
+    }
+  } else if (MODE == OUT_DF_STORE || MODE == OUT_DF_ACCUM || MODE == OUT_DF_ACCUM_F64) {
     // z pass only: row = i + Px*j is also the index of (i, j, 0) in the
     // double-FP32 arrays (pitch Px); the FP64 solution has pitch nx.  The
     // store writes zeros into the pad columns i >= nx (the residual stencil
@@ -363,6 +373,11 @@ struct PassSetup {
 cudaError_t prepare_pass(const Geom& g, int axis, const DevAxis& W, int which, TcBuffers in, TcBuffers out,
                          double* out64, int epi, const float* lamx, const float* lamy, const float* lamz, int* err_flag,
                          DfBuffers df, int nprod, const F16Pass* f16, bool pair, PassSetup& ps);
+
+// One parity block (par = 0 even, 1 odd) of a pass in parity order, for the
+// pair kernel: the block's part of every array by base offset, its own extents.
+cudaError_t prepare_parity_pass(const FoldGeom& g, float c, int axis, const DevAxis* ax, int which, int par,
+                                TcBuffers in, TcBuffers out, float* out32, int epi, int* err_flag, PassSetup& ps);
 
 // Launch the CTA-pair kernel for one prepared pass over `work_pairs` pair
 // tiles (tc_pair_kernels.cu).

@@ -504,7 +504,7 @@ cudaError_t prepare_pass(const Geom& g, int axis, const DevAxis& W, int which, T
     a.normW = W.normW[which];
     a.div_bound = f16->div_bound;
   }
-  a.nx = g.nx; a.ny = g.ny; a.nz = g.nz; a.Px = g.Px;
+  a.nx = g.nx; a.ny = g.ny; a.nz = g.nz; a.Px = g.Px; a.xlim = g.Px;
   a.out_hi = out.hi; a.out_lo = out.lo; a.out64 = out64;
   a.lamx = lamx; a.lamy = lamy; a.lamz = lamz; a.c = (float)g.c;
   a.err = err_flag;
@@ -552,6 +552,62 @@ cudaError_t prepare_pass(const Geom& g, int axis, const DevAxis& W, int which, T
   a.n_tiles = (W.n + a.bn - 1) / a.bn;
   a.k_blocks = (nin + BK - 1) / BK;
   a.kc = (fmt == 1 && SEM3D_TC_CHUNK_KBLOCKS > 0) ? SEM3D_TC_CHUNK_KBLOCKS : a.k_blocks;
+  return cudaSuccess;
+}
+
+cudaError_t prepare_parity_pass(const FoldGeom& g, float c, int axis, const DevAxis* ax, int which, int par,
+                                TcBuffers in, TcBuffers out, float* out32, int epi, int* err_flag, PassSetup& ps) {
+  if ((out32 && (axis != 2 || epi != EPI_STORE)) || (epi == EPI_DIV && axis != 0)) return cudaErrorInvalidValue;
+  const DevAxis& W = ax[axis];
+  const int n = par == 0 ? g.ne[axis] : g.no[axis];  // contracted and output extent of the block
+  const uint64_t Px = (uint64_t)g.Px, ny = (uint64_t)g.ny, nz = (uint64_t)g.nz;
+  // offset of the odd part along the axis
+  const size_t off = par == 0 ? 0 : axis == 0 ? (size_t)g.Pe : axis == 1 ? (size_t)g.ne[1] * Px : (size_t)g.ne[2] * Px * ny;
+  TcArgs& a = ps.a;
+  a = TcArgs{};
+  ps.mode = out32 ? OUT_F32 : epi == EPI_DIV ? OUT_DIV_SPLIT : OUT_SPLIT;
+  a.nx = g.nx; a.ny = g.ny; a.nz = g.nz; a.Px = g.Px;
+  a.xlim = par == 0 ? g.Pe : g.Po;
+  a.out_hi = out.hi + off; a.out_lo = out.lo + off;
+  a.out32 = out32 ? out32 + off : nullptr;
+  a.lamx = ax[0].lamf_par + (axis == 0 && par ? g.ne[0] : 0);
+  a.lamy = ax[1].lamf_par;
+  a.lamz = ax[2].lamf_par;
+  a.c = c;
+  a.err = err_flag;
+  const __nv_bfloat16 *ih = in.hi + off, *il = in.lo + off;
+  bool ok = true;
+  if (axis == 0) {
+    const uint64_t dims[2] = {(uint64_t)n, ny * nz}, str[1] = {Px * 2};
+    const uint32_t box[2] = {BK, 128};
+    ok = make_map(&ps.mAh, ih, 2, dims, str, box, SWZ_K) && make_map(&ps.mAl, il, 2, dims, str, box, SWZ_K);
+    a.rows = g.ny * g.nz; a.batches = 1;
+  } else if (axis == 1) {
+    const uint64_t dims[3] = {Px, (uint64_t)n, nz}, str[2] = {Px * 2, Px * ny * 2};
+    const uint32_t box[3] = {64, BK, 1};
+    ok = make_map(&ps.mAh, ih, 3, dims, str, box, SWZ_MN) && make_map(&ps.mAl, il, 3, dims, str, box, SWZ_MN);
+    a.rows = g.Px; a.batches = g.nz;
+  } else {
+    const uint64_t dims[2] = {Px * ny, (uint64_t)n}, str[1] = {Px * ny * 2};
+    const uint32_t box[2] = {64, BK};
+    ok = make_map(&ps.mAh, ih, 2, dims, str, box, SWZ_MN) && make_map(&ps.mAl, il, 2, dims, str, box, SWZ_MN);
+    a.rows = g.Px * g.ny; a.batches = 1;
+  }
+  a.bn = tile_outputs(n);
+  {
+    const int pitch = pad16(n);
+    const size_t woff = par == 0 ? 0 : (size_t)g.ne[axis] * pad16(g.ne[axis]);
+    const uint64_t dims[2] = {(uint64_t)n, (uint64_t)n}, str[1] = {(uint64_t)pitch * 2};
+    const uint32_t box[2] = {BK, (uint32_t)(a.bn / 2)};
+    ok = ok && make_map(&ps.mBh, W.Wp_hi[which] + woff, 2, dims, str, box, SWZ_K) &&
+         make_map(&ps.mBl, W.Wp_lo[which] + woff, 2, dims, str, box, SWZ_K);
+  }
+  if (!ok) return cudaErrorInvalidValue;
+  a.nout = n;
+  a.m_tiles = (a.rows + BM - 1) / BM;
+  a.n_tiles = (n + a.bn - 1) / a.bn;
+  a.k_blocks = (n + BK - 1) / BK;
+  a.kc = a.k_blocks;
   return cudaSuccess;
 }
 

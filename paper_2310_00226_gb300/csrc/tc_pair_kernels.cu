@@ -30,11 +30,20 @@ using namespace tcx;
 // epilogue warps of both CTAs release a TMEM buffer on the leader's "tempty"
 // barrier.  Pairs of clusters pack every SM (clusters of 4 leave SMs idle on
 // GPCs whose SM count is not a multiple of 4).
-constexpr int P_STAGES = 6;
+//
+// Epilogue warps: as the one-CTA kernel, but 16 for the division pass, whose
+// epilogue (a reciprocal and a shuffle per value) otherwise outlasts the
+// loads: n = 511 in parity order 207 -> 186 us.  Their staging buffers take
+// the place of one operand stage.  16 warps are worth nothing to the other
+// split outputs.
+__host__ __device__ constexpr int pair_epi(int mode) { return mode == OUT_DIV_SPLIT ? 16 : epi_warps(mode); }
+__host__ __device__ constexpr int pair_threads(int mode) { return 64 + 32 * pair_epi(mode); }
+__host__ __device__ constexpr int pair_stages(int mode) { return mode == OUT_DIV_SPLIT ? 5 : 6; }
 constexpr int P_B_TILE_BYTES = (BN / 2) * BK * 2;  // 8 KB: this CTA's half of W
 constexpr int P_STAGE_BYTES = 2 * A_TILE_BYTES + 2 * P_B_TILE_BYTES;  // 32 KB
-__host__ __device__ constexpr int pair_smem_bytes(int pass) {
-  return P_STAGES * P_STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/ + (pass == 0 ? 8 * XSTAGE_BYTES : 0);
+__host__ __device__ constexpr int pair_smem_bytes(int pass, int mode) {
+  return pair_stages(mode) * P_STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/ +
+         (pass == 0 ? pair_epi(mode) * XSTAGE_BYTES : 0);
 }
 
 __device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
@@ -84,6 +93,7 @@ struct ProblemGroup {
 
 template <int PASS, int MODE, int NP, class Src>
 __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
+  constexpr int P_STAGES = pair_stages(MODE);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P_STAGES * P_STAGE_BYTES);
@@ -104,7 +114,7 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < P_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 2 * epi_warps(MODE)); }
+    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 2 * pair_epi(MODE)); }
     mbar_init(drain_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -227,7 +237,7 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
     const int quad = warp & 3;
     const int slice = (warp - 2) >> 2;
     uint8_t* xstage = PASS == 0 ? smem + P_STAGES * P_STAGE_BYTES + 256 + (warp - 2) * XSTAGE_BYTES : nullptr;
-    constexpr int SLICES = epi_warps(MODE) / 4;  // warps per lane quadrant; they take 32-output chunks in turn
+    constexpr int SLICES = pair_epi(MODE) / 4;  // warps per lane quadrant; they take 32-output chunks in turn
     const uint32_t tempty_leader0 = mapa_shared(tempty_bar(0), 0);
     float vmax = 0.f;
     int cc = 0, cursor = 0;
@@ -242,17 +252,25 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
       const int buf = cc & 1;
       if (!mbar_wait(tfull_bar(buf), (cc >> 1) & 1, err, KERN_SPLIT_PAIR | WAIT_EPILOGUE)) break;
       tc_fence_after();
+      // this warp's chunks of the tile (warp-uniform); the accumulator goes back
+      // once the last one is in registers, before it is converted and stored
+      const int cols = any ? min(a.bn, a.nout - t.nt * a.bn) : 0;
+      if (slice * 32 >= cols) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_remote(tempty_leader0 + 8u * buf);
+      }
 #pragma unroll 1
-      for (int ch = slice; ch * 32 < a.bn; ch += SLICES) {
-        const int col0 = t.nt * a.bn + ch * 32;
-        if (col0 >= a.nout || !any) break;  // warp-uniform
+      for (int ch = slice; ch * 32 < cols; ch += SLICES) {
         float v[32];
         tmem_ld32(lane_addr + (uint32_t)(buf * BN + ch * 32), v);
-        epilogue_chunk<PASS, MODE, NP, 0>(a, row, col0, b, v, 1.f, 1.f, vmax, xstage);
+        if ((ch + SLICES) * 32 >= cols) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_remote(tempty_leader0 + 8u * buf);
+        }
+        epilogue_chunk<PASS, MODE, NP, 0>(a, row, t.nt * a.bn + ch * 32, b, v, 1.f, 1.f, vmax, xstage);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(tempty_leader0 + 8u * buf);
     }
   }
   __syncwarp();
@@ -266,7 +284,7 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
 }
 
 template <int PASS, int MODE, int NP>
-__global__ void __launch_bounds__(num_threads(MODE), 1)
+__global__ void __launch_bounds__(pair_threads(MODE), 1)
     mode_product_bf16x3_pair_kernel(const __grid_constant__ CUtensorMap tmA_hi,
                                     const __grid_constant__ CUtensorMap tmA_lo,
                                     const __grid_constant__ CUtensorMap tmB_hi,
@@ -280,33 +298,45 @@ __global__ void __launch_bounds__(num_threads(MODE), 1)
 // starting at tab[q].tile0; each problem brings its own tensor maps and
 // epilogue arguments in the device table (64-byte aligned).
 template <int PASS, int MODE, int NP>
-__global__ void __launch_bounds__(num_threads(MODE), 1)
+__global__ void __launch_bounds__(pair_threads(MODE), 1)
     mode_product_bf16x3_pair_group_kernel(const TcGroupEntry* __restrict__ tab, int count, int total, int* err,
                                           int stall) {
   const ProblemGroup src{tab, count, total};
   pair_body<PASS, MODE, NP>(src, err, stall);
 }
 
+// One pass in parity order: its two blocks as a group of two problems, kept
+// in the kernel's parameters.
+struct FoldPass {
+  TcGroupEntry e[2];
+};
+
+template <int PASS, int MODE>
+__global__ void __launch_bounds__(pair_threads(MODE), 1)
+    mode_product_fold_kernel(const __grid_constant__ FoldPass f, int total, int* err, int stall) {
+  const ProblemGroup src{f.e, 2, total};
+  pair_body<PASS, MODE, 3>(src, err, stall);
+}
+
 // CTA-pair launch: clusters of 2, one pair per pair of SMs, persistent over
 // pair tiles.
-template <int PASS, int MODE, int NP>
-cudaError_t launch_tc_pair(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
-                           const TcArgs& a, long long work_pairs, int num_sms, cudaStream_t s) {
-  auto kern = mode_product_bf16x3_pair_kernel<PASS, MODE, NP>;
-  static std::atomic<int> max_pairs_cache{0};  // per instantiation: co-resident clusters of 2 CTAs
+// `max_pairs`: the kernel's co-resident clusters of 2 CTAs, asked for once.
+template <class Kern, class... Args>
+cudaError_t launch_pairs(Kern kern, std::atomic<int>& max_pairs_cache, int pass, int mode, long long work_pairs,
+                         int num_sms, cudaStream_t s, const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(num_threads(MODE));
-  cfg.dynamicSmemBytes = pair_smem_bytes(PASS);
+  cfg.blockDim = dim3(pair_threads(mode));
+  cfg.dynamicSmemBytes = pair_smem_bytes(pass, mode);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int max_pairs = max_pairs_cache.load(std::memory_order_relaxed);
   if (max_pairs == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pair_smem_bytes(PASS));
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pair_smem_bytes(pass, mode));
     if (e != cudaSuccess) return e;
     cfg.gridDim = dim3(2 * (num_sms / 2));
     int n = 0;
@@ -319,7 +349,22 @@ cudaError_t launch_tc_pair(const CUtensorMap& a0, const CUtensorMap& a1, const C
   const long long pairs = work_pairs < max_pairs ? work_pairs : max_pairs;
   cfg.gridDim = dim3((unsigned)(2 * pairs));
   cfg.stream = s;
-  return cudaLaunchKernelEx(&cfg, kern, a0, a1, b0, b1, a);
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+template <int PASS, int MODE, int NP>
+cudaError_t launch_tc_pair(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
+                           const TcArgs& a, long long work_pairs, int num_sms, cudaStream_t s) {
+  static std::atomic<int> max_pairs{0};
+  return launch_pairs(mode_product_bf16x3_pair_kernel<PASS, MODE, NP>, max_pairs, PASS, MODE, work_pairs, num_sms, s,
+                      a0, a1, b0, b1, a);
+}
+
+template <int PASS, int MODE>
+cudaError_t launch_fold_pass(const FoldPass& f, int total, int* err, int stall, int num_sms, cudaStream_t s) {
+  static std::atomic<int> max_pairs{0};
+  return launch_pairs(mode_product_fold_kernel<PASS, MODE>, max_pairs, PASS, MODE, total, num_sms, s, f, total, err,
+                      stall);
 }
 
 template <int PASS>
@@ -354,34 +399,9 @@ cudaError_t launch_tc_pair_mode(int mode, int nprod, const CUtensorMap& a0, cons
 template <int PASS, int MODE, int NP>
 cudaError_t launch_pair_group_t(const TcGroupEntry* tab, int count, int total, int* err, int stall, int num_sms,
                                 cudaStream_t s) {
-  auto kern = mode_product_bf16x3_pair_group_kernel<PASS, MODE, NP>;
-  static std::atomic<int> max_pairs_cache{0};
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(num_threads(MODE));
-  cfg.dynamicSmemBytes = pair_smem_bytes(PASS);
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int max_pairs = max_pairs_cache.load(std::memory_order_relaxed);
-  if (max_pairs == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pair_smem_bytes(PASS));
-    if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3(2 * (num_sms / 2));
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (n < 1) return cudaErrorInvalidConfiguration;
-    max_pairs = n;
-    max_pairs_cache.store(n, std::memory_order_relaxed);
-  }
-  const int pairs = total < max_pairs ? total : max_pairs;
-  cfg.gridDim = dim3((unsigned)(2 * pairs));
-  cfg.stream = s;
-  return cudaLaunchKernelEx(&cfg, kern, tab, count, total, err, stall);
+  static std::atomic<int> max_pairs{0};
+  return launch_pairs(mode_product_bf16x3_pair_group_kernel<PASS, MODE, NP>, max_pairs, PASS, MODE, total, num_sms, s,
+                      tab, count, total, err, stall);
 }
 
 cudaError_t launch_pair_group(int axis, int mode, int nprod, const TcGroupEntry* tab, int count, int total, int* err,
@@ -393,6 +413,7 @@ cudaError_t launch_pair_group(int axis, int mode, int nprod, const TcGroupEntry*
     if (axis == 0 && mode == OUT_DIV_SPLIT) return launch_pair_group_t<0, OUT_DIV_SPLIT, 3>(tab, count, total, err, stall, num_sms, s);
     if (axis == 1 && mode == OUT_SPLIT) return launch_pair_group_t<1, OUT_SPLIT, 3>(tab, count, total, err, stall, num_sms, s);
     if (axis == 2 && mode == OUT_SPLIT) return launch_pair_group_t<2, OUT_SPLIT, 3>(tab, count, total, err, stall, num_sms, s);
+    if (axis == 2 && mode == OUT_F32) return launch_pair_group_t<2, OUT_F32, 3>(tab, count, total, err, stall, num_sms, s);
     if (axis == 2 && mode == OUT_F64) return launch_pair_group_t<2, OUT_F64, 3>(tab, count, total, err, stall, num_sms, s);
     if (axis == 2 && mode == OUT_F64_ACCUM) return launch_pair_group_t<2, OUT_F64_ACCUM, 3>(tab, count, total, err, stall, num_sms, s);
     if (axis == 2 && mode == OUT_DF_STORE) return launch_pair_group_t<2, OUT_DF_STORE, 3>(tab, count, total, err, stall, num_sms, s);
@@ -411,7 +432,8 @@ cudaError_t launch_pair_group(int axis, int mode, int nprod, const TcGroupEntry*
 
 }  // namespace
 
-size_t tc_group_table_bytes(int count) { return ((size_t)count * sizeof(TcGroupEntry) + 255) & ~size_t(255); }
+// Two entries per problem: a parity-order problem queues its two blocks.
+size_t tc_group_table_bytes(int count) { return ((size_t)count * 2 * sizeof(TcGroupEntry) + 255) & ~size_t(255); }
 
 cudaError_t launch_mode_product_bf16x3_grouped(int count, const TcGroupItem* items, int axis, int which, int epi,
                                                int nprod, int* err_flag, void* dev_table, void* host_table,
@@ -421,27 +443,58 @@ cudaError_t launch_mode_product_bf16x3_grouped(int count, const TcGroupItem* ite
     return cudaErrorInvalidValue;
   TcGroupEntry* tab = static_cast<TcGroupEntry*>(host_table);
   long long total = 0;
-  int mode = -1;
+  int mode = -1, entries = 0;
   for (int q = 0; q < count; ++q) {
     const TcGroupItem& it = items[q];
+    if (it.fold && nprod != 3) return cudaErrorInvalidValue;
+    for (int par = 0; par < (it.fold ? 2 : 1); ++par) {
+      PassSetup ps;
+      cudaError_t e = it.fold ? prepare_parity_pass(*it.fold, it.c, axis, it.ax, which, par, it.in, it.out, it.out32,
+                                                    epi, err_flag, ps)
+                              : prepare_pass(*it.g, axis, *it.W, which, it.in, it.out, it.out64, epi, it.lamx, it.lamy,
+                                             it.lamz, err_flag, it.df, nprod, nullptr, true, ps);
+      if (e != cudaSuccess) return e;
+      if (mode >= 0 && ps.mode != mode) return cudaErrorInvalidValue;  // one epilogue mode per launch
+      mode = ps.mode;
+      TcGroupEntry& en = tab[entries++];
+      en.A_hi = ps.mAh; en.A_lo = ps.mAl; en.B_hi = ps.mBh; en.B_lo = ps.mBl;
+      en.a = ps.a;
+      en.tile0 = (int)total;
+      total += pair_tiles(ps.a);
+      if (total >= (1LL << 31)) return cudaErrorInvalidValue;
+    }
+  }
+  cudaError_t e = cudaMemcpyAsync(dev_table, host_table, (size_t)entries * sizeof(TcGroupEntry), cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return e;
+  if (total == 0) return cudaSuccess;
+  return launch_pair_group(axis, mode, nprod, static_cast<const TcGroupEntry*>(dev_table), entries, (int)total, err_flag,
+                           tc_take_stall(), num_sms, s);
+}
+
+cudaError_t launch_mode_product_fold(const FoldGeom& g, float c, int axis, const DevAxis* ax, int which, TcBuffers in,
+                                     TcBuffers out, float* out32, int epi, int* err_flag, int num_sms, cudaStream_t s) {
+  FoldPass f;
+  long long total = 0;
+  int mode = 0;
+  for (int par = 0; par < 2; ++par) {
     PassSetup ps;
-    cudaError_t e = prepare_pass(*it.g, axis, *it.W, which, it.in, it.out, it.out64, epi, it.lamx, it.lamy, it.lamz,
-                                 err_flag, it.df, nprod, nullptr, true, ps);
+    const cudaError_t e = prepare_parity_pass(g, c, axis, ax, which, par, in, out, out32, epi, err_flag, ps);
     if (e != cudaSuccess) return e;
-    if (mode >= 0 && ps.mode != mode) return cudaErrorInvalidValue;  // one epilogue mode per launch
-    mode = ps.mode;
-    TcGroupEntry& en = tab[q];
+    TcGroupEntry& en = f.e[par];
     en.A_hi = ps.mAh; en.A_lo = ps.mAl; en.B_hi = ps.mBh; en.B_lo = ps.mBl;
     en.a = ps.a;
     en.tile0 = (int)total;
     total += pair_tiles(ps.a);
-    if (total >= (1LL << 31)) return cudaErrorInvalidValue;
+    mode = ps.mode;
   }
-  cudaError_t e = cudaMemcpyAsync(dev_table, host_table, (size_t)count * sizeof(TcGroupEntry), cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return e;
-  if (total == 0) return cudaSuccess;
-  return launch_pair_group(axis, mode, nprod, static_cast<const TcGroupEntry*>(dev_table), count, (int)total, err_flag,
-                           tc_take_stall(), num_sms, s);
+  if (total >= (1LL << 31)) return cudaErrorInvalidValue;
+  const int stall = tc_take_stall(), t = (int)total;
+  if (axis == 0 && mode == OUT_SPLIT) return launch_fold_pass<0, OUT_SPLIT>(f, t, err_flag, stall, num_sms, s);
+  if (axis == 0 && mode == OUT_DIV_SPLIT) return launch_fold_pass<0, OUT_DIV_SPLIT>(f, t, err_flag, stall, num_sms, s);
+  if (axis == 1 && mode == OUT_SPLIT) return launch_fold_pass<1, OUT_SPLIT>(f, t, err_flag, stall, num_sms, s);
+  if (axis == 2 && mode == OUT_SPLIT) return launch_fold_pass<2, OUT_SPLIT>(f, t, err_flag, stall, num_sms, s);
+  if (axis == 2 && mode == OUT_F32) return launch_fold_pass<2, OUT_F32>(f, t, err_flag, stall, num_sms, s);
+  return cudaErrorInvalidValue;
 }
 
 namespace tcx {

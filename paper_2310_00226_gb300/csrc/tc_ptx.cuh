@@ -108,9 +108,14 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
   return r;
 }
 
-// Arrive on an mbarrier given by its shared::cluster address (any CTA of the cluster).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+// Arrive on an mbarrier given by its shared::cluster address (any CTA of the
+// cluster), with the default release at CTA scope: the epilogues use it to
+// hand back an accumulator, whose reads are complete (tcgen05.wait::ld) and
+// ordered by tcgen05.fence::before_thread_sync; no other memory is handed
+// over.  A cluster-scope release would also wait for every global store of the
+// tile to be acknowledged before the next accumulator can be started.
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {

@@ -407,17 +407,24 @@ __global__ void __launch_bounds__(t_threads(MODE), 1)
       tc_fence_after();
       const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * T_BN + slice * COLS);
       const int row = mt * T_BM + quad * 32 + lane;
-#pragma unroll 1
-      for (int ch = 0; ch < COLS / 32; ++ch) {
-        const int col0 = nt * T_BN + slice * COLS + ch * 32;
-        if (col0 >= a.nout || mt >= a.m_tiles) break;  // warp-uniform
-        float v[32];
-        tmem_ld32(lane_addr + (uint32_t)(ch * 32), v);
-        tf32_epilogue<MODE>(a, row, col0, v);
+      // the accumulator goes back once the warp's last chunk is in registers
+      const int cols = mt < a.m_tiles ? min(COLS, a.nout - nt * T_BN - slice * COLS) : 0;  // warp-uniform
+      if (cols <= 0) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_remote(tempty_leader0 + 8u * buf);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(tempty_leader0 + 8u * buf);
+#pragma unroll 1
+      for (int c0 = 0; c0 < cols; c0 += 32) {
+        float v[32];
+        tmem_ld32(lane_addr + (uint32_t)c0, v);
+        if (c0 + 32 >= cols) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_remote(tempty_leader0 + 8u * buf);
+        }
+        tf32_epilogue<MODE>(a, row, nt * T_BN + slice * COLS + c0, v);
+      }
     }
   }
   __syncwarp();

@@ -47,3 +47,64 @@ def check(n3, k, bc, prec, sweeps, run):
 @pytest.mark.parametrize("n3,k,bc", GRIDS)
 def test_fp64_solve(n3, k, bc):
     check(n3, k, bc, "fp64", 1, lambda m, p, f, u: p.solve(f, u))
+
+
+# Split-bf16 solves in parity order (all axes >= 255): even and odd n, pads in
+# either half of the x pitch, output tiles of 128 to 256, both boundary
+# conditions, k with and without the vector residuals, k > 8 and Neumann data
+# (FP64 residuals), one node more and less than the rule's limit.
+FOLD_GRIDS = [
+    ((255, 255, 255), 4, "dirichlet"), ((256, 257, 271), 1, "dirichlet"), ((275, 257, 260), 3, "dirichlet"),
+    ((254, 255, 289), 1, "dirichlet"), ((323, 255, 259), 2, "dirichlet"), ((266, 256, 261), 5, "neumann"),
+    ((269, 259, 299), 10, "dirichlet"),
+]
+
+
+@pytest.mark.parametrize("residual", ["mixed", "fp64"])
+@pytest.mark.parametrize("n3,k,bc", FOLD_GRIDS)
+def test_refined_solve_in_parity_order(n3, k, bc, residual):
+    def run(m, p, f, u):
+        p.set_residual(residual)
+        p.solve(f, u)
+    check(n3, k, bc, "bf16x3", 3 if bc == "dirichlet" else 4, run)
+
+
+def test_parity_order_with_double_fp32_residuals_and_fp64_fmas():
+    # every residual in double-FP32: 2^-48 of the operator's terms, amplified by
+    # the conditioning (the bound), and the exact residual in FP64 FMAs
+    from paper_2310_00226_gb300 import sem3d
+    n3, k, L, c = (255, 259, 267), 4, (1.0, 1.3, 0.8), 1.5
+    axes = [sem_1d(k, (n + 1) // k, 0.0, Lb) for n, Lb in zip(n3, L)]
+    F = random_rhs(*n3, seed=5)
+    f = torch.from_numpy(F).cuda()
+    ref = refined_solve(F, *axes, c, 1)
+    with sem3d.Plan(*n3, k, L, c) as p:
+        p.set_precision("bf16x3", 3)
+        for residual, exact, bound in (("df", "fixed", kappa(axes, c) * 2.0**-48), ("mixed", "fp64", 1e-12)):
+            p.set_residual(residual)
+            p.set_exact_residual(exact)
+            u = torch.full_like(f, float("nan"))
+            p.solve(f, u)
+            p.sync_check()
+            assert np.abs(u.cpu().numpy() - ref).max() / np.abs(ref).max() <= bound
+
+
+def test_batch_of_both_orders_is_bit_identical_to_single_solves():
+    from paper_2310_00226_gb300 import sem3d
+    probs = [((255, 256, 257), 1), ((63, 95, 127), 2), ((257, 260, 299), 3), ((255, 511, 127), 4), ((263, 255, 255), 4)]
+    plans = [sem3d.Plan(*n3, k, (1.0, 1.0, 1.0), 0.5 * q) for q, (n3, k) in enumerate(probs)]
+    fs = [torch.from_numpy(random_rhs(*n3, seed=q)).cuda() for q, (n3, _) in enumerate(probs)]
+    for residual in ("mixed", "fp64"):
+        for p in plans:
+            p.set_precision("bf16x3", 3)
+            p.set_residual(residual)
+        us = [torch.full_like(f, float("nan")) for f in fs]
+        sem3d.solve_batched(plans, fs, us)
+        plans[0].sync_check()
+        for p, f, u in zip(plans, fs, us):
+            one = torch.full_like(f, float("nan"))
+            p.solve(f, one)
+            p.sync_check()
+            assert torch.equal(one, u)
+    for p in plans:
+        p.close()
