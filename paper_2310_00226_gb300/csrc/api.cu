@@ -109,33 +109,101 @@ struct sem3d_plan {
 
 namespace {
 
-template <class T>
-sem3d_status dev_upload(sem3d_plan* p, T** dst, const T* src, size_t count) {
-  void* d = nullptr;
-  cudaError_t e = cudaMalloc(&d, count * sizeof(T) + 16);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(setup)");
-  p->owned.push_back(d);
-  e = cudaMemcpy(d, src, count * sizeof(T), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(setup)");
-  *dst = static_cast<T*>(d);
-  return SEM3D_OK;
-}
-
-// Append W (n x n row-major FP64) split into bf16 hi + lo with row pitch Kp.
-void split_matrix(const double* W, int n, int Kp, std::vector<__nv_bfloat16>& hi, std::vector<__nv_bfloat16>& lo) {
-  const size_t at = hi.size();
-  hi.resize(at + (size_t)n * Kp, __float2bfloat16_rn(0.f));
-  lo.resize(at + (size_t)n * Kp, __float2bfloat16_rn(0.f));
-  for (int o = 0; o < n; ++o)
-    for (int t = 0; t < n; ++t) {
-      const float x = (float)W[(size_t)o * n + t];
-      const __nv_bfloat16 h = __float2bfloat16_rn(x);
-      hi[at + (size_t)o * Kp + t] = h;
-      lo[at + (size_t)o * Kp + t] = __float2bfloat16_rn(x - __bfloat162float(h));
-    }
-}
-
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
+
+// One device allocation carved into 256-byte aligned arrays: `add` them all
+// (the pointers are offsets until then), then `alloc`, which makes them
+// addresses and uploads what has host data.
+struct Slab {
+  struct Part { void** dst; size_t at, bytes; const void* src; };
+  std::vector<Part> parts;
+  size_t bytes = 0;
+  template <class T>
+  void add(T** dst, size_t count, const T* src = nullptr) {
+    parts.push_back({reinterpret_cast<void**>(dst), bytes, count * sizeof(T), src});
+    bytes += align256(count * sizeof(T) + 16);
+  }
+  sem3d_status alloc(std::vector<void*>& owned) {
+    void* d = nullptr;
+    cudaError_t e = cudaMalloc(&d, bytes + 256);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(setup)");
+    owned.push_back(d);
+    for (const Part& q : parts) {
+      *q.dst = static_cast<char*>(d) + q.at;
+      if (q.src && q.bytes && (e = cudaMemcpy(*q.dst, q.src, q.bytes, cudaMemcpyHostToDevice)) != cudaSuccess)
+        return cuda_fail(e, "cudaMemcpy(setup)");
+    }
+    return SEM3D_OK;
+  }
+};
+
+// Device data of one axis.  `same`: an axis of this plan with the same nodes,
+// whose basis is shared (the rows of H are not: the x axis has c on them).
+sem3d_status setup_axis(sem3d_plan* p, int a, const DevAxis* same, double* scratch, std::vector<double>& hq) {
+  const Axis1D& A = *p->ax[a];
+  DevAxis& D = p->dev[a];
+  const int k = p->k, n = A.n;
+  sem3d_status st;
+  if (same) {
+    D = *same;
+  } else {
+    D.n = n; D.k = k; D.Kp = pad16(n); D.ne = A.ne; D.no = A.no;
+    const size_t nn = (size_t)n * n, nk = (size_t)n * D.Kp;
+    const size_t np = (size_t)A.ne * pad16(A.ne) + (size_t)A.no * pad16(A.no);
+    const std::vector<float> lf(A.lam.begin(), A.lam.end()), lp(A.lam_par.begin(), A.lam_par.end());
+    Slab s;
+    s.add(&D.M, n, A.M.data());
+    s.add(&D.lam, n, A.lam.data());
+    s.add(&D.lam_par, n, A.lam_par.data());
+    s.add(&D.lamf, n, lf.data());
+    s.add(&D.lamf_par, n, lp.data());
+    s.add(&D.Hband, A.Hband.size(), A.Hband.data());
+    s.add(&D.band_lo, n, A.band_lo.data());
+    s.add(&D.band_hi, n, A.band_hi.data());
+    for (int w = 0; w < 2; ++w) {
+      s.add(&D.par[w], A.par[w].size(), A.par[w].data());
+      s.add(&D.Wf[w], nn);
+      s.add(&D.Wt32[w], nk);
+      s.add(&D.W16_hi[w], nk);
+      s.add(&D.W16_lo[w], nk);
+      s.add(&D.W_hi[w], nk);
+      s.add(&D.W_lo[w], nk);
+      s.add(&D.Wp_hi[w], np);
+      s.add(&D.Wp_lo[w], np);
+      // fp16 pairs hold W * 2^eW16 (F16X3 tier)
+      D.eW16[w] = A.wmax[w] > 0.0 ? std::ilogb(16384.0 / A.wmax[w]) : 0;
+      D.normW[w] = (float)A.wnorm[w];
+    }
+    if ((st = s.alloc(p->owned)) != SEM3D_OK) return st;
+    CUDA_TRY(cudaMemcpy(scratch, A.Tinv.data(), nn * sizeof(double), cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpy(scratch + nn, A.T.data(), nn * sizeof(double), cudaMemcpyHostToDevice));
+    const double* const w[2] = {scratch, scratch + nn};
+    CUDA_TRY(launch_axis_copies(D, w, cudaStreamLegacy));
+  }
+  hq = A.Hq;  // the shift c joins the x operator's diagonal
+  if (a == 0)
+    for (int q = 0; q < k; ++q) hq[(size_t)q * (2 * k + 1) + k] += p->g.c;
+  // Three FP32 terms: hi + lo holds 48 bits; the remainder lo2 makes the
+  // sum exact (53 bits need at most three 24-bit pieces).
+  std::vector<float> hh(hq.size()), hl(hq.size()), hl2(hq.size());
+  for (size_t q = 0; q < hq.size(); ++q) {
+    hh[q] = (float)hq[q];
+    hl[q] = (float)(hq[q] - (double)hh[q]);
+    hl2[q] = (float)(hq[q] - (double)hh[q] - (double)hl[q]);
+  }
+  if (k <= 4)
+    for (size_t q = 0; q < hq.size(); ++q) {
+      D.Hq_hi_host[q] = hh[q];
+      D.Hq_lo_host[q] = hl[q];
+      D.Hq_lo2_host[q] = hl2[q];
+    }
+  Slab s;
+  s.add(&D.Hq, hq.size(), hq.data());
+  s.add(&D.Hq_hi, hq.size(), hh.data());
+  s.add(&D.Hq_lo, hq.size(), hl.data());
+  s.add(&D.Hq_lo2, hq.size(), hl2.data());
+  return s.alloc(p->owned);
+}
 
 // Kernel classes for sem3d_profile_read; tensor-core launches are also
 // counted per pass (x / y / z, and the last pass that writes FP64 u).
@@ -478,103 +546,22 @@ sem3d_status sem3d_setup_bc(int nx, int ny, int nz, int k, double Lx, double Ly,
   p->k = k;
   for (int a = 0; a < 3; ++a) p->L[a] = L3[a];
   std::vector<double> hq_rows[3];
-  for (int a = 0; a < 3; ++a) {
-    const Axis1D& A = *p->ax[a];
-    DevAxis& D = p->dev[a];
-    D.n = A.n; D.k = k; D.Kp = pad16(A.n);
-    sem3d_status st;
-    if ((st = dev_upload(p.get(), &D.M, A.M.data(), A.M.size())) != SEM3D_OK) return st;
-    D.ne = A.ne; D.no = A.no;
-    for (int w = 0; w < 2; ++w)
-      if ((st = dev_upload(p.get(), &D.par[w], A.par[w].data(), A.par[w].size())) != SEM3D_OK) return st;
-    if ((st = dev_upload(p.get(), &D.lam_par, A.lam_par.data(), A.lam_par.size())) != SEM3D_OK) return st;
-    {
-      std::vector<float> lp(A.lam_par.begin(), A.lam_par.end());
-      if ((st = dev_upload(p.get(), &D.lamf_par, lp.data(), lp.size())) != SEM3D_OK) return st;
+  {
+    const size_t nmax = std::max(nx, std::max(ny, nz));
+    void* d = nullptr;
+    CUDA_TRY(cudaMalloc(&d, 2 * nmax * nmax * sizeof(double)));
+    struct Scratch {
+      void* d;
+      ~Scratch() { cudaFree(d); }
+    } scratch{d};
+    for (int a = 0; a < 3; ++a) {
+      const DevAxis* same = nullptr;
+      for (int b = 0; b < a && !same; ++b)
+        if (p->ax[b] == p->ax[a]) same = &p->dev[b];
+      const sem3d_status st = setup_axis(p.get(), a, same, static_cast<double*>(scratch.d), hq_rows[a]);
+      if (st != SEM3D_OK) return st;
     }
-    if ((st = dev_upload(p.get(), &D.lam, A.lam.data(), A.lam.size())) != SEM3D_OK) return st;
-    std::vector<float> lf(A.lam.begin(), A.lam.end());
-    if ((st = dev_upload(p.get(), &D.lamf, lf.data(), lf.size())) != SEM3D_OK) return st;
-    if ((st = dev_upload(p.get(), &D.Hband, A.Hband.data(), A.Hband.size())) != SEM3D_OK) return st;
-    {
-      std::vector<double>& hq = hq_rows[a];
-      hq = A.Hq;  // the shift c joins the x operator's diagonal
-      if (a == 0)
-        for (int q = 0; q < k; ++q) hq[(size_t)q * (2 * k + 1) + k] += c;
-      if ((st = dev_upload(p.get(), &D.Hq, hq.data(), hq.size())) != SEM3D_OK) return st;
-      // Three FP32 terms: hi + lo holds 48 bits; the remainder lo2 makes the
-      // sum exact (53 bits need at most three 24-bit pieces).
-      std::vector<float> hh(hq.size()), hl(hq.size()), hl2(hq.size());
-      for (size_t q = 0; q < hq.size(); ++q) {
-        hh[q] = (float)hq[q];
-        hl[q] = (float)(hq[q] - (double)hh[q]);
-        hl2[q] = (float)(hq[q] - (double)hh[q] - (double)hl[q]);
-      }
-      if (k <= 4)
-        for (size_t q = 0; q < hq.size(); ++q) {
-          D.Hq_hi_host[q] = hh[q];
-          D.Hq_lo_host[q] = hl[q];
-          D.Hq_lo2_host[q] = hl2[q];
-        }
-      if ((st = dev_upload(p.get(), &D.Hq_hi, hh.data(), hh.size())) != SEM3D_OK) return st;
-      if ((st = dev_upload(p.get(), &D.Hq_lo, hl.data(), hl.size())) != SEM3D_OK) return st;
-      if ((st = dev_upload(p.get(), &D.Hq_lo2, hl2.data(), hl2.size())) != SEM3D_OK) return st;
-    }
-    if ((st = dev_upload(p.get(), &D.band_lo, A.band_lo.data(), A.band_lo.size())) != SEM3D_OK) return st;
-    if ((st = dev_upload(p.get(), &D.band_hi, A.band_hi.data(), A.band_hi.size())) != SEM3D_OK) return st;
-    for (int w = 0; w < 2; ++w) {
-      const std::vector<double>& Wd = (w == 0) ? A.Tinv : A.T;
-      std::vector<float> wf(Wd.begin(), Wd.end());
-      if ((st = dev_upload(p.get(), &D.Wf[w], wf.data(), wf.size())) != SEM3D_OK) return st;
-    }
-    for (int w = 0; w < 2; ++w) {  // TF32-rounded W for the TF32 tier, row pitch Kp
-      const std::vector<double>& Wd = (w == 0) ? A.Tinv : A.T;
-      std::vector<float> wt((size_t)A.n * D.Kp, 0.f);
-      for (int o = 0; o < A.n; ++o)
-        for (int t = 0; t < A.n; ++t) wt[(size_t)o * D.Kp + t] = tf32_round((float)Wd[(size_t)o * A.n + t]);
-      if ((st = dev_upload(p.get(), &D.Wt32[w], wt.data(), wt.size())) != SEM3D_OK) return st;
-    }
-    for (int w = 0; w < 2; ++w) {  // fp16 pairs of W * 2^eW for the F16X3 tier
-      const std::vector<double>& Wd = (w == 0) ? A.Tinv : A.T;
-      const int n = A.n;
-      double mx = 0.0, norm = 0.0;
-      for (int o = 0; o < n; ++o) {
-        double rs = 0.0;
-        for (int t = 0; t < n; ++t) {
-          const double v = std::fabs(Wd[(size_t)o * n + t]);
-          mx = std::max(mx, v);
-          rs += v;
-        }
-        norm = std::max(norm, rs);
-      }
-      const int eW = mx > 0.0 ? std::ilogb(16384.0 / mx) : 0;
-      D.eW16[w] = eW;
-      D.normW[w] = (float)norm;
-      std::vector<__half> h16((size_t)n * D.Kp, __float2half_rn(0.f)), l16((size_t)n * D.Kp, __float2half_rn(0.f));
-      for (int o = 0; o < n; ++o)
-        for (int t = 0; t < n; ++t) {
-          const float x = (float)std::ldexp(Wd[(size_t)o * n + t], eW);
-          const __half hh = __float2half_rn(x);
-          h16[(size_t)o * D.Kp + t] = hh;
-          l16[(size_t)o * D.Kp + t] = __float2half_rn(x - __half2float(hh));
-        }
-      if ((st = dev_upload(p.get(), &D.W16_hi[w], h16.data(), h16.size())) != SEM3D_OK) return st;
-      if ((st = dev_upload(p.get(), &D.W16_lo[w], l16.data(), l16.size())) != SEM3D_OK) return st;
-    }
-    std::vector<__nv_bfloat16> hi, lo;
-    for (int w = 0; w < 2; ++w) {
-      hi.clear();
-      lo.clear();
-      split_matrix((w == 0 ? A.Tinv : A.T).data(), A.n, D.Kp, hi, lo);
-      if ((st = dev_upload(p.get(), &D.W_hi[w], hi.data(), hi.size())) != SEM3D_OK) return st;
-      if ((st = dev_upload(p.get(), &D.W_lo[w], lo.data(), lo.size())) != SEM3D_OK) return st;
-      hi.clear();
-      lo.clear();
-      split_matrix(A.par[w].data(), A.ne, pad16(A.ne), hi, lo);
-      split_matrix(A.par[w].data() + (size_t)A.ne * A.ne, A.no, pad16(A.no), hi, lo);
-      if ((st = dev_upload(p.get(), &D.Wp_hi[w], hi.data(), hi.size())) != SEM3D_OK) return st;
-      if ((st = dev_upload(p.get(), &D.Wp_lo[w], lo.data(), lo.size())) != SEM3D_OK) return st;
-    }
+    CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));  // the copies, for solves on any stream
   }
   {
     void* d = nullptr;

@@ -100,6 +100,7 @@ struct Axis1D {
   int ne = 0, no = 0;
   std::vector<double> par[2];
   std::vector<double> lam_par;
+  double wmax[2] = {0, 0}, wnorm[2] = {0, 0};  // largest |entry| and largest row sum of |.| of T^{-1}, T
 };
 
 void gll_rule(int N, std::vector<double>& r, std::vector<double>& w);
@@ -111,6 +112,9 @@ Axis1D build_axis(int n, int k, double L, int bc = 0);
 // Pitch (elements) of the x dimension of the tensor-core working arrays and
 // of the bf16 matrices: a multiple of 16 so that every bf16 row starts on a
 // 32-byte boundary (TMA needs 16; 32 keeps row segments sector-aligned).
+#ifdef __CUDACC__
+__host__ __device__
+#endif
 inline int pad16(int n) { return (n + 15) & ~15; }
 
 struct DevAxis {
@@ -146,6 +150,11 @@ struct DevAxis {
   float normW[2] = {0.f, 0.f};
   __nv_bfloat16* W_lo[2] = {nullptr, nullptr};
 };
+
+// Fill every low-precision copy of an axis's T^{-1} and T (Wf, Wt32, W16_*,
+// W_*, Wp_*) from their FP64 form on the device: w[0] = T^{-1}, w[1] = T (n x n
+// row-major), D.par as uploaded.  (setup_kernels.cu)
+cudaError_t launch_axis_copies(const DevAxis& D, const double* const w[2], cudaStream_t s);
 
 // Epilogues of a mode-product pass.
 enum Epi : int {

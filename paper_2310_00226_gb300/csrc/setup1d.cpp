@@ -358,6 +358,16 @@ Axis1D build_axis(int n, int k, double L, int bc) {
       ax.Tinv[(size_t)j * n + i] = Q[(size_t)i * n + j] * sm;
     }
   }
+  for (int w = 0; w < 2; ++w)
+    for (int o = 0; o < n; ++o) {
+      double rs = 0.0;
+      for (int t = 0; t < n; ++t) {
+        const double v = std::fabs((w == 0 ? ax.Tinv : ax.T)[(size_t)o * n + t]);
+        ax.wmax[w] = std::max(ax.wmax[w], v);
+        rs += v;
+      }
+      ax.wnorm[w] = std::max(ax.wnorm[w], rs);
+    }
   build_parity(ax, Q);
   // Band of H = M^{-1} S: row i couples columns [lo_i, hi_i] (one or two
   // elements), stored as H[i][i+d] for d in [-k, k].
