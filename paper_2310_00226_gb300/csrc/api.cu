@@ -185,23 +185,15 @@ sem3d_status setup_axis(sem3d_plan* p, int a, const DevAxis* same, double* scrat
     for (int q = 0; q < k; ++q) hq[(size_t)q * (2 * k + 1) + k] += p->g.c;
   // Three FP32 terms: hi + lo holds 48 bits; the remainder lo2 makes the
   // sum exact (53 bits need at most three 24-bit pieces).
-  std::vector<float> hh(hq.size()), hl(hq.size()), hl2(hq.size());
-  for (size_t q = 0; q < hq.size(); ++q) {
-    hh[q] = (float)hq[q];
-    hl[q] = (float)(hq[q] - (double)hh[q]);
-    hl2[q] = (float)(hq[q] - (double)hh[q] - (double)hl[q]);
-  }
-  if (k <= 4)
+  if (k <= 8)
     for (size_t q = 0; q < hq.size(); ++q) {
-      D.Hq_hi_host[q] = hh[q];
-      D.Hq_lo_host[q] = hl[q];
-      D.Hq_lo2_host[q] = hl2[q];
+      const float hi = (float)hq[q], lo = (float)(hq[q] - (double)hi);
+      D.Hq_hi_host[q] = hi;
+      D.Hq_lo_host[q] = lo;
+      D.Hq_lo2_host[q] = (float)(hq[q] - (double)hi - (double)lo);
     }
   Slab s;
   s.add(&D.Hq, hq.size(), hq.data());
-  s.add(&D.Hq_hi, hq.size(), hh.data());
-  s.add(&D.Hq_lo, hq.size(), hl.data());
-  s.add(&D.Hq_lo2, hq.size(), hl2.data());
   return s.alloc(p->owned);
 }
 
@@ -471,9 +463,8 @@ sem3d_status fold_update(sem3d_plan* h, const FoldBuffers& b, double* u, int sw,
   const bool in_df = sw < ndf;
   const int epi = sw == 0 ? (in_df ? EPI_DF_STORE : EPI_STORE)
                           : in_df ? EPI_DF_ACCUM : sw == ndf ? EPI_DF_ACCUM_F64 : EPI_ACCUM;
-  // the vector double-FP32 residuals know that the first solution has no low parts
-  const bool vec = h->k == 1 || h->k == 2 || h->k == 4;
-  const DfBuffers D{b.D.hi, epi == EPI_DF_STORE && vec ? nullptr : b.D.lo};
+  // the first solution has no low parts: not written, and not read by sweep 1
+  const DfBuffers D{b.D.hi, epi == EPI_DF_STORE ? nullptr : b.D.lo};
   const bool emax = !in_df && sw < h->sweeps && use_fixed_residual(h);  // a fixed-point residual of u follows
   if (emax) CUDA_TRY(cudaMemsetAsync(h->d_fix, 0, sizeof(int), s));
   LAUNCH(h, K_SPLIT, 1, s, launch_unfold(b.g, b.delta, epi, sw == 1, u, D, h->g.Px, emax ? h->d_fix : nullptr, s));
@@ -486,7 +477,7 @@ sem3d_status fold_residual(sem3d_plan* h, const FoldBuffers& b, const double* f,
   if (sw <= df_sweeps(h)) {
     // Every residual in double-FP32 (SEM3D_RESIDUAL_DF): the rows of H must then be exact
     LAUNCH(h, K_STENCIL, 1, s,
-           launch_stencil_df(h->g, h->k, h->dev, b.D, f, nullptr, nullptr, s, b.r32, nullptr,
+           launch_stencil_df(h->g, h->k, h->dev, b.D, f, nullptr, nullptr, h->num_sms, s, b.r32, nullptr,
                              h->residual == SEM3D_RESIDUAL_DF, sw == 1));
   } else if (use_fixed_residual(h)) {
     LAUNCH(h, K_STENCIL, 2, s,
@@ -857,14 +848,13 @@ sem3d_status run_solve(sem3d_plan* h, const double* f, double* u, cudaStream_t s
         if (f16) {
           if ((st = reset_scales()) != SEM3D_OK) return st;
           LAUNCH(h, K_STENCIL, 1, s,
-                 launch_stencil_df(h->g, h->k, h->dev, D, f, nullptr, nullptr, s, r32, h->d_f16, exact_coef, q == 1));
+                 launch_stencil_df(h->g, h->k, h->dev, D, f, nullptr, nullptr, h->num_sms, s, r32, h->d_f16, exact_coef,
+                                   q == 1));
           LAUNCH(h, K_SPLIT, 1, s, launch_split_f16(h->g, r32, false, S0h, S0l, h->d_f16, s));
         } else {
-          // k in {1, 2, 4}: one vector kernel that also writes the pads; otherwise
-          // the element kernel plus a pad-zeroing kernel when Px > nx
-          const int df_launches = (h->k == 1 || h->k == 2 || h->k == 4 || h->g.Px == h->g.nx) ? 1 : 2;
-          LAUNCH(h, K_STENCIL, df_launches, s,
-                 launch_stencil_df(h->g, h->k, h->dev, D, f, S0.hi, S0.lo, s, nullptr, nullptr, exact_coef, q == 1));
+          LAUNCH(h, K_STENCIL, 1, s,
+                 launch_stencil_df(h->g, h->k, h->dev, D, f, S0.hi, S0.lo, h->num_sms, s, nullptr, nullptr, exact_coef,
+                                   q == 1));
         }
         const bool last_df = (q == ndf);
         if ((st = solve_once_bf16x3(h, S0, S1, last_df ? u : nullptr, last_df ? EPI_DF_ACCUM_F64 : EPI_DF_ACCUM, D,
@@ -1546,9 +1536,8 @@ sem3d_status batched_tc(int count, const sem3d_handle* hs, const double* const* 
       LAUNCH(h, K_SPLIT, 1, qs, launch_split(h->g, f[q], S0[q].hi, S0[q].lo, qs, fexp));
     } else if (sw > sweeps) {
     } else if (sw <= ndf) {
-      const int launches = (h->k == 1 || h->k == 2 || h->k == 4 || h->g.Px == h->g.nx) ? 1 : 2;
-      LAUNCH(h, K_STENCIL, launches, qs,
-             launch_stencil_df(h->g, h->k, h->dev, D[q], f[q], S0[q].hi, S0[q].lo, qs, nullptr, nullptr,
+      LAUNCH(h, K_STENCIL, 1, qs,
+             launch_stencil_df(h->g, h->k, h->dev, D[q], f[q], S0[q].hi, S0[q].lo, h->num_sms, qs, nullptr, nullptr,
                                h->residual == SEM3D_RESIDUAL_DF, sw == 1));
     } else if (fixed) {
       LAUNCH(h, K_STENCIL, 3, qs,

@@ -399,317 +399,6 @@ cudaError_t launch_elem(const StencilArgs& a, const DevAxis* ax, int mode, cudaS
   return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ double-FP32 residual
-//
-// The same element-wise operator evaluated in double-FP32 arithmetic: every
-// value is a pair hi + lo of FP32 numbers (about 48 significant bits).  FP32
-// runs at ~70x the FP64 rate on this GPU, so a refinement sweep whose only
-// job is to bring the error down to the level the final FP64 sweep removes
-// can use it.  Products use the FMA error-free transformation
-// (p = a*b, e = fma(a, b, -p)), sums the two-sum of the leading parts.
-
-// Exact split of an FP64 value into hi (first 24 significant bits, truncated)
-// and lo (the next 24, rounded) with integer operations only.  |x| < 2^-126
-// gives (0, 0); 2^-126 <= |x| < 2^-74 gives lo = 0.
-__device__ __forceinline__ void f64_to_df(double x, float& hi, float& lo) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned int sign = (unsigned int)(b >> 63) << 31;
-  const int e = (int)((b >> 52) & 0x7FF) - 1023;
-  if (e < -126) { hi = 0.f; lo = 0.f; return; }
-  const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  hi = __uint_as_float(sign | ((unsigned int)(e + 127) << 23) | (unsigned int)(m >> 29));
-  if (e < -74) { lo = 0.f; return; }
-  const unsigned int rem = (unsigned int)(m & 0x1FFFFFFFull);  // value rem * 2^(e-52)
-  const float scale = __uint_as_float((unsigned int)(e - 52 + 127) << 23);
-  lo = __uint_as_float(__float_as_uint(__uint2float_rn(rem) * scale) | sign);
-}
-
-// (ah, al) -= (ch + cl [+ cl2]) * (uh + ul), dropping cl*ul and cl2*ul; the
-// third coefficient term cl2 enters only when EXACT (else the 48-bit ch + cl).
-// LO0: ul is zero (the solution right after the first solve), and the ch*ul
-// term, exactly 0 there, is not formed (the same result).
-template <bool EXACT = false, bool LO0 = false>
-__device__ __forceinline__ void df_sub_prod(float& ah, float& al, float ch, float cl, float uh, float ul,
-                                            float cl2 = 0.f) {
-  const float p = ch * uh;
-  const float e = fmaf(ch, uh, -p);
-  const float t0 = fmaf(cl, uh, EXACT ? fmaf(cl2, uh, e) : e);
-  const float t = LO0 ? t0 : fmaf(ch, ul, t0);
-  const float s = ah - p;
-  const float bb = s - ah;
-  const float err = (ah - (s - bb)) - (p + bb);
-  ah = s;
-  al = al + (err - t);
-}
-
-struct DfArgs {
-  const float* uh;
-  const float* ul;
-  const double* f;
-  __nv_bfloat16* hi;
-  __nv_bfloat16* lo;
-  float* out32;        // if set: FP32 residual at pitch Px, max |r| -> st slot 0
-  F16State* st;
-  const float *Hxh, *Hxl, *Hyh, *Hyl, *Hzh, *Hzl;
-  const float *Hxl2, *Hyl2, *Hzl2;  // third coefficient terms (read when EXACT)
-  int nx, ny, nz, Px, nex;
-};
-
-template <int K, bool EXACT>
-__global__ void __launch_bounds__(256) stencil_df_kernel(DfArgs a) {
-  constexpr int BW = 2 * K + 1;
-  const long long lines = (long long)a.ny * a.nz;
-  const long long total = (long long)a.nex * lines;
-  float rmax = 0.f;  // FP32 output: max |r| of this thread's nodes
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int ex = (int)(t % a.nex);
-    const long long jl = t / a.nex;
-    const int j = (int)(jl % a.ny), l = (int)(jl / a.ny);
-    const long long line = jl * a.nx;    // f (pitch nx)
-    const long long uline = jl * a.Px;   // u (pitch Px)
-    const int i0 = ex * K - 1;
-    float wh[BW], wl[BW];
-#pragma unroll
-    for (int d = 0; d < BW; ++d) {
-      const int i = i0 - K + d;
-      const bool ok = i >= 0 && i < a.nx;
-      wh[d] = ok ? __ldg(a.uh + uline + i) : 0.f;
-      wl[d] = ok ? __ldg(a.ul + uline + i) : 0.f;
-    }
-    float ah[K], al[K];
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-      const int i = i0 + q;
-      if (i >= 0) f64_to_df(__ldg(a.f + line + i), ah[q], al[q]);
-      else { ah[q] = 0.f; al[q] = 0.f; }
-    }
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-      const int dlo = (q == 0) ? -K : -q, dhi = (q == 0) ? K : K - q;
-#pragma unroll
-      for (int d = dlo; d <= dhi; ++d)
-        df_sub_prod<EXACT>(ah[q], al[q], __ldg(a.Hxh + q * BW + d + K), __ldg(a.Hxl + q * BW + d + K), wh[K + q + d],
-                    wl[K + q + d], EXACT ? __ldg(a.Hxl2 + q * BW + d + K) : 0.f);
-    }
-    {
-      const int qy = (j + 1) % K;
-      const int dlo = (qy == 0) ? -K : -qy, dhi = (qy == 0) ? K : K - qy;
-      for (int d = dlo; d <= dhi; ++d) {
-        const int jj = j + d;
-        if (jj < 0 || jj >= a.ny) continue;
-        const float ch = __ldg(a.Hyh + qy * BW + d + K), cl = __ldg(a.Hyl + qy * BW + d + K);
-        const float cl2 = EXACT ? __ldg(a.Hyl2 + qy * BW + d + K) : 0.f;
-        const long long off = ((long long)l * a.ny + jj) * a.Px;
-#pragma unroll
-        for (int q = 0; q < K; ++q) {
-          const int i = i0 + q;
-          if (i < 0) continue;
-          df_sub_prod<EXACT>(ah[q], al[q], ch, cl, __ldg(a.uh + off + i), __ldg(a.ul + off + i), cl2);
-        }
-      }
-    }
-    {
-      const int qz = (l + 1) % K;
-      const int dlo = (qz == 0) ? -K : -qz, dhi = (qz == 0) ? K : K - qz;
-      for (int d = dlo; d <= dhi; ++d) {
-        const int ll = l + d;
-        if (ll < 0 || ll >= a.nz) continue;
-        const float ch = __ldg(a.Hzh + qz * BW + d + K), cl = __ldg(a.Hzl + qz * BW + d + K);
-        const float cl2 = EXACT ? __ldg(a.Hzl2 + qz * BW + d + K) : 0.f;
-        const long long off = ((long long)ll * a.ny + j) * a.Px;
-#pragma unroll
-        for (int q = 0; q < K; ++q) {
-          const int i = i0 + q;
-          if (i < 0) continue;
-          df_sub_prod<EXACT>(ah[q], al[q], ch, cl, __ldg(a.uh + off + i), __ldg(a.ul + off + i), cl2);
-        }
-      }
-    }
-    if (a.out32) {
-#pragma unroll
-      for (int q = 0; q < K; ++q) {
-        const int i = i0 + q;
-        if (i < 0) continue;
-        const float rf = ah[q] + al[q];
-        a.out32[(long long)i + (long long)a.Px * jl] = rf;
-        rmax = fmaxf(rmax, fabsf(rf));
-      }
-      continue;
-    }
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-      const int i = i0 + q;
-      if (i < 0) continue;
-      const float rf = ah[q] + al[q];
-      const __nv_bfloat16 h16 = __float2bfloat16_rn(rf);
-      const __nv_bfloat16 l16 = __float2bfloat16_rn(rf - __bfloat162float(h16));
-      const long long o = (long long)i + (long long)a.Px * jl;
-      a.hi[o] = h16;
-      a.lo[o] = l16;
-    }
-  }
-  if (a.out32 && a.st) {  // every lane of the warp gets here (after the loop)
-    rmax = warp_max(rmax);
-    if ((threadIdx.x & 31) == 0 && rmax > 0.f) atomicMax(&a.st->maxbits[0], __float_as_uint(rmax));
-  }
-}
-
-// Rows of H per local index for the vector residual (k <= 4), as kernel
-// parameters: the x rows are read at compile-time offsets (no load
-// instructions), the y and z rows at warp-uniform offsets.
-struct DfCoef {
-  float h[3][4 * 9];
-  float l[3][4 * 9];
-  float l2[3][4 * 9];  // third terms (used when EXACT)
-};
-
-// Double-FP32 residual for k in {1, 2, 4}.  A lane handles the 4 consecutive
-// nodes i = 4c .. 4c+3 of one (j, l) line -- one float4 of each of u_hi and
-// u_lo, whose rows (pitch Px, a multiple of 16) are 16-byte aligned and whose
-// pad columns are zero -- and a warp handles one line, its lanes striding over
-// the line's Px/4 chunks.  Since 4 % k == 0, node 4c+p has the local index
-// (p+1) % k for every c: each position's x row of H is known at compile time
-// and only its band is summed.  The y and z rows depend on the warp's (j, l).
-template <int K, bool EXACT, bool LO0>
-__global__ void __launch_bounds__(256, 4) stencil_df4_kernel(DfArgs a, const __grid_constant__ DfCoef cf) {
-  constexpr int BW = 2 * K + 1;
-  const int lane = threadIdx.x & 31;
-  const long long lines = (long long)a.ny * a.nz;
-  const int chunks = a.Px >> 2;
-  const long long splane = (long long)a.ny * chunks;  // float4 per z-plane
-  const float4* UH = reinterpret_cast<const float4*>(a.uh);
-  const float4* UL = reinterpret_cast<const float4*>(a.ul);
-  float rmax = 0.f;
-  for (long long line = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); line < lines;
-       line += (long long)gridDim.x * 8) {  // warp-uniform
-    const int j = (int)(line % a.ny), l = (int)(line / a.ny);
-    const int qy = (j + 1) % K, qz = (l + 1) % K;
-    const int ylo = (qy == 0) ? -K : -qy, yhi = (qy == 0) ? K : K - qy;
-    const int zlo = (qz == 0) ? -K : -qz, zhi = (qz == 0) ? K : K - qz;
-    const long long row4 = line * chunks;
-    const double* frow = a.f + line * a.nx;
-    for (int c = lane; c < chunks; c += 32) {
-      const int i0 = 4 * c;
-      float ah[4], al[4];
-#pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        if (i0 + p < a.nx) f64_to_df(__ldg(frow + i0 + p), ah[p], al[p]);
-        else { ah[p] = 0.f; al[p] = 0.f; }
-      }
-      // x: nodes i0-4 .. i0+7 (the neighbouring chunks; zero outside the line)
-      float wh[12], wl[12];
-      {
-        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 ph = c > 0 ? __ldg(UH + row4 + c - 1) : z4, pl = (c > 0 && !LO0) ? __ldg(UL + row4 + c - 1) : z4;
-        const float4 ch = __ldg(UH + row4 + c), cl = LO0 ? z4 : __ldg(UL + row4 + c);
-        const float4 nh = c + 1 < chunks ? __ldg(UH + row4 + c + 1) : z4;
-        const float4 nl = (c + 1 < chunks && !LO0) ? __ldg(UL + row4 + c + 1) : z4;
-        wh[0] = ph.x; wh[1] = ph.y; wh[2] = ph.z; wh[3] = ph.w; wh[4] = ch.x; wh[5] = ch.y;
-        wh[6] = ch.z; wh[7] = ch.w; wh[8] = nh.x; wh[9] = nh.y; wh[10] = nh.z; wh[11] = nh.w;
-        wl[0] = pl.x; wl[1] = pl.y; wl[2] = pl.z; wl[3] = pl.w; wl[4] = cl.x; wl[5] = cl.y;
-        wl[6] = cl.z; wl[7] = cl.w; wl[8] = nl.x; wl[9] = nl.y; wl[10] = nl.z; wl[11] = nl.w;
-      }
-#pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        const int q = (p + 1) % K;
-        const int dlo = (q == 0) ? -K : -q, dhi = (q == 0) ? K : K - q;
-#pragma unroll
-        for (int d = -K; d <= K; ++d)
-          if (d >= dlo && d <= dhi)  // compile-time after unrolling
-            df_sub_prod<EXACT, LO0>(ah[p], al[p], cf.h[0][q * BW + d + K], cf.l[0][q * BW + d + K], wh[4 + p + d], wl[4 + p + d],
-                        EXACT ? cf.l2[0][q * BW + d + K] : 0.f);
-      }
-      // y and z: the rows of the neighbouring lines, one float4 pair per row
-#pragma unroll
-      for (int d = -K; d <= K; ++d) {
-        if (d < ylo || d > yhi || j + d < 0 || j + d >= a.ny) continue;  // warp-uniform
-        const float chh = cf.h[1][qy * BW + d + K], cll = cf.l[1][qy * BW + d + K];
-        const float cl2 = EXACT ? cf.l2[1][qy * BW + d + K] : 0.f;
-        const float4 vh = __ldg(UH + row4 + (long long)d * chunks + c);
-        const float4 vl = LO0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(UL + row4 + (long long)d * chunks + c);
-        df_sub_prod<EXACT, LO0>(ah[0], al[0], chh, cll, vh.x, vl.x, cl2);
-        df_sub_prod<EXACT, LO0>(ah[1], al[1], chh, cll, vh.y, vl.y, cl2);
-        df_sub_prod<EXACT, LO0>(ah[2], al[2], chh, cll, vh.z, vl.z, cl2);
-        df_sub_prod<EXACT, LO0>(ah[3], al[3], chh, cll, vh.w, vl.w, cl2);
-      }
-#pragma unroll
-      for (int d = -K; d <= K; ++d) {
-        if (d < zlo || d > zhi || l + d < 0 || l + d >= a.nz) continue;  // warp-uniform
-        const float chh = cf.h[2][qz * BW + d + K], cll = cf.l[2][qz * BW + d + K];
-        const float cl2 = EXACT ? cf.l2[2][qz * BW + d + K] : 0.f;
-        const float4 vh = __ldg(UH + row4 + (long long)d * splane + c);
-        const float4 vl = LO0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(UL + row4 + (long long)d * splane + c);
-        df_sub_prod<EXACT, LO0>(ah[0], al[0], chh, cll, vh.x, vl.x, cl2);
-        df_sub_prod<EXACT, LO0>(ah[1], al[1], chh, cll, vh.y, vl.y, cl2);
-        df_sub_prod<EXACT, LO0>(ah[2], al[2], chh, cll, vh.z, vl.z, cl2);
-        df_sub_prod<EXACT, LO0>(ah[3], al[3], chh, cll, vh.w, vl.w, cl2);
-      }
-      float r[4];
-#pragma unroll
-      for (int p = 0; p < 4; ++p) r[p] = (i0 + p < a.nx) ? ah[p] + al[p] : 0.f;  // pads stay zero
-      const long long o = line * a.Px + i0;
-      if (a.out32) {
-        *reinterpret_cast<float4*>(a.out32 + o) = make_float4(r[0], r[1], r[2], r[3]);
-#pragma unroll
-        for (int p = 0; p < 4; ++p) rmax = fmaxf(rmax, fabsf(r[p]));
-      } else {
-        uint32_t hw[2], lw[2];
-#pragma unroll
-        for (int p = 0; p < 4; p += 2) {
-          const __nv_bfloat16 h0 = __float2bfloat16_rn(r[p]), h1 = __float2bfloat16_rn(r[p + 1]);
-          const __nv_bfloat16 l0 = __float2bfloat16_rn(r[p] - __bfloat162float(h0));
-          const __nv_bfloat16 l1 = __float2bfloat16_rn(r[p + 1] - __bfloat162float(h1));
-          hw[p / 2] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-          lw[p / 2] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-        }
-        *reinterpret_cast<uint2*>(a.hi + o) = make_uint2(hw[0], hw[1]);
-        *reinterpret_cast<uint2*>(a.lo + o) = make_uint2(lw[0], lw[1]);
-      }
-    }
-  }
-  if (a.out32 && a.st) {  // every lane of the warp gets here
-    rmax = warp_max(rmax);
-    if ((threadIdx.x & 31) == 0 && rmax > 0.f) atomicMax(&a.st->maxbits[0], __float_as_uint(rmax));
-  }
-}
-
-template <int K>
-cudaError_t launch_df4(const DfArgs& a, const DevAxis* ax, bool exact, bool lo_zero, cudaStream_t s) {
-  DfCoef cf{};
-  for (int w = 0; w < 3; ++w)
-    for (int e = 0; e < K * (2 * K + 1); ++e) {
-      cf.h[w][e] = ax[w].Hq_hi_host[e];
-      cf.l[w][e] = ax[w].Hq_lo_host[e];
-      cf.l2[w][e] = ax[w].Hq_lo2_host[e];
-    }
-  // One block per 8 consecutive lines and no grid stride: the resident blocks
-  // then sweep the grid plane by plane, so the rows 1..K planes away that a
-  // warp reads were read moments earlier by other warps and are still in L2.
-  const long long lines = (long long)a.ny * a.nz;
-  long long blocks = (lines + 7) / 8;
-  if (blocks > 0x7FFFFFFFLL) blocks = 0x7FFFFFFFLL;
-  const unsigned g = (unsigned)(blocks < 1 ? 1 : blocks);
-  if (exact) {
-    if (lo_zero) stencil_df4_kernel<K, true, true><<<g, 256, 0, s>>>(a, cf);
-    else stencil_df4_kernel<K, true, false><<<g, 256, 0, s>>>(a, cf);
-  } else {
-    if (lo_zero) stencil_df4_kernel<K, false, true><<<g, 256, 0, s>>>(a, cf);
-    else stencil_df4_kernel<K, false, false><<<g, 256, 0, s>>>(a, cf);
-  }
-  return cudaGetLastError();
-}
-
-template <int K>
-cudaError_t launch_df(const DfArgs& a, bool exact, cudaStream_t s) {
-  const long long total = (long long)a.nex * a.ny * a.nz;
-  long long b = (total + 255) / 256;
-  if (b > 0x7FFFFFFFLL) b = 0x7FFFFFFFLL;  // one thread per work item (see launch_elem)
-  if (exact) stencil_df_kernel<K, true><<<(int)(b < 1 ? 1 : b), 256, 0, s>>>(a);
-  else stencil_df_kernel<K, false><<<(int)(b < 1 ? 1 : b), 256, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
 // Zero the pad columns i in [nx, Px) of a split array (the stencil writes
 // only i < nx).
 __global__ void zero_pads_kernel(__nv_bfloat16* hi, __nv_bfloat16* lo, int nx, int Px, long long lines) {
@@ -841,37 +530,6 @@ cudaError_t launch_stencil(const Geom& g, int k, const DevAxis* ax, const double
   a.out64 = out64; a.hi = out_hi; a.lo = out_lo;
   const cudaError_t e = launch_stencil_any(a, g, ax, s);
   if (e != cudaSuccess || mode != 2 || g.Px == g.nx) return e;
-  const long long lines = (long long)g.ny * g.nz;
-  zero_pads_kernel<<<grid_for(lines * (g.Px - g.nx), 256), 256, 0, s>>>(out_hi, out_lo, g.nx, g.Px, lines);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_stencil_df(const Geom& g, int k, const DevAxis* ax, DfBuffers u, const double* f,
-                              __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, cudaStream_t s, float* out32,
-                              F16State* st, bool exact_coef, bool lo_zero) {
-  if (g.bc != 0) return cudaErrorInvalidValue;  // element-pattern rows (Dirichlet) only
-  DfArgs a{};
-  a.uh = u.hi; a.ul = u.lo; a.f = f; a.hi = out_hi; a.lo = out_lo;
-  a.out32 = out32; a.st = st;
-  a.Hxh = ax[0].Hq_hi; a.Hxl = ax[0].Hq_lo;
-  a.Hyh = ax[1].Hq_hi; a.Hyl = ax[1].Hq_lo;
-  a.Hzh = ax[2].Hq_hi; a.Hzl = ax[2].Hq_lo;
-  if (exact_coef) { a.Hxl2 = ax[0].Hq_lo2; a.Hyl2 = ax[1].Hq_lo2; a.Hzl2 = ax[2].Hq_lo2; }
-  a.nx = g.nx; a.ny = g.ny; a.nz = g.nz; a.Px = g.Px;
-  a.nex = (g.nx + 1) / k;
-  cudaError_t e;
-  switch (k) {
-    case 1: return launch_df4<1>(a, ax, exact_coef, lo_zero, s);  // pads written as zeros
-    case 2: return launch_df4<2>(a, ax, exact_coef, lo_zero, s);
-    case 4: return launch_df4<4>(a, ax, exact_coef, lo_zero, s);
-    case 3: e = launch_df<3>(a, exact_coef, s); break;
-    case 5: e = launch_df<5>(a, exact_coef, s); break;
-    case 6: e = launch_df<6>(a, exact_coef, s); break;
-    case 7: e = launch_df<7>(a, exact_coef, s); break;
-    case 8: e = launch_df<8>(a, exact_coef, s); break;
-    default: return cudaErrorInvalidValue;
-  }
-  if (e != cudaSuccess || g.Px == g.nx || out32) return e;
   const long long lines = (long long)g.ny * g.nz;
   zero_pads_kernel<<<grid_for(lines * (g.Px - g.nx), 256), 256, 0, s>>>(out_hi, out_lo, g.nx, g.Px, lines);
   return cudaGetLastError();

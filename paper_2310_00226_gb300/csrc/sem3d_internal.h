@@ -131,12 +131,10 @@ struct DevAxis {
   float* lamf = nullptr;        // FP32 copy for the low-precision epilogues
   double* Hband = nullptr;      // FP64 n x (2k+1)
   double* Hq = nullptr;         // FP64 k x (2k+1) per-local-index rows of H (x axis: + c on the diagonal)
-  float* Hq_hi = nullptr;       // the same table as FP32 terms: Hq = Hq_hi + Hq_lo (48 bits) + Hq_lo2 (exact)
-  float* Hq_lo = nullptr;
-  float* Hq_lo2 = nullptr;
-  float Hq_hi_host[4 * 9] = {}; // host copies for k <= 4 (kernel parameters of the vector residual)
-  float Hq_lo_host[4 * 9] = {};
-  float Hq_lo2_host[4 * 9] = {};
+  // the same table on the host as FP32 terms, for k <= 8: hi + lo (48 bits) + lo2 (exact)
+  float Hq_hi_host[8 * 17] = {};
+  float Hq_lo_host[8 * 17] = {};
+  float Hq_lo2_host[8 * 17] = {};
   int* band_lo = nullptr;
   int* band_hi = nullptr;
   float* Wf[2] = {nullptr, nullptr};            // FP32 copies: [0] = T^{-1}, [1] = T; n x n row-major
@@ -245,6 +243,7 @@ cudaError_t launch_mode_product_f32_grouped(int count, const Geom* geoms, int ax
 // r  = same, written as bf16 hi/lo at pitch Px   (mode 2)
 cudaError_t launch_stencil(const Geom& g, int k, const DevAxis* ax, const double* u, const double* f, double* out64,
                            __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, int mode, cudaStream_t s);
+// ---- double-FP32 residual (df_kernels.cu)
 // r = f - (c + H_x (+) H_y (+) H_z) u in double-FP32 arithmetic (about 48
 // significant bits), u given as a double-FP32 pair (pitch Px, zero pads), f as
 // FP64 (pitch nx); r written as bf16 hi/lo at pitch Px with zero pads, or as
@@ -253,12 +252,11 @@ cudaError_t launch_stencil(const Geom& g, int k, const DevAxis* ax, const double
 // (48 bits); with exact_coef also the third term lo2, which makes them exact:
 // a 48-bit operator is a different operator, whose solution a refinement with
 // only these residuals would converge to (off by ~kappa * 2^-48).
-// lo_zero: u's low parts are all zero (right after the first solve); the
-// vector kernel (k in {1, 2, 4}) then skips them (the same result).
+// lo_zero: u's low parts are all zero (right after the first solve) and are not
+// read (the same result).  The pads of the output are written too.
 cudaError_t launch_stencil_df(const Geom& g, int k, const DevAxis* ax, DfBuffers u, const double* f,
-                              __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, cudaStream_t s,
-                              float* out32 = nullptr, F16State* st = nullptr, bool exact_coef = false,
-                              bool lo_zero = false);
+                              __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, int num_sms, cudaStream_t s, float* out32,
+                              F16State* st, bool exact_coef, bool lo_zero);
 // FP64 residual written as FP32 at pitch Px; with st, its max |r| goes to
 // state slot 0 (the F16X3 tier then splits it with launch_split_f16).
 cudaError_t launch_stencil_f32out(const Geom& g, int k, const DevAxis* ax, const double* u, const double* f,
