@@ -163,6 +163,7 @@ sem3d_status setup_axis(sem3d_plan* p, int a, const DevAxis* same, double* scrat
     for (int w = 0; w < 2; ++w) {
       s.add(&D.par[w], A.par[w].size(), A.par[w].data());
       s.add(&D.Wf[w], nn);
+      s.add(&D.Wpf[w], A.par[w].size());
       s.add(&D.Wt32[w], nk);
       s.add(&D.W16_hi[w], nk);
       s.add(&D.W16_lo[w], nk);
@@ -298,20 +299,23 @@ sem3d_status solve_once_f64(sem3d_plan* p, const double* in, double* out, bool a
 }
 
 // ---- FP32 path: FP64 in -> FP64 out (store or accumulate), FP32 ping-pong.
+// By parity blocks in solves of two sweeps or more (see fp32_kernels.cu).
+bool f32_parity(const sem3d_plan* h) { return h->sweeps >= 2; }
+
 sem3d_status solve_once_f32(sem3d_plan* p, const double* in, double* out, bool accumulate, cudaStream_t s) {
   const size_t N = (size_t)p->g.nx * p->g.ny * p->g.nz;
   float* A = static_cast<float*>(p->ws);
   float* B = reinterpret_cast<float*>(static_cast<char*>(p->ws) + align256(N * sizeof(float)));
   const Geom& g = p->g;
   const DevAxis* d = p->dev;
-  const double *lx = d[0].lam, *ly = d[1].lam, *lz = d[2].lam;
-  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 2, d[2].Wf[0], in, true, A, false, EPI_STORE, lx, ly, lz, s));
-  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 1, d[1].Wf[0], A, false, B, false, EPI_STORE, lx, ly, lz, s));
-  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 0, d[0].Wf[0], B, false, A, false, EPI_DIV, lx, ly, lz, s));
-  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 0, d[0].Wf[1], A, false, B, false, EPI_STORE, lx, ly, lz, s));
-  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 1, d[1].Wf[1], B, false, A, false, EPI_STORE, lx, ly, lz, s));
-  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 2, d[2].Wf[1], A, false, out, true,
-                                                 accumulate ? EPI_ACCUM : EPI_STORE, lx, ly, lz, s));
+  const bool par = f32_parity(p);
+  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 2, d, 0, par, in, true, A, false, EPI_STORE, s));
+  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 1, d, 0, par, A, false, B, false, EPI_STORE, s));
+  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 0, d, 0, par, B, false, A, false, EPI_DIV, s));
+  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 0, d, 1, par, A, false, B, false, EPI_STORE, s));
+  LAUNCH(p, K_F32, 1, s, launch_mode_product_f32(g, 1, d, 1, par, B, false, A, false, EPI_STORE, s));
+  LAUNCH(p, K_F32, 1, s,
+         launch_mode_product_f32(g, 2, d, 1, par, A, false, out, true, accumulate ? EPI_ACCUM : EPI_STORE, s));
   return SEM3D_OK;
 }
 
@@ -1129,18 +1133,17 @@ sem3d_status ch_step_core(sem3d_plan* h, const double* phi_n, const double* phi_
     float* A = reinterpret_cast<float*>(w);
     float* B = reinterpret_cast<float*>(w + align256(N * sizeof(float)));
     float* C = reinterpret_cast<float*>(w + 2 * align256(N * sizeof(float)));
-    const double *lx = d[0].lam, *ly = d[1].lam, *lz = d[2].lam;
     LAUNCH(h, K_STENCIL, 1, s, launch_ch_prep(SEM3D_FP32, g, phi_n, phi_nm1, A, B, nb, nb, c, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 2, d[2].Wf[0], A, false, C, false, EPI_STORE, lx, ly, lz, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 1, d[1].Wf[0], C, false, A, false, EPI_STORE, lx, ly, lz, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 0, d[0].Wf[0], A, false, C, false, EPI_STORE, lx, ly, lz, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 2, d[2].Wf[0], B, false, A, false, EPI_STORE, lx, ly, lz, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 1, d[1].Wf[0], A, false, B, false, EPI_STORE, lx, ly, lz, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 0, d[0].Wf[0], B, false, A, false, EPI_STORE, lx, ly, lz, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 2, d, 0, false, A, false, C, false, EPI_STORE, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 1, d, 0, false, C, false, A, false, EPI_STORE, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 0, d, 0, false, A, false, C, false, EPI_STORE, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 2, d, 0, false, B, false, A, false, EPI_STORE, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 1, d, 0, false, A, false, B, false, EPI_STORE, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 0, d, 0, false, B, false, A, false, EPI_STORE, s));
     LAUNCH(h, K_STENCIL, 1, s, launch_ch_combine(SEM3D_FP32, g, d, C, A, B, nb, nb, nb, c, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 0, d[0].Wf[1], B, false, A, false, EPI_STORE, lx, ly, lz, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 1, d[1].Wf[1], A, false, C, false, EPI_STORE, lx, ly, lz, s));
-    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 2, d[2].Wf[1], C, false, phi_np1, true, EPI_STORE, lx, ly, lz, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 0, d, 1, false, B, false, A, false, EPI_STORE, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 1, d, 1, false, A, false, C, false, EPI_STORE, s));
+    LAUNCH(h, K_F32, 1, s, launch_mode_product_f32(g, 2, d, 1, false, C, false, phi_np1, true, EPI_STORE, s));
   } else {
     const size_t Ns = align256((size_t)g.Px * g.ny * g.nz * sizeof(__nv_bfloat16));
     TcBuffers S0{reinterpret_cast<__nv_bfloat16*>(w), reinterpret_cast<__nv_bfloat16*>(w + Ns)};
@@ -1335,17 +1338,17 @@ sem3d_status batched_f32(int count, const sem3d_handle* hs, const double* const*
   if (st != SEM3D_OK) return st;
   StagingRelease release{s};
   std::vector<Geom> geo(count);
-  std::vector<const float*> W(count);
+  std::vector<const DevAxis*> ax(count);
   std::vector<const void*> in(count);
   std::vector<void*> out(count);
-  std::vector<const double*> lx(count), ly(count), lz(count);
+  const bool par = f32_parity(hs[0]);  // one sweep count for all
   std::vector<float*> A(count), B(count);
   std::vector<double*> R(count);
   for (int q = 0; q < count; ++q) {
     sem3d_plan* h = hs[q];
     const size_t N = (size_t)h->g.nx * h->g.ny * h->g.nz;
     geo[q] = h->g;
-    lx[q] = h->dev[0].lam; ly[q] = h->dev[1].lam; lz[q] = h->dev[2].lam;
+    ax[q] = h->dev;
     A[q] = static_cast<float*>(h->ws);
     B[q] = reinterpret_cast<float*>(static_cast<char*>(h->ws) + align256(N * sizeof(float)));
     R[q] = reinterpret_cast<double*>(static_cast<char*>(h->ws) + 2 * align256(N * sizeof(float)));
@@ -1353,7 +1356,6 @@ sem3d_status batched_f32(int count, const sem3d_handle* hs, const double* const*
   size_t stage = 0;
   auto pass = [&](int axis, int which, bool in64, bool out64, int epi, auto in_of, auto out_of) -> sem3d_status {
     for (int q = 0; q < count; ++q) {
-      W[q] = hs[q]->dev[axis].Wf[which];
       in[q] = in_of(q);
       out[q] = out_of(q);
     }
@@ -1361,8 +1363,8 @@ sem3d_status batched_f32(int count, const sem3d_handle* hs, const double* const*
     char* dt = static_cast<char*>(g_batch.dev_table) + stage * kStageTableBytes;
     ++stage;
     LAUNCH(hs[0], K_F32, 1, s,
-           launch_mode_product_f32_grouped(count, geo.data(), axis, W.data(), in.data(), in64, out.data(), out64, epi,
-                                           lx.data(), ly.data(), lz.data(), dt, kStageTableBytes, ht, s));
+           launch_mode_product_f32_grouped(count, geo.data(), axis, ax.data(), which, par, in.data(), in64, out.data(),
+                                           out64, epi, dt, kStageTableBytes, ht, s));
     return SEM3D_OK;
   };
   auto solve_group = [&](auto src, bool accumulate) -> sem3d_status {

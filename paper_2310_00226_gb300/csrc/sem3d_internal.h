@@ -137,6 +137,7 @@ struct DevAxis {
   float Hq_lo2_host[8 * 17] = {};
   int* band_lo = nullptr;
   int* band_hi = nullptr;
+  float* Wpf[2] = {nullptr, nullptr};           // FP32 parity blocks (as par)
   float* Wf[2] = {nullptr, nullptr};            // FP32 copies: [0] = T^{-1}, [1] = T; n x n row-major
   float* Wt32[2] = {nullptr, nullptr};          // TF32-rounded copies, n rows x Kp (TF32 tier)
   __nv_bfloat16* W_hi[2] = {nullptr, nullptr};  // [0] = T^{-1}, [1] = T; n rows x Kp
@@ -149,8 +150,8 @@ struct DevAxis {
   __nv_bfloat16* W_lo[2] = {nullptr, nullptr};
 };
 
-// Fill every low-precision copy of an axis's T^{-1} and T (Wf, Wt32, W16_*,
-// W_*, Wp_*) from their FP64 form on the device: w[0] = T^{-1}, w[1] = T (n x n
+// Fill every low-precision copy of an axis's T^{-1} and T (Wf, Wpf, Wt32,
+// W16_*, W_*, Wp_*) from their FP64 form on the device: w[0] = T^{-1}, w[1] = T (n x n
 // row-major), D.par as uploaded.  (setup_kernels.cu)
 cudaError_t launch_axis_copies(const DevAxis& D, const double* const w[2], cudaStream_t s);
 
@@ -219,11 +220,12 @@ FoldGeom fold_geom(const Geom& g);
 cudaError_t launch_mode_product_f64(const Geom& g, int axis, const DevAxis* ax, int which, const double* in,
                                     double* out, int epi, int num_sms, cudaStream_t s);
 // ---- FP32 CUDA-core kernels (fp32_kernels.cu)
-// One mode product in FP32 arithmetic; `in` is FP64 (first pass) or FP32,
-// `out` FP64 (last pass, EPI_STORE or EPI_ACCUM) or FP32.
-cudaError_t launch_mode_product_f32(const Geom& g, int axis, const float* W, const void* in, bool in_f64, void* out,
-                                    bool out_f64, int epi, const double* lamx, const double* lamy, const double* lamz,
-                                    cudaStream_t s);
+// One mode product in FP32 arithmetic with T^{-1} (which = 0) or T; `in` is
+// FP64 (first pass) or FP32, `out` FP64 (last pass, EPI_STORE or EPI_ACCUM) or
+// FP32; EPI_DIV in the x pass.  parity: by the parity blocks (modes, and the
+// eigenvalues of EPI_DIV, in mode order), else by the full matrices.
+cudaError_t launch_mode_product_f32(const Geom& g, int axis, const DevAxis* ax, int which, bool parity, const void* in,
+                                    bool in_f64, void* out, bool out_f64, int epi, cudaStream_t s);
 // Measure the FP32 kernel configurations on the three pass shapes of grid g
 // (once per shape per process; synchronous) and record the fastest; later
 // launches of those shapes use it.  f32_config reports the choice for an axis.
@@ -233,10 +235,9 @@ void f32_set_config(int axis, const Geom& g, int cfg);  // pin a configuration
 // The same pass for `count` independent problems in one grouped launch.
 // The per-problem descriptor table (count * ~160 B) is staged through
 // host_table (pinned, >= table_bytes) into dev_table with an async copy on s.
-cudaError_t launch_mode_product_f32_grouped(int count, const Geom* geoms, int axis, const float* const* W,
-                                            const void* const* in, bool in_f64, void* const* out, bool out_f64,
-                                            int epi, const double* const* lamx, const double* const* lamy,
-                                            const double* const* lamz, void* dev_table, size_t table_bytes,
+cudaError_t launch_mode_product_f32_grouped(int count, const Geom* geoms, int axis, const DevAxis* const* ax, int which,
+                                            bool parity, const void* const* in, bool in_f64, void* const* out,
+                                            bool out_f64, int epi, void* dev_table, size_t table_bytes,
                                             void* host_table, cudaStream_t s);
 // Au = c u + (H_x (+) H_y (+) H_z) u            (mode 0)
 // r  = f - c u - (H_x (+) H_y (+) H_z) u        (mode 1, FP64 r)

@@ -1,5 +1,5 @@
 // Low-precision copies of an axis's eigenbasis, made on the device at plan
-// set-up from the FP64 matrices (n^2 entries, nine arrays each).  Bound by the
+// set-up from the FP64 matrices (n^2 entries, ten arrays each).  Bound by the
 // FP64 upload.  A plan on axes already diagonalised, with the conversions on
 // the host and one allocation per array -> now: n = 63 1.1 -> 0.33 ms, 255
 // 10.0 -> 0.37 ms, 999 140 -> 0.6 ms; 449x320x383 19 -> 0.8 ms.
@@ -17,7 +17,7 @@ __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bflo
 struct AxisCopies {
   const double* w[2];    // T^{-1}, T
   const double* par[2];  // their parity blocks
-  float *f32[2], *t32[2];
+  float *f32[2], *pf32[2], *t32[2];
   __half *h16[2], *l16[2];
   __nv_bfloat16 *hi[2], *lo[2], *phi[2], *plo[2];
   double sc16[2];        // 2^eW16
@@ -49,8 +49,10 @@ __global__ void __launch_bounds__(256) axis_copies_kernel(AxisCopies a) {
     const long long r = odd ? e - even : e;
     const int p = odd ? po : pe, m = odd ? a.no : a.ne;
     const int o = (int)(r / p), t = (int)(r % p);
-    const double x = t < m ? a.par[q][(odd ? (long long)a.ne * a.ne : 0) + (long long)o * m + t] : 0.0;
-    split_bf16((float)x, a.phi[q][e], a.plo[q][e]);
+    const long long at = (odd ? (long long)a.ne * a.ne : 0) + (long long)o * m + t;
+    const float x = t < m ? (float)a.par[q][at] : 0.f;
+    if (t < m) a.pf32[q][at] = x;
+    split_bf16(x, a.phi[q][e], a.plo[q][e]);
   }
 }
 
@@ -62,7 +64,7 @@ cudaError_t launch_axis_copies(const DevAxis& D, const double* const w[2], cudaS
   for (int q = 0; q < 2; ++q) {
     a.w[q] = w[q];
     a.par[q] = D.par[q];
-    a.f32[q] = D.Wf[q]; a.t32[q] = D.Wt32[q];
+    a.f32[q] = D.Wf[q]; a.pf32[q] = D.Wpf[q]; a.t32[q] = D.Wt32[q];
     a.h16[q] = D.W16_hi[q]; a.l16[q] = D.W16_lo[q];
     a.hi[q] = D.W_hi[q]; a.lo[q] = D.W_lo[q];
     a.phi[q] = D.Wp_hi[q]; a.plo[q] = D.Wp_lo[q];

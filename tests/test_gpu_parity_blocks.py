@@ -49,6 +49,21 @@ def test_fp64_solve(n3, k, bc):
     check(n3, k, bc, "fp64", 1, lambda m, p, f, u: p.solve(f, u))
 
 
+# FP32 tier with two sweeps (by parity blocks): every tile configuration, which
+# is pinned per pass shape for the process, on grids of its own.
+FP32_GRIDS = [((1, 1, 2), 1), ((5, 8, 11), 3), ((31, 33, 32), 1), ((65, 127, 63), 2), ((129, 19, 255), 2)]
+
+
+@pytest.mark.parametrize("cfg", range(6))
+@pytest.mark.parametrize("n3,k", FP32_GRIDS)
+def test_fp32_refined_solve(n3, k, cfg):
+    def run(m, p, f, u):
+        for a in range(3):
+            p.set_tuned_config(a, cfg)
+        p.solve(f, u)
+    check(n3, k, "dirichlet", "fp32", 2, run)
+
+
 # Split-bf16 solves in parity order (all axes >= 255): even and odd n, pads in
 # either half of the x pitch, output tiles of 128 to 256, both boundary
 # conditions, k with and without the vector residuals, k > 8 and Neumann data
