@@ -24,7 +24,7 @@
 // formed on load; backward, the epilogue writes E + O and E - O to mirrored
 // nodes.  Bare solves, one sweep and the Cahn-Hilliard step keep the full
 // matrices.  Eight uneven problems (n = 63..255), 18 grouped passes: 8.2 ms
-// (scalar, full matrices, lanes along the outputs in every pass) -> @f32@.
+// (scalar, full matrices, lanes along the outputs in every pass) -> 4.3 ms.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -145,23 +145,20 @@ __device__ __forceinline__ void f32_tile(const F32Pass& p, long long bx, int by,
     const long long row = row0 + (KCONTIG ? e / BK : e % C::BM);
     abase[it] = row < rows ? in + row_offset(p, rows, row) : nullptr;
   }
-  float ra[LA][NP], rw[LW];
+  // Raw loads of the next chunk: converted, and added or subtracted, when they
+  // are stored, after the current chunk's multiply-adds.
+  TIN ra[LA][NP];
+  float rw[LW];
   auto load = [&](int t0) {
 #pragma unroll
     for (int it = 0; it < LA; ++it) {
       const int e = tid + it * 256;
       const int t = t0 + (KCONTIG ? e % BK : e / C::BM);
       const bool ok = abase[it] && t < kmax;
-      const float u = ok ? to_f32(abase[it][(long long)t * p.sm]) : 0.f;
-      if constexpr (MODE == W_FULL) {
-        ra[it][0] = u;
-      } else {
-        // the middle node of an odd n (t = no) has no partner
-        const bool pair = ok && t < p.no;
-        const float v = pair ? to_f32(abase[it][(long long)(MODE == W_FWD ? p.n - 1 - t : p.ne + t) * p.sm]) : 0.f;
-        ra[it][0] = MODE == W_FWD ? u + v : u;
-        ra[it][NP - 1] = MODE == W_FWD ? (pair ? u - v : 0.f) : v;
-      }
+      ra[it][0] = ok ? abase[it][(long long)t * p.sm] : TIN(0);
+      if constexpr (MODE != W_FULL)  // the middle node of an odd n (t = no) has no partner
+        ra[it][NP - 1] =
+            ok && t < p.no ? abase[it][(long long)(MODE == W_FWD ? p.n - 1 - t : p.ne + t) * p.sm] : TIN(0);
     }
 #pragma unroll
     for (int it = 0; it < LW; ++it) {
@@ -171,15 +168,24 @@ __device__ __forceinline__ void f32_tile(const F32Pass& p, long long bx, int by,
       rw[it] = (o < m && t < m) ? __ldg(p.W + (q == 0 ? 0 : (long long)p.ne * p.ne) + (long long)o * m + t) : 0.f;
     }
   };
-  auto store = [&](int st) {
+  auto store = [&](int st, int t0) {
     float* a = As + st * C::BK * C::A_LD;
     float* w = Ws + st * NP * BK * W_LD;
 #pragma unroll
     for (int it = 0; it < LA; ++it) {
       const int e = tid + it * 256;
       const int kk = KCONTIG ? e % BK : e / C::BM, r = KCONTIG ? e / BK : e % C::BM;
-#pragma unroll
-      for (int q = 0; q < NP; ++q) a[(q * BK + kk) * C::A_LD + r] = ra[it][q];
+      float u = to_f32(ra[it][0]);
+      if constexpr (MODE != W_FULL) {
+        float v = to_f32(ra[it][NP - 1]);
+        if (MODE == W_FWD) {
+          const float d = t0 + kk < p.no ? u - v : 0.f;
+          u = u + v;
+          v = d;
+        }
+        a[(BK + kk) * C::A_LD + r] = v;
+      }
+      a[kk * C::A_LD + r] = u;
     }
 #pragma unroll
     for (int it = 0; it < LW; ++it) {
@@ -216,7 +222,7 @@ __device__ __forceinline__ void f32_tile(const F32Pass& p, long long bx, int by,
 
   const int nch = (kmax + BK - 1) / BK;
   load(0);
-  store(0);
+  store(0, 0);
   __syncthreads();
   for (int ch = 0; ch < nch; ++ch) {
     if (C::STAGES == 2) {
@@ -225,72 +231,82 @@ __device__ __forceinline__ void f32_tile(const F32Pass& p, long long bx, int by,
       const int cur = ch & 1;
       if (ch + 1 < nch) load((ch + 1) * BK);
       compute(cur);
-      if (ch + 1 < nch) store(cur ^ 1);
+      if (ch + 1 < nch) store(cur ^ 1, (ch + 1) * BK);
       __syncthreads();
     } else {
       compute(0);
       __syncthreads();
       if (ch + 1 < nch) {
         load((ch + 1) * BK);
-        store(0);
+        store(0, (ch + 1) * BK);
         __syncthreads();
       }
     }
   }
   TOUT* out = static_cast<TOUT*>(p.out);
-  auto put = [&](long long base, int o, float v) {
-    TOUT* dst = out + base + (long long)o * p.sm;
-    if constexpr (sizeof(TOUT) == 8) {
-      if (p.epi == EPI_ACCUM) *dst += to_f64(v);
-      else *dst = to_f64(v);
-    } else {
-      *dst = v;
-    }
-  };
 #pragma unroll
   for (int g = 0; g < TG; ++g)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const long long row = row0 + 2 * ty + 2 * C::TY * g + h;
       if (row >= rows) continue;
-      const long long base = row_offset(p, rows, row);
+      TOUT* dst = out + row_offset(p, rows, row);
       double ly = 0.0, lz = 0.0;
       if (KCONTIG && p.epi == EPI_DIV) {  // x pass: row = (j, l)
-        ly = p.lamy[(int)(row % p.ny)];
-        lz = p.lamz[row / p.ny];
+        const unsigned int l = (unsigned int)row / (unsigned int)p.ny;  // R1 = ny nz is an int
+        ly = p.lamy[(unsigned int)row - l * (unsigned int)p.ny];
+        lz = p.lamz[l];
       }
+      // the row's values and where they go (at < 0: outside), then all reads of
+      // an accumulating pass before the first write
+      float v[NP][TN];
+      int at[NP][TN];
 #pragma unroll
       for (int c = 0; c < TN; ++c) {
         const int o = o0 + out_of(c);
-        float v[2];
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
           float x, y;
           unpack2(acc[q][g][c], x, y);
-          v[q] = h ? y : x;
+          v[q][c] = h ? y : x;
         }
         if constexpr (MODE == W_FULL) {
-          if (o >= p.n) continue;
-          if (KCONTIG && p.epi == EPI_DIV) v[0] = v[0] / (float)(p.lamx[o] + ly + lz + p.c);
-          put(base, o, v[0]);
-        } else if constexpr (MODE == W_FWD) {
-          if (o >= p.ne) continue;
-          if (KCONTIG && p.epi == EPI_DIV) {
-            const double d = ly + lz + p.c;
-            v[0] = v[0] / f64_to_f32_rn(p.lamx[o] + d);
-            if (o < p.no) v[1] = v[1] / f64_to_f32_rn(p.lamx[p.ne + o] + d);
-          }
-          put(base, o, v[0]);
-          if (o < p.no) put(base, p.ne + o, v[1]);
+          at[0][c] = o < p.n ? o : -1;
+          if (KCONTIG && p.epi == EPI_DIV && o < p.n) v[0][c] = v[0][c] / (float)(p.lamx[o] + ly + lz + p.c);
         } else {
-          if (o >= p.ne) continue;
-          if (o < p.no) {
-            put(base, o, v[0] + v[1]);
-            put(base, p.n - 1 - o, v[0] - v[1]);
-          } else {
-            put(base, o, v[0]);  // the middle of an odd n
+          const bool pair = o < p.no;  // else the middle of an odd n
+          at[0][c] = o < p.ne ? o : -1;
+          at[NP - 1][c] = !pair ? -1 : MODE == W_FWD ? p.ne + o : p.n - 1 - o;
+          if (MODE == W_BWD) {
+            const float e = v[0][c], d = pair ? v[NP - 1][c] : 0.f;
+            v[0][c] = e + d;
+            v[NP - 1][c] = e - d;
+          } else if (KCONTIG && p.epi == EPI_DIV) {
+            const double d = ly + lz + p.c;
+            if (o < p.ne) v[0][c] = v[0][c] / f64_to_f32_rn(p.lamx[o] + d);
+            if (pair) v[NP - 1][c] = v[NP - 1][c] / f64_to_f32_rn(p.lamx[p.ne + o] + d);
           }
         }
+      }
+      if constexpr (sizeof(TOUT) == 8) {
+        double old[NP][TN];
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+#pragma unroll
+          for (int c = 0; c < TN; ++c)
+            old[q][c] = p.epi == EPI_ACCUM && at[q][c] >= 0 ? dst[(long long)at[q][c] * p.sm] : 0.0;
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+#pragma unroll
+          for (int c = 0; c < TN; ++c)
+            if (at[q][c] >= 0)
+              dst[(long long)at[q][c] * p.sm] = p.epi == EPI_ACCUM ? old[q][c] + to_f64(v[q][c]) : to_f64(v[q][c]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+#pragma unroll
+          for (int c = 0; c < TN; ++c)
+            if (at[q][c] >= 0) dst[(long long)at[q][c] * p.sm] = v[q][c];
       }
     }
 }
@@ -352,8 +368,14 @@ cudaError_t launch_cfg(const F32Pass& p, bool kcontig, cudaStream_t s) {
   const long long bx = (rows + cfg_bm(CFG) - 1) / cfg_bm(CFG);
   if (bx >= (1LL << 31)) return cudaErrorInvalidValue;
   dim3 grid((unsigned)bx, (unsigned)out_tiles(p, CFG, MODE));
-  if (kcontig) mode_product_f32_kernel<CFG, TIN, TOUT, true, MODE><<<grid, 256, 0, s>>>(p);
-  else mode_product_f32_kernel<CFG, TIN, TOUT, false, MODE><<<grid, 256, 0, s>>>(p);
+  if constexpr (sizeof(TIN) + sizeof(TOUT) == 8) {
+    if (kcontig) {
+      mode_product_f32_kernel<CFG, TIN, TOUT, true, MODE><<<grid, 256, 0, s>>>(p);
+      return cudaGetLastError();
+    }
+  }
+  if (kcontig) return cudaErrorInvalidValue;  // FP64 operands: the z passes' only
+  mode_product_f32_kernel<CFG, TIN, TOUT, false, MODE><<<grid, 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -371,8 +393,14 @@ cudaError_t launch_f32(const F32Pass& p, bool kcontig, cudaStream_t s) {
 
 template <typename TIN, typename TOUT, int MODE>
 cudaError_t launch_f32_grouped(const F32Group& grp, long long blocks, bool kcontig, cudaStream_t s) {
-  if (kcontig) mode_product_f32_grouped_kernel<TIN, TOUT, true, MODE><<<(unsigned)blocks, 256, 0, s>>>(grp);
-  else mode_product_f32_grouped_kernel<TIN, TOUT, false, MODE><<<(unsigned)blocks, 256, 0, s>>>(grp);
+  if constexpr (sizeof(TIN) + sizeof(TOUT) == 8) {
+    if (kcontig) {
+      mode_product_f32_grouped_kernel<TIN, TOUT, true, MODE><<<(unsigned)blocks, 256, 0, s>>>(grp);
+      return cudaGetLastError();
+    }
+  }
+  if (kcontig) return cudaErrorInvalidValue;  // FP64 operands: the z passes' only
+  mode_product_f32_grouped_kernel<TIN, TOUT, false, MODE><<<(unsigned)blocks, 256, 0, s>>>(grp);
   return cudaGetLastError();
 }
 
