@@ -22,11 +22,6 @@ int ch_grid(long long n) {
   return (int)(b < 1 ? 1 : b);
 }
 
-// Grid of the line kernels: a block walks lines blockIdx.x, + gridDim.x, ...;
-// 16 blocks per SM (two waves of 8 resident), so that block launches are few
-// against the work (a line of Px elements is only 2-4 elements per thread).
-int line_grid(long long lines) { return (int)(lines < 152LL * 16 ? (lines < 1 ? 1 : lines) : 152LL * 16); }
-
 __device__ __forceinline__ void split2f(float v, __nv_bfloat16& h, __nv_bfloat16& l) {
   h = __float2bfloat16_rn(v);
   l = __float2bfloat16_rn(v - __bfloat162float(h));
@@ -44,28 +39,59 @@ __global__ void __launch_bounds__(CH_THREADS) ch_prep_kernel(const double* phi_n
   }
 }
 
-// Split-bf16 inputs (pitch Px, zero pads), FP32 arithmetic.  Blocks walk the
-// (j, l) lines, their threads along i.
-__global__ void __launch_bounds__(CH_THREADS) ch_prep_split_kernel(const double* phi_n, const double* phi_nm1,
+// Four values split into bf16 hi + lo, packed for one 8-byte store each.
+__device__ __forceinline__ void split4(const float (&v)[4], uint2& h, uint2& l) {
+  __nv_bfloat16 hh[4], ll[4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) split2f(v[p], hh[p], ll[p]);
+  auto pack = [](__nv_bfloat16 a, __nv_bfloat16 b) {
+    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+  };
+  h = make_uint2(pack(hh[0], hh[1]), pack(hh[2], hh[3]));
+  l = make_uint2(pack(ll[0], ll[1]), pack(ll[2], ll[3]));
+}
+
+// Split-bf16 inputs (pitch Px, zero pads), FP32 arithmetic.  Threads walk the
+// nodes in order, a thread takes 4 consecutive ones of a line: the bf16 arrays are then
+// written (and, below, read) 8 bytes at a time.  Bound by HBM (24 B per node);
+// n = 511, one node a thread and 2-byte stores -> this: 749 -> 463 us.
+__global__ void __launch_bounds__(CH_THREADS) ch_prep_split_kernel(const double* __restrict__ phi_n,
+                                                                   const double* __restrict__ phi_nm1,
                                                                    __nv_bfloat16* gh_hi, __nv_bfloat16* gh_lo,
                                                                    __nv_bfloat16* g_hi, __nv_bfloat16* g_lo, int nx,
                                                                    int Px, long long lines, ChParams c) {
   const float S = (float)c.S, inv_eps = (float)(1.0 / c.eps);
-  for (long long line = blockIdx.x; line < lines; line += gridDim.x) {
-    const double* pn_row = phi_n + line * nx;
-    const double* pm_row = phi_nm1 + line * nx;
-    const long long o = line * Px;
-    for (int i = threadIdx.x; i < Px; i += blockDim.x) {
-      float gh = 0.f, gg = 0.f;
-      if (i < nx) {
-        const float pn = f64_to_f32_rn(pn_row[i]), pm = f64_to_f32_rn(pm_row[i]);
-        const float bar = 2.f * pn - pm;
-        gh = 2.f * pn - 0.5f * pm;
-        gg = (bar * bar * bar - bar - S * bar) * inv_eps;
-      }
-      split2f(gh, gh_hi[o + i], gh_lo[o + i]);
-      split2f(gg, g_hi[o + i], g_lo[o + i]);
+  const int chunks = Px >> 2;
+  const long long total = lines * chunks;
+  for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < total;
+       w += (long long)gridDim.x * blockDim.x) {
+    const long long line = w / chunks;
+    const int i0 = (int)(w - line * chunks) * 4;
+    const double* pn_row = phi_n + line * nx + i0;
+    const double* pm_row = phi_nm1 + line * nx + i0;
+    double dn[4], dm[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      dn[p] = i0 + p < nx ? __ldg(pn_row + p) : 0.0;
+      dm[p] = i0 + p < nx ? __ldg(pm_row + p) : 0.0;
     }
+    float gh[4], gg[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {  // zero beyond the line, as its inputs are
+      const float pn = f64_to_f32_rn(dn[p]), pm = f64_to_f32_rn(dm[p]);
+      const float bar = 2.f * pn - pm;
+      gh[p] = 2.f * pn - 0.5f * pm;
+      gg[p] = (bar * bar * bar - bar - S * bar) * inv_eps;
+      if (i0 + p >= nx) gh[p] = gg[p] = 0.f;
+    }
+    const long long o = line * Px + i0;
+    uint2 h, l;
+    split4(gh, h, l);
+    *reinterpret_cast<uint2*>(gh_hi + o) = h;
+    *reinterpret_cast<uint2*>(gh_lo + o) = l;
+    split4(gg, h, l);
+    *reinterpret_cast<uint2*>(g_hi + o) = h;
+    *reinterpret_cast<uint2*>(g_lo + o) = l;
   }
 }
 
@@ -83,24 +109,45 @@ __global__ void __launch_bounds__(CH_THREADS) ch_combine_kernel(const T* a1, con
   }
 }
 
+// As ch_prep_split_kernel (12 B per node): n = 511 458 -> 283 us.
 __global__ void __launch_bounds__(CH_THREADS) ch_combine_split_kernel(
-    const __nv_bfloat16* a1h, const __nv_bfloat16* a1l, const __nv_bfloat16* a2h, const __nv_bfloat16* a2l,
-    __nv_bfloat16* oh, __nv_bfloat16* ol, const float* lx, const float* ly, const float* lz, int nx, int ny, int Px,
+    const __nv_bfloat16* __restrict__ a1h, const __nv_bfloat16* __restrict__ a1l,
+    const __nv_bfloat16* __restrict__ a2h, const __nv_bfloat16* __restrict__ a2l, __nv_bfloat16* oh, __nv_bfloat16* ol,
+    const float* __restrict__ lx, const float* __restrict__ ly, const float* __restrict__ lz, int nx, int ny, int Px,
     long long lines, ChParams c) {
   const float dtm = (float)(c.dt * c.m), eps = (float)c.eps, s_eps = (float)(c.S / c.eps);
-  for (long long line = blockIdx.x; line < lines; line += gridDim.x) {
-    const float lyz = ly[line % ny] + lz[line / ny];  // block-uniform
-    const long long o = line * Px;
-    for (int i = threadIdx.x; i < Px; i += blockDim.x) {
-      float v = 0.f;
-      if (i < nx) {
-        const float L = lx[i] + lyz;
-        const float x1 = __bfloat162float(a1h[o + i]) + __bfloat162float(a1l[o + i]);
-        const float x2 = __bfloat162float(a2h[o + i]) + __bfloat162float(a2l[o + i]);
-        v = (x1 - dtm * L * x2) / (1.5f + dtm * (eps * L * L + s_eps * L));
+  const int chunks = Px >> 2;
+  const long long total = lines * chunks;
+  auto ld4 = [](const __nv_bfloat16* p, float (&v)[4]) {
+    const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
+    v[0] = __uint_as_float(r.x << 16); v[1] = __uint_as_float(r.x & 0xFFFF0000u);
+    v[2] = __uint_as_float(r.y << 16); v[3] = __uint_as_float(r.y & 0xFFFF0000u);
+  };
+  for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < total;
+       w += (long long)gridDim.x * blockDim.x) {
+    const long long line = w / chunks;
+    const int i0 = (int)(w - line * chunks) * 4;
+    const float lyz = __ldg(ly + (int)(line % ny)) + __ldg(lz + (int)(line / ny));
+    const long long o = line * Px + i0;
+    float h1[4], l1[4], h2[4], l2[4], v[4];
+    ld4(a1h + o, h1);
+    ld4(a1l + o, l1);
+    ld4(a2h + o, h2);
+    ld4(a2l + o, l2);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      v[p] = 0.f;
+      if (i0 + p < nx) {
+        const float L = __ldg(lx + i0 + p) + lyz;
+        const float x1 = h1[p] + l1[p];
+        const float x2 = h2[p] + l2[p];
+        v[p] = (x1 - dtm * L * x2) / (1.5f + dtm * (eps * L * L + s_eps * L));
       }
-      split2f(v, oh[o + i], ol[o + i]);
     }
+    uint2 h, l;
+    split4(v, h, l);
+    *reinterpret_cast<uint2*>(oh + o) = h;
+    *reinterpret_cast<uint2*>(ol + o) = l;
   }
 }
 
@@ -117,7 +164,7 @@ cudaError_t launch_ch_prep(int tier, const Geom& g, const double* phi_n, const d
                                                               static_cast<float*>(gg), N, c);
   } else {
     const long long lines = (long long)g.ny * g.nz;
-    ch_prep_split_kernel<<<line_grid(lines), CH_THREADS, 0, s>>>(phi_n, phi_nm1, sh.hi, sh.lo, sg.hi, sg.lo, g.nx,
+    ch_prep_split_kernel<<<ch_grid(lines * (g.Px / 4)), CH_THREADS, 0, s>>>(phi_n, phi_nm1, sh.hi, sh.lo, sg.hi, sg.lo, g.nx,
                                                                   g.Px, lines, c);
   }
   return cudaGetLastError();
@@ -136,7 +183,7 @@ cudaError_t launch_ch_combine(int tier, const Geom& g, const DevAxis* ax, const 
         ax[1].lam, ax[2].lam, g.nx, g.ny, N, c);
   } else {
     const long long lines = (long long)g.ny * g.nz;
-    ch_combine_split_kernel<<<line_grid(lines), CH_THREADS, 0, s>>>(
+    ch_combine_split_kernel<<<ch_grid(lines * (g.Px / 4)), CH_THREADS, 0, s>>>(
         s1.hi, s1.lo, s2.hi, s2.lo, so.hi, so.lo, ax[0].lamf, ax[1].lamf, ax[2].lamf, g.nx, g.ny, g.Px, lines, c);
   }
   return cudaGetLastError();
