@@ -322,6 +322,8 @@ template <> struct CfgOf<5> { using T = Cfg5; };
 
 template <int CFG, typename TIN, typename TOUT, bool KCONTIG, int MODE>
 __global__ void __launch_bounds__(256, 2) mode_product_f32_kernel(F32Pass p) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ __align__(16) float smem[CfgOf<CFG>::T::SMEM_FLOATS];
   f32_tile<typename CfgOf<CFG>::T, TIN, TOUT, KCONTIG, MODE>(p, blockIdx.x, blockIdx.y, smem);
 }
@@ -369,14 +371,10 @@ cudaError_t launch_cfg(const F32Pass& p, bool kcontig, cudaStream_t s) {
   if (bx >= (1LL << 31)) return cudaErrorInvalidValue;
   dim3 grid((unsigned)bx, (unsigned)out_tiles(p, CFG, MODE));
   if constexpr (sizeof(TIN) + sizeof(TOUT) == 8) {
-    if (kcontig) {
-      mode_product_f32_kernel<CFG, TIN, TOUT, true, MODE><<<grid, 256, 0, s>>>(p);
-      return cudaGetLastError();
-    }
+    if (kcontig) return launch_pdl(mode_product_f32_kernel<CFG, TIN, TOUT, true, MODE>, grid, dim3(256), 0, s, p);
   }
   if (kcontig) return cudaErrorInvalidValue;  // FP64 operands: the z passes' only
-  mode_product_f32_kernel<CFG, TIN, TOUT, false, MODE><<<grid, 256, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(mode_product_f32_kernel<CFG, TIN, TOUT, false, MODE>, grid, dim3(256), 0, s, p);
 }
 
 template <typename TIN, typename TOUT, int MODE>

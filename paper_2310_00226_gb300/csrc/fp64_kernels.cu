@@ -53,6 +53,8 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
   const int o0 = blockIdx.y * F64_BN;
   const int wr = (warp & 1) * (BM / 2), wc = (warp >> 1) * 8;
 
+  // (no pdl_trigger: blocks set up early would share the SMs that idle in this
+  // pass, and with them one FP64 pipe, in their own: 63^3 315 -> 480 us)
   // The rows this thread loads are the same in every chunk.
   const double* abase[LA];
 #pragma unroll
@@ -106,6 +108,7 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
 #pragma unroll
     for (int b = 0; b < 2; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
 
+  pdl_wait();
   load(0);
   for (int t0 = 0; t0 < p.ne; t0 += F64_BK) {
     store();
@@ -181,10 +184,9 @@ cudaError_t launch_f64(const F64Pass& p, int num_sms, cudaStream_t s) {
   const long long bx = (rows + best - 1) / best;
   if (bx >= (1LL << 31)) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)bx, (unsigned)nt);
-  if (best == 64) mode_product_f64_kernel<KCONTIG, FWD, 64><<<grid, 256, 0, s>>>(p);
-  else if (best == 32) mode_product_f64_kernel<KCONTIG, FWD, 32><<<grid, 256, 0, s>>>(p);
-  else mode_product_f64_kernel<KCONTIG, FWD, 16><<<grid, 256, 0, s>>>(p);
-  return cudaGetLastError();
+  if (best == 64) return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, 64>, grid, dim3(256), 0, s, p);
+  if (best == 32) return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, 32>, grid, dim3(256), 0, s, p);
+  return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, 16>, grid, dim3(256), 0, s, p);
 }
 
 // ------------------------------------------------------------------ stencil

@@ -48,6 +48,39 @@ __device__ __forceinline__ float f64_to_f32_rn(double x) {
   return __uint_as_float(sign | (q + ((rem > half || (rem == half && (q & 1u))) ? 1u : 0u)));
 }
 
+// Programmatic dependent launch, used by the mode-product kernels: the next
+// kernel's blocks may be set up while this one's last blocks run (pdl_trigger),
+// and every thread executes pdl_wait before it first touches memory that
+// earlier kernels write: it returns when all earlier kernels of the stream are
+// complete and their writes visible.  So only launch latency and prologues
+// (barriers, tensor memory) overlap.  Kernels launched with launch_pdl's
+// attribute read what their predecessors wrote by TMA or ordinary loads, never
+// through the non-coherent path (__ldg, const __restrict__), which assumes data
+// that does not change while the kernel is resident.  A small solve is a chain
+// of short kernels: 63^3 refined 268 -> 204 us, FP64 315 -> 290.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+inline cudaLaunchAttribute pdl_attribute() {
+  cudaLaunchAttribute a;
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1] = {pdl_attribute()};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // Round an FP32 value to TF32 (10 explicit mantissa bits) to nearest, ties to
 // even, on the binary32 bit pattern; the result is an FP32 number whose 13 low
 // mantissa bits are zero.  Infinities and NaN pass through; finite values

@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(num_threads(MODE), 1)
   const int rank = (CL > 1) ? (int)cluster_ctarank() : 0;
   const int cid = blockIdx.x / CL, ncl = gridDim.x / CL;
 
+  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), CL); }
     for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), epi_warps(MODE)); }
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(num_threads(MODE), 1)
   tc_fence_before();
   __syncthreads();
   if (CL > 1) cluster_sync_all();  // peers' barriers are initialised before any multicast
+  pdl_wait();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
 
@@ -367,17 +369,18 @@ cudaError_t launch_tc(const CUtensorMap& a0, const CUtensorMap& a1, const CUtens
   }
   const long long clusters = work_clusters < max_clusters ? work_clusters : max_clusters;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CLUSTER;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1] = pdl_attribute();
   cfg.gridDim = dim3((unsigned)(clusters * CLUSTER));
   cfg.blockDim = dim3(num_threads(MODE));
   cfg.dynamicSmemBytes = smem_bytes(PASS);
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, a0, a1, b0, b1, a);
 }
 

@@ -112,6 +112,7 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
   const int rank = (int)cluster_ctarank();
   const int pid = blockIdx.x >> 1, npairs = gridDim.x >> 1;
 
+  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < P_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 2 * pair_epi(MODE)); }
@@ -127,6 +128,7 @@ __device__ __forceinline__ void pair_body(const Src& src, int* err, int stall) {
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers are initialised before any cross-CTA signal
+  pdl_wait();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
 
@@ -325,7 +327,7 @@ template <class Kern, class... Args>
 cudaError_t launch_pairs(Kern kern, std::atomic<int>& max_pairs_cache, int pass, int mode, long long work_pairs,
                          int num_sms, cudaStream_t s, const Args&... args) {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
@@ -349,6 +351,8 @@ cudaError_t launch_pairs(Kern kern, std::atomic<int>& max_pairs_cache, int pass,
   const long long pairs = work_pairs < max_pairs ? work_pairs : max_pairs;
   cfg.gridDim = dim3((unsigned)(2 * pairs));
   cfg.stream = s;
+  attr[1] = pdl_attribute();
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 

@@ -313,6 +313,7 @@ __global__ void __launch_bounds__(t_threads(MODE), 1)
   const int rank = (int)cluster_ctarank();
   const int pid = blockIdx.x >> 1, npairs = gridDim.x >> 1;
 
+  pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < TP_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 2 * t_epi_warps(MODE)); }
@@ -328,6 +329,7 @@ __global__ void __launch_bounds__(t_threads(MODE), 1)
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers are initialised before any cross-CTA signal
+  pdl_wait();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
 
@@ -498,7 +500,7 @@ cudaError_t launch_tf32_pair(const CUtensorMap& mA, const CUtensorMap& mB, const
   auto kern = mode_product_tf32_pair_kernel<MODE>;
   static std::atomic<int> max_pairs_cache{0};
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
@@ -522,6 +524,8 @@ cudaError_t launch_tf32_pair(const CUtensorMap& mA, const CUtensorMap& mB, const
   const long long pairs = work_pairs < max_pairs ? work_pairs : max_pairs;
   cfg.gridDim = dim3((unsigned)(2 * pairs));
   cfg.stream = s;
+  attr[1] = pdl_attribute();
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, mA, mB, a);
 }
 
