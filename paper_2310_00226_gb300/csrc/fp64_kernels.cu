@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(256) stencil_kernel(StencilArgs a) {
 }
 
 // Element-wise variant of the same operator for a uniform mesh and
-// 1 <= K <= 8.  Along x, one thread owns the K global nodes g = ex*K + q
+// 1 <= K <= 8, bound by the FP64 pipe.  Along x, one thread owns the K global nodes g = ex*K + q
 // (q = 0..K-1) of element ex: node q = 0 is the vertex shared with element
 // ex-1 (row of 2K+1 entries), q > 0 are the element's other nodes (K+1
 // entries each).  The thread keeps the 2K+1 node values of elements ex-1 and
@@ -275,34 +275,43 @@ __global__ void __launch_bounds__(256) stencil_kernel(StencilArgs a) {
 // y and z bands are uniform across a warp (its lanes share j and l).
 // Work per node: k+2 FMAs per axis on average (6 at k = 4), accumulated from
 // f in residual modes.
-template <int K, int MODE>
+// With Neumann data (NEU) every global node is an unknown, and a boundary row is
+// the vertex row applied to values mirrored at the boundary (its stiffness and
+// mass are half an inner vertex's, so its entries are twice the one-sided
+// ones: the same numbers, halved and doubled exactly).  The last node of a
+// line has an element of its own.  (321x161x241, k = 5: 679 us with a thread per
+// node and per-row band tables -> 477.)
+template <int K, int MODE, bool NEU>
 __global__ void __launch_bounds__(256) stencil_elem_kernel(StencilArgs a, const double* __restrict__ Hqx,
                                                            const double* __restrict__ Hqy,
                                                            const double* __restrict__ Hqz, int nex) {
-  constexpr int BW = 2 * K + 1;
+  constexpr int BW = 2 * K + 1, OFF = NEU ? 0 : 1;  // unknown index = global node - OFF
   const long long lines = (long long)a.ny * a.nz;
   const long long total = (long long)nex * lines;
   const long long plane = (long long)a.nx * a.ny;
   float rmax = 0.f;  // MODE 3: max |r| of this thread's nodes
+  // unknown `i` of an axis of n nodes, mirrored at a Neumann boundary
+  auto mirror = [](int i, int n) { return NEU ? (i < 0 ? -i : i >= n ? 2 * (n - 1) - i : i) : i; };
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
     const int ex = (int)(t % nex);
     const long long jl = t / nex;
     const int j = (int)(jl % a.ny), l = (int)(jl / a.ny);
     const long long line = jl * a.nx;
-    const int i0 = ex * K - 1;  // unknown index of node q = 0 (g = ex*K)
+    const int i0 = ex * K - OFF;  // unknown index of node q = 0 (g = ex*K)
+    auto own = [&](int i) { return NEU ? i < a.nx : i >= 0; };  // a node of this thread's that exists
     // x window: global nodes (ex-1)K .. (ex+1)K -> unknowns i0-K .. i0+K
     double w[BW];
 #pragma unroll
     for (int d = 0; d < BW; ++d) {
-      const int i = i0 - K + d;
+      const int i = mirror(i0 - K + d, a.nx);
       w[d] = (i >= 0 && i < a.nx) ? __ldg(a.u + line + i) : 0.0;
     }
     double acc[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) {
       const int i = i0 + q;
-      acc[q] = (MODE != 0 && i >= 0) ? __ldg(a.f + line + i) : 0.0;
+      acc[q] = (MODE != 0 && own(i)) ? __ldg(a.f + line + i) : 0.0;
     }
     // x part
 #pragma unroll
@@ -315,19 +324,19 @@ __global__ void __launch_bounds__(256) stencil_elem_kernel(StencilArgs a, const 
         else acc[q] -= hv * w[K + q + d];
       }
     }
-    // y part: row j of H_y, local index qy = (j+1) % K
+    // y part: row j of H_y, local index qy = (j+OFF) % K
     {
-      const int qy = (j + 1) % K;
+      const int qy = (j + OFF) % K;
       const int dlo = (qy == 0) ? -K : -qy, dhi = (qy == 0) ? K : K - qy;
       for (int d = dlo; d <= dhi; ++d) {
-        const int jj = j + d;
+        const int jj = mirror(j + d, a.ny);
         if (jj < 0 || jj >= a.ny) continue;
         const double hv = __ldg(Hqy + qy * BW + d + K);
         const double* src = a.u + ((long long)l * a.ny + jj) * a.nx;
 #pragma unroll
         for (int q = 0; q < K; ++q) {
           const int i = i0 + q;
-          const double uv = (i >= 0) ? __ldg(src + i) : 0.0;
+          const double uv = own(i) ? __ldg(src + i) : 0.0;
           if (MODE == 0) acc[q] += hv * uv;
           else acc[q] -= hv * uv;
         }
@@ -335,17 +344,17 @@ __global__ void __launch_bounds__(256) stencil_elem_kernel(StencilArgs a, const 
     }
     // z part
     {
-      const int qz = (l + 1) % K;
+      const int qz = (l + OFF) % K;
       const int dlo = (qz == 0) ? -K : -qz, dhi = (qz == 0) ? K : K - qz;
       for (int d = dlo; d <= dhi; ++d) {
-        const int ll = l + d;
+        const int ll = mirror(l + d, a.nz);
         if (ll < 0 || ll >= a.nz) continue;
         const double hv = __ldg(Hqz + qz * BW + d + K);
         const double* src = a.u + (long long)ll * plane + (long long)j * a.nx;
 #pragma unroll
         for (int q = 0; q < K; ++q) {
           const int i = i0 + q;
-          const double uv = (i >= 0) ? __ldg(src + i) : 0.0;
+          const double uv = own(i) ? __ldg(src + i) : 0.0;
           if (MODE == 0) acc[q] += hv * uv;
           else acc[q] -= hv * uv;
         }
@@ -355,7 +364,7 @@ __global__ void __launch_bounds__(256) stencil_elem_kernel(StencilArgs a, const 
 #pragma unroll
       for (int q = 0; q < K; ++q) {
         const int i = i0 + q;
-        if (i < 0) continue;
+        if (!own(i)) continue;
         const float rf = (float)acc[q];
         a.out32[(long long)i + (long long)a.Px * jl] = rf;
         rmax = fmaxf(rmax, fabsf(rf));
@@ -365,7 +374,7 @@ __global__ void __launch_bounds__(256) stencil_elem_kernel(StencilArgs a, const 
 #pragma unroll
     for (int q = 0; q < K; ++q) {
       const int i = i0 + q;
-      if (i < 0) continue;
+      if (!own(i)) continue;
       if (MODE != 2) {
         a.out64[line + i] = acc[q];
       } else {
@@ -384,9 +393,9 @@ __global__ void __launch_bounds__(256) stencil_elem_kernel(StencilArgs a, const 
   }
 }
 
-template <int K>
+template <int K, bool NEU>
 cudaError_t launch_elem(const StencilArgs& a, const DevAxis* ax, int mode, cudaStream_t s) {
-  const int nex = (a.nx + 1) / K;
+  const int nex = NEU ? (a.nx - 1) / K + 1 : (a.nx + 1) / K;
   const long long total = (long long)nex * a.ny * a.nz;
   long long b = (total + 255) / 256;
   // One thread per work item (no grid-stride wrap): blocks are issued in
@@ -394,10 +403,11 @@ cudaError_t launch_elem(const StencilArgs& a, const DevAxis* ax, int mode, cudaS
   // neighbours of a plane are still in L2 when they are read again.
   if (b > 0x7FFFFFFFLL) b = 0x7FFFFFFFLL;
   const int grid = (int)(b < 1 ? 1 : b);
-  if (mode == 0) stencil_elem_kernel<K, 0><<<grid, 256, 0, s>>>(a, ax[0].Hq, ax[1].Hq, ax[2].Hq, nex);
-  else if (mode == 1) stencil_elem_kernel<K, 1><<<grid, 256, 0, s>>>(a, ax[0].Hq, ax[1].Hq, ax[2].Hq, nex);
-  else if (mode == 2) stencil_elem_kernel<K, 2><<<grid, 256, 0, s>>>(a, ax[0].Hq, ax[1].Hq, ax[2].Hq, nex);
-  else stencil_elem_kernel<K, 3><<<grid, 256, 0, s>>>(a, ax[0].Hq, ax[1].Hq, ax[2].Hq, nex);
+  const double *hx = ax[0].Hq, *hy = ax[1].Hq, *hz = ax[2].Hq;
+  if (mode == 0) stencil_elem_kernel<K, 0, NEU><<<grid, 256, 0, s>>>(a, hx, hy, hz, nex);
+  else if (mode == 1) stencil_elem_kernel<K, 1, NEU><<<grid, 256, 0, s>>>(a, hx, hy, hz, nex);
+  else if (mode == 2) stencil_elem_kernel<K, 2, NEU><<<grid, 256, 0, s>>>(a, hx, hy, hz, nex);
+  else stencil_elem_kernel<K, 3, NEU><<<grid, 256, 0, s>>>(a, hx, hy, hz, nex);
   return cudaGetLastError();
 }
 
@@ -509,16 +519,17 @@ StencilArgs stencil_args(const Geom& g, int k, const DevAxis* ax, const double* 
 
 cudaError_t launch_stencil_any(const StencilArgs& a, const Geom& g, const DevAxis* ax, cudaStream_t s) {
   const long long N = (long long)g.nx * g.ny * g.nz;
-  switch (g.bc == 0 ? a.k : 0) {  // the element-pattern kernels assume Dirichlet rows
-    case 1: return launch_elem<1>(a, ax, a.mode, s);
-    case 2: return launch_elem<2>(a, ax, a.mode, s);
-    case 3: return launch_elem<3>(a, ax, a.mode, s);
-    case 4: return launch_elem<4>(a, ax, a.mode, s);
-    case 5: return launch_elem<5>(a, ax, a.mode, s);
-    case 6: return launch_elem<6>(a, ax, a.mode, s);
-    case 7: return launch_elem<7>(a, ax, a.mode, s);
-    case 8: return launch_elem<8>(a, ax, a.mode, s);
-    default:  // higher degrees and Neumann data: one thread per node, per-row band ranges
+  const bool neu = g.bc != 0;
+  switch (a.k) {
+    case 1: return neu ? launch_elem<1, true>(a, ax, a.mode, s) : launch_elem<1, false>(a, ax, a.mode, s);
+    case 2: return neu ? launch_elem<2, true>(a, ax, a.mode, s) : launch_elem<2, false>(a, ax, a.mode, s);
+    case 3: return neu ? launch_elem<3, true>(a, ax, a.mode, s) : launch_elem<3, false>(a, ax, a.mode, s);
+    case 4: return neu ? launch_elem<4, true>(a, ax, a.mode, s) : launch_elem<4, false>(a, ax, a.mode, s);
+    case 5: return neu ? launch_elem<5, true>(a, ax, a.mode, s) : launch_elem<5, false>(a, ax, a.mode, s);
+    case 6: return neu ? launch_elem<6, true>(a, ax, a.mode, s) : launch_elem<6, false>(a, ax, a.mode, s);
+    case 7: return neu ? launch_elem<7, true>(a, ax, a.mode, s) : launch_elem<7, false>(a, ax, a.mode, s);
+    case 8: return neu ? launch_elem<8, true>(a, ax, a.mode, s) : launch_elem<8, false>(a, ax, a.mode, s);
+    default:  // higher degrees: one thread per node, per-row band ranges
       stencil_kernel<<<(int)((N + 255) / 256 < 0x7FFFFFFF ? (N + 255) / 256 : 0x7FFFFFFF), 256, 0, s>>>(a);
       return cudaGetLastError();
   }
