@@ -51,8 +51,9 @@ constexpr int T_CL = 4;                // cluster size of the W multicast
 // or the FP64 solution (stored, or added to).
 enum : int { T_OUT_T32 = 0, T_OUT_T32_DIV = 1, T_OUT_F64 = 2, T_OUT_F64_ACCUM = 3 };
 // Epilogue warps: two per TMEM lane quadrant, four for the FP64 outputs
-// (8-16 bytes per element instead of 4).
-__host__ __device__ constexpr int t_epi_warps(int mode) { return mode >= 2 ? 16 : 8; }
+// (8-16 bytes per element instead of 4) and for the division (a reciprocal, a
+// product and a shuffle per element: 310 -> 241 us a pass at n = 511).
+__host__ __device__ constexpr int t_epi_warps(int mode) { return mode >= T_OUT_T32_DIV ? 16 : 8; }
 __host__ __device__ constexpr int t_threads(int mode) { return 64 + 32 * t_epi_warps(mode); }
 
 // Instruction descriptor, kind::tf32: FP32 accumulator (bits 4-5 = 1), A and
@@ -439,24 +440,26 @@ __global__ void __launch_bounds__(t_threads(MODE), 1)
   }
 }
 
-// FP64 array (x fastest, pitch nx) -> TF32-rounded FP32 array at pitch Px.
-// Blocks walk the (j, l) lines; a lane converts 4 consecutive entries and
-// writes them as one 16-byte store (rows of pitch Px, a multiple of 16, are
-// 64-byte aligned); the pad entries i >= nx are written as zeros.
+// FP64 array (x fastest, pitch nx) -> TF32-rounded FP32 array at pitch Px,
+// zeros in the pad entries i >= nx.  Bound by memory: a warp takes a line and
+// walks it 256 entries at a time, eight loads a lane in flight, a lane's
+// entries 32 apart (each load and store of the warp one contiguous piece; nx
+// may be odd, so a wider load has no alignment to count on).  n = 511:
+// 322 us with four adjacent entries a lane and 128 of 256 lanes busy -> 246 us, 6.5 TB/s.
 __global__ void __launch_bounds__(256) to_tf32_kernel(const double* __restrict__ in, float* __restrict__ out, int nx,
                                                       int Px, long long lines) {
-  const int chunks = Px >> 2;
-  for (long long line = blockIdx.x; line < lines; line += gridDim.x) {
+  const int lane = threadIdx.x & 31;
+  const long long warps = (long long)gridDim.x * 8;
+  for (long long line = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); line < lines; line += warps) {
     const double* row = in + line * nx;
-    float4* orow = reinterpret_cast<float4*>(out + line * Px);
-    for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-      const int i = 4 * c;
-      float4 v;
-      v.x = i < nx ? tf32_round(f64_to_f32_rn(row[i])) : 0.f;
-      v.y = i + 1 < nx ? tf32_round(f64_to_f32_rn(row[i + 1])) : 0.f;
-      v.z = i + 2 < nx ? tf32_round(f64_to_f32_rn(row[i + 2])) : 0.f;
-      v.w = i + 3 < nx ? tf32_round(f64_to_f32_rn(row[i + 3])) : 0.f;
-      orow[c] = v;
+    float* orow = out + line * Px;
+    for (int i0 = lane; i0 < Px; i0 += 256) {
+      double x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[q] = i0 + 32 * q < nx ? row[i0 + 32 * q] : 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (i0 + 32 * q < Px) orow[i0 + 32 * q] = tf32_round(f64_to_f32_rn(x[q]));
     }
   }
 }
@@ -556,7 +559,9 @@ int tf32_config(int nK, int d1, int d2) { return tf32_variant(nK, d1, d2); }
 
 cudaError_t launch_to_tf32(const Geom& g, const double* in, float* out, cudaStream_t s) {
   const long long lines = (long long)g.ny * g.nz;
-  const long long blocks = lines < 152LL * 16 ? (lines < 1 ? 1 : lines) : 152LL * 16;
+  long long blocks = (lines + 7) / 8;  // a warp per line
+  if (blocks > 152LL * 16) blocks = 152LL * 16;
+  if (blocks < 1) blocks = 1;
   to_tf32_kernel<<<(unsigned)blocks, 256, 0, s>>>(in, out, g.nx, g.Px, lines);
   return cudaGetLastError();
 }
