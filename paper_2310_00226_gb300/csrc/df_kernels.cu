@@ -10,7 +10,9 @@
 // Two kernels, both bound by their FP32 operations (12 a term, k + 2 terms per
 // axis and node, beside 20 bytes of HBM per node):
 //  - k in {1, 2, 4}: a warp per line, a lane per 4 nodes, whose x rows are known
-//    at compile time because 4 % k == 0 (stencil_df4_kernel);
+//    at compile time because 4 % k == 0 (stencil_df4_kernel); the nodes in pairs
+//    in packed f32x2 instructions and the loads of a row's lines together:
+//    n = 255, k = 4 178 -> 157 us with u's low half zero, 194 -> 180 else;
 //  - other k: blocks of 8 lines x 64 nodes marching along z (stencil_df_kernel).
 //    Every plane is staged once in shared memory (cp.async, two planes ahead),
 //    adds its z terms to the running sums of its element's k + 1 planes, and
@@ -20,7 +22,7 @@
 //    offsets enter, with zeros outside the node's band.  A thread per element
 //    and line, which this replaces, read its neighbours at a stride of k and
 //    waited on L1: 449x320x383, k = 3 1.02 -> 0.60 ms; 383^3, k = 6 1.16 -> 0.88.
-//    At k = 4 it takes 11.7 ms at n = 999 against the vector kernel's 11.4.
+//    At k = 4 it takes 11.7 ms at n = 999, more than the vector kernel.
 // Tried: summing onto an offset that dominates every term, so that a fast
 // two-sum suffices (6 operations a term, n = 999 8.2 ms): its noise, relative to
 // the largest sum on the grid, is some 80 times the two-sum's and took the
@@ -62,6 +64,8 @@ __device__ __forceinline__ f2 mul2(f2 a, f2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+// -a as a multiply-add: a sign flip is two integer instructions
+__device__ __forceinline__ f2 neg2(f2 a) { return fma2(a, 0xBF800000BF800000ull, 0x8000000080000000ull); }
 
 // Exact split of an FP64 value into hi (first 24 significant bits, truncated)
 // and lo (the next 24, rounded) with integer operations only.  |x| < 2^-126
@@ -101,7 +105,7 @@ struct DfArgs {
 template <bool EXACT, bool LO0>
 __device__ __forceinline__ void df_term(f2& S, f2& Sl, f2 nh, f2 nl, f2 nl2, f2 uh, f2 ul) {
   const f2 p = mul2(nh, uh);
-  f2 t = fma2(nh, uh, p ^ 0x8000000080000000ull);
+  f2 t = fma2(nh, uh, neg2(p));
   if (EXACT) t = fma2(nl2, uh, t);
   t = fma2(nl, uh, t);
   if (!LO0) t = fma2(nh, ul, t);
@@ -387,32 +391,36 @@ cudaError_t launch_df(DfArgs a, const DevAxis* ax, bool exact, bool lo_zero, int
   return lo_zero ? run_df<K, false, true>(a, cf, grid, s) : run_df<K, false, false>(a, cf, grid, s);
 }
 
-// (ah, al) -= (ch + cl [+ cl2]) * (uh + ul), dropping cl*ul and cl2*ul; the
-// third coefficient term cl2 enters only when EXACT (else the 48-bit ch + cl).
-// LO0: ul is zero (the solution right after the first solve), and the ch*ul
-// term, exactly 0 there, is not formed (the same result).
-template <bool EXACT = false, bool LO0 = false>
-__device__ __forceinline__ void df_sub_prod(float& ah, float& al, float ch, float cl, float uh, float ul,
-                                            float cl2 = 0.f) {
-  const float p = ch * uh;
-  const float e = fmaf(ch, uh, -p);
-  const float t0 = fmaf(cl, uh, EXACT ? fmaf(cl2, uh, e) : e);
-  const float t = LO0 ? t0 : fmaf(ch, ul, t0);
-  const float s = ah - p;
-  const float bb = s - ah;
-  const float err = (ah - (s - bb)) - (p + bb);
-  ah = s;
-  al = al + (err - t);
+// One term of one node's running sum: (S, Sl) += (nh + nl [+ nl2]) (uh + ul),
+// dropping nl ul and nl2 ul; the third coefficient term enters only when EXACT
+// (else the 48-bit nh + nl).  LO0: ul is zero (the solution right after the
+// first solve), and nh ul, exactly 0 there, is not formed (the same result).
+template <bool EXACT, bool LO0>
+__device__ __forceinline__ void df_add_prod(float& S, float& Sl, float nh, float nl, float uh, float ul, float nl2) {
+  const float p = nh * uh;
+  float t = fmaf(nh, uh, -p);
+  if (EXACT) t = fmaf(nl2, uh, t);
+  t = fmaf(nl, uh, t);
+  if (!LO0) t = fmaf(nh, ul, t);
+  const float s = S + p;
+  const float bb = s - S;
+  const float err = (S - (s - bb)) + (p - bb);
+  S = s;
+  Sl = Sl + (err + t);
 }
 
-// Rows of H per local index for the vector residual (k <= 4), as kernel
-// parameters: the x rows are read at compile-time offsets (no load
-// instructions), the y and z rows at warp-uniform offsets.
+// Negated rows of H for the vector residual (k <= 4), as kernel parameters.
+// x: entry [P][m] holds what node m of a lane's 12-node window contributes to
+// the lane's nodes 2P and 2P + 1 (read at compile-time offsets); y and z: the
+// rows per local index, each entry twice (read at warp-uniform offsets).
 struct Df4Coef {
-  float h[3][4 * 9];
-  float l[3][4 * 9];
-  float l2[3][4 * 9];  // third terms (used when EXACT)
+  float2 xh[2][12], xl[2][12], xl2[2][12];     // l2: third terms (used when EXACT)
+  float2 h[2][4 * 9], l[2][4 * 9], l2[2][4 * 9];
 };
+
+// Window nodes (4 + p + d) in the band of the row at position p of a lane's 4.
+__host__ __device__ constexpr int df4_lo(int K, int p) { return 4 + p - ((p + 1) % K == 0 ? K : (p + 1) % K); }
+__host__ __device__ constexpr int df4_hi(int K, int p) { return 4 + p + K - (p + 1) % K; }
 
 // Double-FP32 residual for k in {1, 2, 4}.  A lane handles the 4 consecutive
 // nodes i = 4c .. 4c+3 of one (j, l) line -- one float4 of each of u_hi and
@@ -435,17 +443,19 @@ __global__ void __launch_bounds__(256, 4) stencil_df4_kernel(DfArgs a, const __g
        line += (long long)gridDim.x * 8) {  // warp-uniform
     const int j = (int)(line % a.ny), l = (int)(line / a.ny);
     const int qy = (j + 1) % K, qz = (l + 1) % K;
-    const int ylo = (qy == 0) ? -K : -qy, yhi = (qy == 0) ? K : K - qy;
-    const int zlo = (qz == 0) ? -K : -qz, zhi = (qz == 0) ? K : K - qz;
     const long long row4 = line * chunks;
     const double* frow = a.f + line * a.nx;
     for (int c = lane; c < chunks; c += 32) {
       const int i0 = 4 * c;
-      float ah[4], al[4];
+      f2 S[2], Sl[2];  // running sums of the node pairs (0, 1) and (2, 3)
 #pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        if (i0 + p < a.nx) f64_to_df(__ldg(frow + i0 + p), ah[p], al[p]);
-        else { ah[p] = 0.f; al[p] = 0.f; }
+      for (int P = 0; P < 2; ++P) {
+        float h[2] = {0.f, 0.f}, l[2] = {0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (i0 + 2 * P + e < a.nx) f64_to_df(__ldg(frow + i0 + 2 * P + e), h[e], l[e]);
+        S[P] = pack2(h[0], h[1]);
+        Sl[P] = pack2(l[0], l[1]);
       }
       // x: nodes i0-4 .. i0+7 (the neighbouring chunks; zero outside the line)
       float wh[12], wl[12];
@@ -461,40 +471,65 @@ __global__ void __launch_bounds__(256, 4) stencil_df4_kernel(DfArgs a, const __g
         wl[6] = cl.z; wl[7] = cl.w; wl[8] = nl.x; wl[9] = nl.y; wl[10] = nl.z; wl[11] = nl.w;
       }
 #pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        const int q = (p + 1) % K;
-        const int dlo = (q == 0) ? -K : -q, dhi = (q == 0) ? K : K - q;
+      for (int m = 0; m < 12; ++m) {
 #pragma unroll
-        for (int d = -K; d <= K; ++d)
-          if (d >= dlo && d <= dhi)  // compile-time after unrolling
-            df_sub_prod<EXACT, LO0>(ah[p], al[p], cf.h[0][q * BW + d + K], cf.l[0][q * BW + d + K], wh[4 + p + d], wl[4 + p + d],
-                        EXACT ? cf.l2[0][q * BW + d + K] : 0.f);
+        for (int P = 0; P < 2; ++P) {
+          const bool in0 = m >= df4_lo(K, 2 * P) && m <= df4_hi(K, 2 * P);  // compile-time after unrolling
+          const bool in1 = m >= df4_lo(K, 2 * P + 1) && m <= df4_hi(K, 2 * P + 1);
+          const float2 nh = cf.xh[P][m], nl = cf.xl[P][m], n2 = EXACT ? cf.xl2[P][m] : make_float2(0.f, 0.f);
+          if (in0 && in1) {
+            df_term<EXACT, LO0>(S[P], Sl[P], as2(nh), as2(nl), as2(n2), pack2(wh[m], wh[m]),
+                                LO0 ? 0ull : pack2(wl[m], wl[m]));
+          } else if (in0 || in1) {
+            float s0, s1, l0, l1;
+            unpack2(S[P], s0, s1);
+            unpack2(Sl[P], l0, l1);
+            if (in0) df_add_prod<EXACT, LO0>(s0, l0, nh.x, nl.x, wh[m], wl[m], n2.x);
+            else df_add_prod<EXACT, LO0>(s1, l1, nh.y, nl.y, wh[m], wl[m], n2.y);
+            S[P] = pack2(s0, s1);
+            Sl[P] = pack2(l0, l1);
+          }
+        }
       }
-      // y and z: the rows of the neighbouring lines, one float4 pair per row
+      // y and z: the rows of the neighbouring lines, in order of their offset: at
+      // a vertex (q = 0) the k before it, then the k + 1 of the element.  The
+      // latter's loads depend on no branch and go out together, lines outside
+      // the grid counting as zeros, except where both halves of five lines
+      // would not fit the registers (n = 511, k = 4: 1.37 ms with a branch at
+      // every offset, 1.43 without; with one half 1.23 and 1.17).
+      auto rows = [&](int w, int q, int pos, int n, long long pitch) {
+        auto load = [&](const float4* U, int d) {
+          return pos + d >= 0 && pos + d < n ? __ldg(reinterpret_cast<const ulonglong2*>(U + row4 + d * pitch + c))
+                                             : make_ulonglong2(0, 0);
+        };
+        auto term = [&](int at, ulonglong2 vh, ulonglong2 vl) {
+          const f2 nh = as2(cf.h[w][at]), nl = as2(cf.l[w][at]), n2 = EXACT ? as2(cf.l2[w][at]) : 0ull;
+          df_term<EXACT, LO0>(S[0], Sl[0], nh, nl, n2, vh.x, vl.x);
+          df_term<EXACT, LO0>(S[1], Sl[1], nh, nl, n2, vh.y, vl.y);
+        };
+        if constexpr (K == 4 && !LO0) {
 #pragma unroll
-      for (int d = -K; d <= K; ++d) {
-        if (d < ylo || d > yhi || j + d < 0 || j + d >= a.ny) continue;  // warp-uniform
-        const float chh = cf.h[1][qy * BW + d + K], cll = cf.l[1][qy * BW + d + K];
-        const float cl2 = EXACT ? cf.l2[1][qy * BW + d + K] : 0.f;
-        const float4 vh = __ldg(UH + row4 + (long long)d * chunks + c);
-        const float4 vl = LO0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(UL + row4 + (long long)d * chunks + c);
-        df_sub_prod<EXACT, LO0>(ah[0], al[0], chh, cll, vh.x, vl.x, cl2);
-        df_sub_prod<EXACT, LO0>(ah[1], al[1], chh, cll, vh.y, vl.y, cl2);
-        df_sub_prod<EXACT, LO0>(ah[2], al[2], chh, cll, vh.z, vl.z, cl2);
-        df_sub_prod<EXACT, LO0>(ah[3], al[3], chh, cll, vh.w, vl.w, cl2);
-      }
+          for (int d = -K; d <= K; ++d) {  // warp-uniform conditions
+            if (d < (q == 0 ? -K : -q) || d > (q == 0 ? K : K - q) || pos + d < 0 || pos + d >= n) continue;
+            term(q * BW + d + K, load(UH, d), load(UL, d));
+          }
+        } else {
+          if (q == 0) {  // warp-uniform
 #pragma unroll
-      for (int d = -K; d <= K; ++d) {
-        if (d < zlo || d > zhi || l + d < 0 || l + d >= a.nz) continue;  // warp-uniform
-        const float chh = cf.h[2][qz * BW + d + K], cll = cf.l[2][qz * BW + d + K];
-        const float cl2 = EXACT ? cf.l2[2][qz * BW + d + K] : 0.f;
-        const float4 vh = __ldg(UH + row4 + (long long)d * splane + c);
-        const float4 vl = LO0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(UL + row4 + (long long)d * splane + c);
-        df_sub_prod<EXACT, LO0>(ah[0], al[0], chh, cll, vh.x, vl.x, cl2);
-        df_sub_prod<EXACT, LO0>(ah[1], al[1], chh, cll, vh.y, vl.y, cl2);
-        df_sub_prod<EXACT, LO0>(ah[2], al[2], chh, cll, vh.z, vl.z, cl2);
-        df_sub_prod<EXACT, LO0>(ah[3], al[3], chh, cll, vh.w, vl.w, cl2);
-      }
+            for (int d = -K; d < 0; ++d) term(d + K, load(UH, d), LO0 ? make_ulonglong2(0, 0) : load(UL, d));
+          }
+#pragma unroll
+          for (int t = 0; t <= K; ++t)
+            term(q * (BW - 1) + K + t, load(UH, t - q), LO0 ? make_ulonglong2(0, 0) : load(UL, t - q));
+        }
+      };
+      rows(0, qy, j, a.ny, chunks);
+      rows(1, qz, l, a.nz, splane);
+      float ah[4], al[4];
+      unpack2(S[0], ah[0], ah[1]);
+      unpack2(S[1], ah[2], ah[3]);
+      unpack2(Sl[0], al[0], al[1]);
+      unpack2(Sl[1], al[2], al[3]);
       float r[4];
 #pragma unroll
       for (int p = 0; p < 4; ++p) r[p] = (i0 + p < a.nx) ? ah[p] + al[p] : 0.f;  // pads stay zero
@@ -528,11 +563,22 @@ __global__ void __launch_bounds__(256, 4) stencil_df4_kernel(DfArgs a, const __g
 template <int K>
 cudaError_t launch_df4(const DfArgs& a, const DevAxis* ax, bool exact, bool lo_zero, cudaStream_t s) {
   Df4Coef cf{};
-  for (int w = 0; w < 3; ++w)
-    for (int e = 0; e < K * (2 * K + 1); ++e) {
-      cf.h[w][e] = ax[w].Hq_hi_host[e];
-      cf.l[w][e] = ax[w].Hq_lo_host[e];
-      cf.l2[w][e] = ax[w].Hq_lo2_host[e];
+  constexpr int BW = 2 * K + 1;
+  for (int m = 0; m < 12; ++m)
+    for (int p = 0; p < 4; ++p) {
+      if (m < df4_lo(K, p) || m > df4_hi(K, p)) continue;
+      const int e = (p + 1) % K * BW + m - 4 - p + K;
+      const float h = -ax[0].Hq_hi_host[e], l = -ax[0].Hq_lo_host[e], l2 = -ax[0].Hq_lo2_host[e];
+      float2 *ph = &cf.xh[p / 2][m], *pl = &cf.xl[p / 2][m], *p2 = &cf.xl2[p / 2][m];
+      if (p % 2 == 0) { ph->x = h; pl->x = l; p2->x = l2; }
+      else { ph->y = h; pl->y = l; p2->y = l2; }
+    }
+  for (int w = 0; w < 2; ++w)
+    for (int e = 0; e < K * BW; ++e) {
+      const float h = -ax[w + 1].Hq_hi_host[e], l = -ax[w + 1].Hq_lo_host[e], l2 = -ax[w + 1].Hq_lo2_host[e];
+      cf.h[w][e] = make_float2(h, h);
+      cf.l[w][e] = make_float2(l, l);
+      cf.l2[w][e] = make_float2(l2, l2);
     }
   // One block per 8 consecutive lines and no grid stride: the resident blocks
   // then sweep the grid plane by plane, so the rows 1..K planes away that a
