@@ -34,6 +34,13 @@ METRIC = "1000^3 Q^4 solve ms & GDoF/s on 1 GB300: FP64 vs refined split-BF16 at
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 
 
+def mode_flops(n: int, parity: bool) -> float:
+    """Flops of one mode product on n^3 nodes: 2 n^4 with the full matrix; in
+    parity order (symmetric mesh) the matrix is two blocks of about n / 2."""
+    h = (n + 1) // 2
+    return 2.0 * n * n * (h * h + (n - h) * (n - h)) if parity else 2.0 * n**4
+
+
 def tc_traffic_per_launch(n: int):
     """DRAM bytes (read + write) of one tensor-core pass from the committed ncu
     capture, scaled to n by the DoF processed; None once the kernel source has
@@ -353,7 +360,7 @@ def run_ours(args, rank: int, world: int, local_rank: int):
                 "steps": args.fp64_steps, "warmup": args.fp64_warmup, "path": "FP64 DMMA mode products + 1 FP64 sweep",
                 "rel_linf_bf16x3_vs_fp64": diff, "speedup_bf16x3_over_fp64": ms64 / ms,
                 "dmma_kernel_avg_ms": f64_ms / max(1, f64_n),
-                "dmma_achieved_tflops": 2.0 * n**4 / (f64_ms / max(1, f64_n) / 1e3) / 1e12}
+                "dmma_achieved_tflops": mode_flops(n, True) / (f64_ms / max(1, f64_n) / 1e3) / 1e12}
         plan.set_precision("bf16x3", args.sweeps)
 
     # ---- FP32 CUDA-core tier (autotuned tiles) with FP64 refinement sweeps
@@ -374,7 +381,7 @@ def run_ours(args, rank: int, world: int, local_rank: int):
                 "rel_linf_vs_exact_solution": float((u - u_ex).abs().max() / u_ex.abs().max()),
                 "rel_linf_vs_bf16x3": float((u - u_bf).abs().max() / u_bf.abs().max()),
                 "pass_avg_ms": f_ms / max(1, f_n),
-                "pass_tflops": 2.0 * n**4 / (f_ms / max(1, f_n) / 1e3) / 1e12,
+                "pass_tflops": mode_flops(n, args.fp32_sweeps >= 2) / (f_ms / max(1, f_n) / 1e3) / 1e12,
                 "tiles": [plan.tuned_config(a) for a in range(3)]}
         del u_ex
         plan.set_precision("bf16x3", args.sweeps)
@@ -433,13 +440,17 @@ def run_ours(args, rank: int, world: int, local_rank: int):
 
     # ---- roofline of the dominant kernel (tcgen05 BF16x3 mode product)
     tc_avg_ms = tc_ms / max(1, tc_n)
-    flops_per_launch = 3 * 2.0 * n**4  # 3 bf16 products per useful FMA, 2 flops each, n^4 FMA per pass
+    # 3 bf16 products per useful multiply-add; refined solves on 255 nodes an axis
+    # and more run their passes in parity order
+    parity = args.sweeps >= 2 and n >= 255
+    flops_per_launch = 3 * mode_flops(n, parity)
     achieved = flops_per_launch / (tc_avg_ms / 1e3) / 1e12
     peak = float(peaks.get("bf16_tflops_sustained", PEAKS_FALLBACK["bf16_tflops_sustained"]))
-    roofline = {"kernel": "mode_product_bf16x3 (tcgen05)", "bound": "tensor", "achieved": achieved, "peak": peak,
+    roofline = {"kernel": "mode_product_fold (tcgen05, split bf16, parity order)" if parity else
+                "mode_product_bf16x3 (tcgen05)", "bound": "tensor", "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": achieved / peak, "traffic": tc_traffic_per_launch(n),
                 "traffic_source": "profiles/roofline_inputs.json (ncu at n=511, scaled by DoF per launch)",
-                "algorithmic_bytes_per_launch": 8.0 * ((n + 15) // 16 * 16) * n * n,
+                "algorithmic_bytes_per_launch": 8.0 * ((n + 15) // 16 * 16) * n * n,  # 4 read, 4 written
                 "peak_source": f"{peak_src} bf16_tflops_sustained",
                 "flops_per_launch": flops_per_launch, "avg_launch_ms": tc_avg_ms, "launches": tc_n,
                 "share_of_step": tc_ms / (ms_profiled * args.steps),
@@ -460,8 +471,9 @@ def run_ours(args, rank: int, world: int, local_rank: int):
                "residuals": {"launches": st_n, "ms_per_step": st_ms / max(1, args.steps),
                              "note": "every residual kernel of a step (double-FP32 sweeps, the FP64-accurate "
                                      "sweep and its scale reductions / conversion)"},
-               "split": {"launches": sp_n, "avg_ms": sp_ms / max(1, sp_n),
-                         "gbs": 12.0 * dofs / (sp_ms / max(1, sp_n) / 1e3) / 1e9}}
+               "split": {"launches": sp_n, "ms_per_step": sp_ms / max(1, args.steps),
+                         "note": "conversion of f, and in parity order the folding of each right-hand side and the "
+                                 "unfolding of each correction onto the solution"}}
 
     cpu = None
     if rank == 0 and world == 1 and args.cpu_baseline:

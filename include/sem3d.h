@@ -71,6 +71,11 @@ typedef enum {
  *                  significant bits per pass) of arrays scaled by powers of
  *                  two chosen on the device from tracked maxima (fp16's
  *                  range is small); needs k <= 8.
+ * The 1D operators of a uniform mesh commute with its mirror image, so T and
+ * T^-1 split into blocks acting on the even and the odd part of a field, which
+ * is half the work.  In use for every FP64 product, for FP32 with two sweeps
+ * or more, and for BF16X3 with two sweeps or more on at least 255 nodes along
+ * every axis (results that do not depend on how a correction solve rounds).
  * FP64 accuracy is recovered by iterative refinement (sem3d_set_precision). */
 typedef enum {
   SEM3D_FP64 = 0,
@@ -317,8 +322,9 @@ sem3d_status sem3d_sync_check(sem3d_handle h, void* stream);
  * kernel class, the number of kernels launched and their summed device time
  * in milliseconds.  Kernel classes: 0 = tensor-core (tcgen05) mode product,
  * 1 = FP64 (DMMA) mode product, 2 = FP64 stencil / residual, 3 = FP64 ->
- * split-bf16 conversion; the tensor-core launches of class 0 are also counted
- * by pass: 4 = x pass, 5 = y pass, 6 = z pass writing split-bf16 output,
+ * split-bf16 conversion (in parity order also the folding of right-hand sides
+ * and the unfolding of corrections); the tensor-core launches of class 0 are
+ * also counted by pass: 4 = x pass, 5 = y pass, 6 = z pass writing split-bf16 output,
  * 7 = the last pass of a solve (writes or accumulates FP64 u); 8 = FP32
  * CUDA-core mode product. */
 sem3d_status sem3d_profile(sem3d_handle h, int enable);
@@ -357,7 +363,8 @@ sem3d_status sem3d_set_tuned_config(sem3d_handle h, int axis, int config);
  * tier (0 for a shape never measured); sem3d_set_tc_config pins `config` (0
  * or 1) for this plan's pass along `axis` in all three tiers, for every plan
  * of the process with that shape (sem3d_set_precision does not re-measure a
- * known shape). */
+ * known shape).  The parity-order passes of refined BF16X3 solves (see
+ * sem3d_precision) always run on CTA pairs; the choice does not touch them. */
 sem3d_status sem3d_tc_config(sem3d_handle h, int axis, int* config);
 sem3d_status sem3d_set_tc_config(sem3d_handle h, int axis, int config);
 

@@ -398,8 +398,7 @@ sem3d_status solve_once_bf16x3(sem3d_plan* p, TcBuffers S0, TcBuffers S1, double
 // cost what is saved.  Refined solves, node order -> parity order: n = 127
 // 377 -> 421 us, 255 1647 -> 1644 (a group of 16 problems, most of them 255
 // and larger, 52.0 -> 51.3 ms), 383 5455 -> 5160, 511 12.6 -> 11.5 ms, 767
-// 49.7 -> 42.7 ms, 999 133.8 ->
-// 102.8 ms; 511x63x255 978 -> 1007 us.
+// 49.7 -> 42.7 ms, 999 133.8 -> 102.8 ms; 511x63x255 978 -> 1007 us.
 constexpr int kFoldMin = 255;
 bool use_fold(const sem3d_plan* h) {
   return h->prec == SEM3D_BF16X3 && h->sweeps >= 2 && std::min(h->g.nx, std::min(h->g.ny, h->g.nz)) >= kFoldMin;

@@ -10,7 +10,7 @@ refined solve of the library is held to, 1e-12 of the largest value
 import numpy as np
 import pytest
 
-from oracle import refined_solve, sem_1d
+from oracle import apply_h, refined_solve, sem_1d
 from paper_2310_00226_gb300.inputs import random_rhs
 
 torch = pytest.importorskip("torch")
@@ -123,3 +123,41 @@ def test_batch_of_both_orders_is_bit_identical_to_single_solves():
             assert torch.equal(one, u)
     for p in plans:
         p.close()
+
+
+@pytest.mark.parametrize("ne3", [(1, 1, 1), (2, 3, 1), (45, 2, 3)])
+@pytest.mark.parametrize("k", range(1, 10))  # 9: the per-node kernel
+def test_neumann_apply_by_elements(k, ne3):
+    # tolerance: 1e-13 of the largest possible sum of the terms' magnitudes (at
+    # most 3 (2k + 1) roundings of 2^-53, and rows that differ in their last digits)
+    from paper_2310_00226_gb300 import sem3d
+    L, c = (1.0, 1.4, 0.8), 0.7
+    axes = [sem_1d(k, ne, 0.0, Lb, "neumann") for ne, Lb in zip(ne3, L)]
+    U = random_rhs(*[ax.n for ax in axes], seed=k)
+    u = torch.from_numpy(U).cuda()
+    Au = torch.full_like(u, float("nan"))
+    with sem3d.Plan(*[ax.n for ax in axes], k, L, c, bc="neumann") as p:
+        p.apply(u, Au)
+        p.sync_check()
+    scale = (sum(abs(ax.H_sparse()).sum(axis=1).max() for ax in axes) + c) * np.abs(U).max()
+    assert np.abs(Au.cpu().numpy() - apply_h(U, *axes, c)).max() <= 1e-13 * scale
+
+
+@pytest.mark.parametrize("k,ne3", [(1, (6, 4, 8)), (1, (150, 3, 2)), (2, (3, 5, 4)), (2, (70, 2, 9)), (4, (2, 3, 2)),
+                                   (4, (40, 5, 3)), (4, (33, 2, 2))])
+def test_double_fp32_residual_in_pairs(k, ne3):
+    # every residual in double-FP32: 2^-48 of the operator's terms, amplified by the conditioning
+    from paper_2310_00226_gb300 import sem3d
+    L, c = (1.0, 1.3, 0.8), 1.5
+    n3 = [k * ne - 1 for ne in ne3]
+    axes = [sem_1d(k, ne, 0.0, Lb) for ne, Lb in zip(ne3, L)]
+    F = random_rhs(*n3, seed=k)
+    f = torch.from_numpy(F).cuda()
+    u = torch.full_like(f, float("nan"))
+    with sem3d.Plan(*n3, k, L, c) as p:
+        p.set_precision("bf16x3", 4)
+        p.set_residual("df")
+        p.solve(f, u)
+        p.sync_check()
+    ref = refined_solve(F, *axes, c, 1)
+    assert np.abs(u.cpu().numpy() - ref).max() / np.abs(ref).max() <= max(1e-12, kappa(axes, c) * 2.0**-48)
