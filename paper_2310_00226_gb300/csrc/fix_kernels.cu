@@ -44,6 +44,7 @@
 // the operator exactly that of the FP64 rows.
 #include "sem3d_internal.h"
 
+#include <algorithm>
 #include <cmath>
 
 namespace sem3d {
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(256) max_exponent_kernel(const double* __restr
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
     m = max(m, biased_exp(__ldg(in + i)));
   m = (int)__reduce_max_sync(0xFFFFFFFFu, (unsigned int)m);
-  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(slot, m);
+  if ((threadIdx.x & 31) == 0 && m > __ldcg(slot)) atomicMax(slot, m);  // most warps skip it
 }
 
 // The scale exponent s of U = round(u 2^s): |U| <= 2^57 and
@@ -486,7 +487,7 @@ cudaError_t launch_residual_fixed(const Geom& g, int k, const FixCoef& cf, const
   if (g.bc != 0 || k < 1 || k > 8) return cudaErrorInvalidValue;
   const long long N = (long long)g.nx * g.ny * g.nz;
   const long long lines = (long long)g.ny * g.nz;
-  const int red_grid = num_sms * 8;
+  const int red_grid = (int)std::min<long long>((N + 1023) / 1024, (long long)num_sms * 8);  // 4 values a thread
   cudaError_t e = cudaSuccess;
   if (!u_exponent_known) e = cudaMemsetAsync(state, 0, sizeof(int), s);
   if (e == cudaSuccess && !f_exponent_known) e = cudaMemsetAsync(state + 1, 0, sizeof(int), s);
