@@ -7,6 +7,7 @@
 #pragma once
 
 #include "sem3d_internal.h"
+#include "tc_index.h"
 #include "tc_ptx.cuh"
 
 namespace sem3d {
@@ -247,17 +248,16 @@ __device__ __forceinline__ void epilogue_chunk(const TcArgs& a, int row, int col
   }
   if (row >= a.rows) return;
   int i, j = 0;
-  uint32_t rowoff, cs;
+  uint32_t cs;
   if (PASS == 1) {  // row = i, column = j, batch = l
     i = row;
-    rowoff = (uint32_t)row + (uint32_t)a.Px * (uint32_t)a.ny * (uint32_t)batch;
     cs = (uint32_t)a.Px;
   } else {          // row = i + Px*j, column = l
     i = row % a.Px;
     j = row / a.Px;
-    rowoff = (uint32_t)row;
     cs = (uint32_t)a.Px * (uint32_t)a.ny;
   }
+  const size_t rowoff = tc_row_offset(PASS, row, batch, a.Px, a.ny);
   if (MODE == OUT_DIV_SPLIT) {
     const float li = __ldg(a.lamx + (i < a.nx ? i : 0)) + a.c;
     const float fixed = (PASS == 1) ? __ldg(a.lamz + batch) : __ldg(a.lamy + j);
