@@ -27,8 +27,6 @@
 // two-sum suffices (6 operations a term, n = 999 8.2 ms): its noise, relative to
 // the largest sum on the grid, is some 80 times the two-sum's and took the
 // normwise backward error of the refined solution from 2.5e-16 to 1.1e-15.
-#include <atomic>
-
 #include "sem3d_internal.h"
 
 namespace sem3d {
@@ -353,12 +351,12 @@ cudaError_t run_df(const DfArgs& a, const DfCoef<K>& cf, dim3 grid, cudaStream_t
   auto kern = stencil_df_kernel<K, EXACT, LO0>;
   constexpr int smem = DF_STAGES * DfTile<K>::stage_bytes(LO0);
   if (smem > 40 * 1024) {
-    static std::atomic<bool> set{false};
-    if (!set.load(std::memory_order_relaxed)) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-      set.store(true, std::memory_order_relaxed);
-    }
+    static PerDevice ready;
+    const cudaError_t e = on_device(ready, [&](int& set) {
+      set = 1;
+      return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    });
+    if (e != cudaSuccess) return e;
   }
   kern<<<grid, 256, smem, s>>>(a, cf);
   return cudaGetLastError();

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "../../include/sem3d.h"
+#include "per_device.h"
 
 namespace sem3d {
 
@@ -60,6 +61,16 @@ __device__ __forceinline__ float f64_to_f32_rn(double x) {
 // of short kernels: 63^3 refined 268 -> 204 us, FP64 315 -> 290.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// PerDevice::get on the current device (the one that the launch goes to).
+template <class Make>
+cudaError_t on_device(PerDevice& p, Make make, int* out = nullptr) {
+  int device = 0, value = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e == cudaSuccess) e = p.get(device, value, make);
+  if (out) *out = value;
+  return e;
+}
 
 inline cudaLaunchAttribute pdl_attribute() {
   cudaLaunchAttribute a;

@@ -340,33 +340,30 @@ template <int PASS, int MODE, int NP, int FMT = 0>
 cudaError_t launch_tc(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
                       const TcArgs& a, long long work_clusters, int num_sms, cudaStream_t s) {
   auto kern = mode_product_bf16x3_kernel<PASS, MODE, CLUSTER, NP, FMT>;
-  static std::atomic<int> max_clusters_cache{0};  // per instantiation: co-resident clusters of CLUSTER CTAs
-  int max_clusters = max_clusters_cache.load(std::memory_order_relaxed);
-  if (max_clusters == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(PASS));
-    if (e != cudaSuccess) return e;
-    if (CLUSTER > 1) {
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = CLUSTER;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.gridDim = dim3(CLUSTER * (num_sms / CLUSTER));
-      cfg.blockDim = dim3(num_threads(MODE));
-      cfg.dynamicSmemBytes = smem_bytes(PASS);
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      int n = 0;
-      e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-      if (e != cudaSuccess) return e;
-      if (n < 1) return cudaErrorInvalidConfiguration;
-      max_clusters = n;
-    } else {
-      max_clusters = num_sms;
+  static PerDevice resident;  // per instantiation: co-resident clusters of CLUSTER CTAs
+  int max_clusters = 0;
+  const cudaError_t e = on_device(resident, [&](int& n) {
+    cudaError_t q = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(PASS));
+    if (q != cudaSuccess) return q;
+    if (CLUSTER == 1) {
+      n = num_sms;
+      return cudaSuccess;
     }
-    max_clusters_cache.store(max_clusters, std::memory_order_relaxed);
-  }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CLUSTER;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(CLUSTER * (num_sms / CLUSTER));
+    cfg.blockDim = dim3(num_threads(MODE));
+    cfg.dynamicSmemBytes = smem_bytes(PASS);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    q = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    return q == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : q;
+  }, &max_clusters);
+  if (e != cudaSuccess) return e;
   const long long clusters = work_clusters < max_clusters ? work_clusters : max_clusters;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];

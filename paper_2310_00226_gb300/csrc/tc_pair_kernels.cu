@@ -6,7 +6,6 @@
 #include "tc_common.cuh"
 
 #include <algorithm>
-#include <atomic>
 
 namespace sem3d {
 
@@ -322,9 +321,9 @@ __global__ void __launch_bounds__(pair_threads(MODE), 1)
 
 // CTA-pair launch: clusters of 2, one pair per pair of SMs, persistent over
 // pair tiles.
-// `max_pairs`: the kernel's co-resident clusters of 2 CTAs, asked for once.
+// `resident`: the kernel's co-resident clusters of 2 CTAs, asked for once per device.
 template <class Kern, class... Args>
-cudaError_t launch_pairs(Kern kern, std::atomic<int>& max_pairs_cache, int pass, int mode, long long work_pairs,
+cudaError_t launch_pairs(Kern kern, PerDevice& resident, int pass, int mode, long long work_pairs,
                          int num_sms, cudaStream_t s, const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
@@ -336,18 +335,14 @@ cudaError_t launch_pairs(Kern kern, std::atomic<int>& max_pairs_cache, int pass,
   cfg.dynamicSmemBytes = pair_smem_bytes(pass, mode);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  int max_pairs = max_pairs_cache.load(std::memory_order_relaxed);
-  if (max_pairs == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pair_smem_bytes(pass, mode));
-    if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3(2 * (num_sms / 2));
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (n < 1) return cudaErrorInvalidConfiguration;
-    max_pairs = n;
-    max_pairs_cache.store(n, std::memory_order_relaxed);
-  }
+  int max_pairs = 0;
+  cfg.gridDim = dim3(2 * (num_sms / 2));
+  const cudaError_t e = on_device(resident, [&](int& n) {
+    cudaError_t q = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pair_smem_bytes(pass, mode));
+    if (q == cudaSuccess) q = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    return q == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : q;
+  }, &max_pairs);
+  if (e != cudaSuccess) return e;
   const long long pairs = work_pairs < max_pairs ? work_pairs : max_pairs;
   cfg.gridDim = dim3((unsigned)(2 * pairs));
   cfg.stream = s;
@@ -359,15 +354,15 @@ cudaError_t launch_pairs(Kern kern, std::atomic<int>& max_pairs_cache, int pass,
 template <int PASS, int MODE, int NP>
 cudaError_t launch_tc_pair(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
                            const TcArgs& a, long long work_pairs, int num_sms, cudaStream_t s) {
-  static std::atomic<int> max_pairs{0};
-  return launch_pairs(mode_product_bf16x3_pair_kernel<PASS, MODE, NP>, max_pairs, PASS, MODE, work_pairs, num_sms, s,
+  static PerDevice resident;
+  return launch_pairs(mode_product_bf16x3_pair_kernel<PASS, MODE, NP>, resident, PASS, MODE, work_pairs, num_sms, s,
                       a0, a1, b0, b1, a);
 }
 
 template <int PASS, int MODE>
 cudaError_t launch_fold_pass(const FoldPass& f, int total, int* err, int stall, int num_sms, cudaStream_t s) {
-  static std::atomic<int> max_pairs{0};
-  return launch_pairs(mode_product_fold_kernel<PASS, MODE>, max_pairs, PASS, MODE, total, num_sms, s, f, total, err,
+  static PerDevice resident;
+  return launch_pairs(mode_product_fold_kernel<PASS, MODE>, resident, PASS, MODE, total, num_sms, s, f, total, err,
                       stall);
 }
 
@@ -403,8 +398,8 @@ cudaError_t launch_tc_pair_mode(int mode, int nprod, const CUtensorMap& a0, cons
 template <int PASS, int MODE, int NP>
 cudaError_t launch_pair_group_t(const TcGroupEntry* tab, int count, int total, int* err, int stall, int num_sms,
                                 cudaStream_t s) {
-  static std::atomic<int> max_pairs{0};
-  return launch_pairs(mode_product_bf16x3_pair_group_kernel<PASS, MODE, NP>, max_pairs, PASS, MODE, total, num_sms, s,
+  static PerDevice resident;
+  return launch_pairs(mode_product_bf16x3_pair_group_kernel<PASS, MODE, NP>, resident, PASS, MODE, total, num_sms, s,
                       tab, count, total, err, stall);
 }
 

@@ -27,7 +27,6 @@
 #include "tc_ptx.cuh"
 
 #include <algorithm>
-#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -468,7 +467,7 @@ template <int MODE>
 cudaError_t launch_tf32(const CUtensorMap& mA, const CUtensorMap& mB, const Tf32Args& a, long long work_clusters,
                         int num_sms, cudaStream_t s) {
   auto kern = mode_product_tf32_kernel<MODE>;
-  static std::atomic<int> max_clusters_cache{0};  // co-resident clusters of this instantiation
+  static PerDevice resident;  // co-resident clusters of this instantiation
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -479,18 +478,14 @@ cudaError_t launch_tf32(const CUtensorMap& mA, const CUtensorMap& mB, const Tf32
   cfg.dynamicSmemBytes = T_SMEM;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  int max_clusters = max_clusters_cache.load(std::memory_order_relaxed);
-  if (max_clusters == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T_SMEM);
-    if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3(T_CL * (num_sms / T_CL));
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (n < 1) return cudaErrorInvalidConfiguration;
-    max_clusters = n;
-    max_clusters_cache.store(n, std::memory_order_relaxed);
-  }
+  int max_clusters = 0;
+  cfg.gridDim = dim3(T_CL * (num_sms / T_CL));
+  const cudaError_t e = on_device(resident, [&](int& n) {
+    cudaError_t q = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T_SMEM);
+    if (q == cudaSuccess) q = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    return q == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : q;
+  }, &max_clusters);
+  if (e != cudaSuccess) return e;
   const long long clusters = work_clusters < max_clusters ? work_clusters : max_clusters;
   cfg.gridDim = dim3((unsigned)(clusters * T_CL));
   cfg.stream = s;
@@ -501,7 +496,7 @@ template <int MODE>
 cudaError_t launch_tf32_pair(const CUtensorMap& mA, const CUtensorMap& mB, const Tf32Args& a, long long work_pairs,
                              int num_sms, cudaStream_t s) {
   auto kern = mode_product_tf32_pair_kernel<MODE>;
-  static std::atomic<int> max_pairs_cache{0};
+  static PerDevice resident;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -512,18 +507,14 @@ cudaError_t launch_tf32_pair(const CUtensorMap& mA, const CUtensorMap& mB, const
   cfg.dynamicSmemBytes = TP_SMEM;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  int max_pairs = max_pairs_cache.load(std::memory_order_relaxed);
-  if (max_pairs == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TP_SMEM);
-    if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3(2 * (num_sms / 2));
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (n < 1) return cudaErrorInvalidConfiguration;
-    max_pairs = n;
-    max_pairs_cache.store(n, std::memory_order_relaxed);
-  }
+  int max_pairs = 0;
+  cfg.gridDim = dim3(2 * (num_sms / 2));
+  const cudaError_t e = on_device(resident, [&](int& n) {
+    cudaError_t q = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TP_SMEM);
+    if (q == cudaSuccess) q = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    return q == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : q;
+  }, &max_pairs);
+  if (e != cudaSuccess) return e;
   const long long pairs = work_pairs < max_pairs ? work_pairs : max_pairs;
   cfg.gridDim = dim3((unsigned)(2 * pairs));
   cfg.stream = s;
