@@ -334,7 +334,10 @@ sem3d_status sem3d_profile_read(sem3d_handle h, int kind, long long* launches, d
  * pass along `axis` (0 = x, 1 = y, 2 = z).  sem3d_set_precision(h, SEM3D_FP32,
  * ...) measures six configurations of the FP32 CUDA-core kernel on each pass
  * shape of the plan that the process has not measured before (synchronous;
- * scratch buffers of up to 65536 * n floats twice) and keeps the fastest:
+ * scratch buffers of up to 65536 * n floats twice) and keeps the fastest, apart
+ * for parity blocks (two sweeps or more) and full matrices (fewer; also the
+ * Cahn-Hilliard step).  What is reported is the choice for the plan's sweeps;
+ * a form not measured yet takes the other's:
  *   0 = 128 x 128 output tile, 8 x 8 per thread, two shared-memory stages,
  *   1 = 128 x 64, 8 x 4, two stages,   2 = 64 x 64, 4 x 4, two stages,
  *   3..5 = the same three tiles with one stage.
@@ -342,8 +345,8 @@ sem3d_status sem3d_profile_read(sem3d_handle h, int kind, long long* launches, d
  * sem3d_solve_batched uses the two-stage tile of the same shape. */
 sem3d_status sem3d_tuned_config(sem3d_handle h, int axis, int* config);
 /* Pin `config` (0..5) for the pass shape of this plan's `axis`, replacing the
- * measured choice for every plan of the process with that pass shape (until
- * the next pin; sem3d_set_precision does not re-measure a known shape). */
+ * measured choices of both forms for every plan of the process with that pass
+ * shape (until the next pin; sem3d_set_precision does not re-measure a known shape). */
 sem3d_status sem3d_set_tuned_config(sem3d_handle h, int axis, int config);
 
 /* Tensor-core kernel of this plan's mode product along `axis` (0 = x, 1 = y,

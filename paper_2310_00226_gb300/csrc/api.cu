@@ -590,7 +590,7 @@ sem3d_status sem3d_set_precision(sem3d_handle h, sem3d_precision prec, int sweep
     if (major != 10 || minor != 3) return fail(SEM3D_ERR_UNSUPPORTED, "tensor-core tiers need an sm_103 GPU");
   }
   if (prec == SEM3D_FP32) {
-    const cudaError_t e = f32_autotune(h->g, h->dev);
+    const cudaError_t e = f32_autotune(h->g, h->dev, sweeps >= 2);  // as f32_parity will say
     if (e != cudaSuccess) return fail(SEM3D_ERR_CUDA, std::string("FP32 autotuning: ") + cudaGetErrorString(e));
   }
   if (prec == SEM3D_BF16X3 || prec == SEM3D_BF16) {
@@ -624,7 +624,7 @@ sem3d_status sem3d_set_tuned_config(sem3d_handle h, int axis, int config) {
 sem3d_status sem3d_tuned_config(sem3d_handle h, int axis, int* config) {
   if (!h || !config) return fail(SEM3D_ERR_INVALID_ARG, "NULL argument");
   if (axis < 0 || axis > 2) return fail(SEM3D_ERR_INVALID_ARG, "axis must be 0, 1 or 2");
-  *config = f32_config(axis, h->g);
+  *config = f32_config(axis, h->g, f32_parity(h));
   return SEM3D_OK;
 }
 

@@ -13,8 +13,8 @@
 // advances in chunks of 16 staged in shared memory, with one buffer (load,
 // sync, compute, sync) or two (the next chunk's global loads are in flight in
 // registers while the current chunk is multiplied).  Which of the
-// configurations runs is decided per pass shape by measuring them
-// (f32_autotune), since the best one depends on n and on the number of rows: a
+// configurations runs is decided per pass shape and form of W by measuring
+// them (f32_autotune), since the best one depends on n and on the number of rows: a
 // 63-wide output axis wastes half of a 128-wide tile, while large passes want
 // the larger register tiles.
 //
@@ -421,21 +421,27 @@ cudaError_t dispatch_f32(bool in_f64, bool out_f64, int mode, Run run) {
 }
 
 // ---------------------------------------------------------------- autotuner
-// Pass shape -> configuration, filled by f32_autotune from measurements.
-// Rows are capped at the tuning size: beyond a few waves of tiles the ranking
-// no longer changes with the row count.
+// Pass shape and form (full matrices or parity blocks) -> configuration, filled
+// by f32_autotune from measurements.  Each form is measured for itself: the
+// tiles of the blocks hold half the outputs of either parity, and a choice
+// made for one costs the other up to 45% (63x255x127 bare: 244 us with the
+// blocks' choice, 169 with its own; 127^3 194 and 145).  Rows are capped at the
+// tuning size: beyond a few waves of tiles the ranking no longer changes with
+// the row count.
 constexpr long long TUNE_ROWS = 65536;
-using TuneKey = std::tuple<int, int, long long>;  // (K contiguous, n, min(rows, TUNE_ROWS))
+using TuneKey = std::tuple<int, int, long long, int>;  // (K contiguous, n, min(rows, TUNE_ROWS), parity)
 std::mutex g_tune_mu;
 std::map<TuneKey, int> g_tune;
 
-TuneKey tune_key(bool kcontig, int n, long long rows) {
-  return TuneKey{kcontig ? 1 : 0, n, rows < TUNE_ROWS ? rows : TUNE_ROWS};
+TuneKey tune_key(bool kcontig, int n, long long rows, bool parity) {
+  return TuneKey{kcontig ? 1 : 0, n, rows < TUNE_ROWS ? rows : TUNE_ROWS, parity ? 1 : 0};
 }
 
-int tuned_cfg(bool kcontig, int n, long long rows) {
+// A form that has not been measured takes the other's choice.
+int tuned_cfg(bool kcontig, int n, long long rows, bool parity) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  auto it = g_tune.find(tune_key(kcontig, n, rows));
+  auto it = g_tune.find(tune_key(kcontig, n, rows, parity));
+  if (it == g_tune.end()) it = g_tune.find(tune_key(kcontig, n, rows, !parity));
   return it == g_tune.end() ? 0 : it->second;
 }
 
@@ -465,7 +471,7 @@ F32Pass make_pass(const Geom& g, int axis, const DevAxis* ax, int which, bool pa
   } else {
     p.R1 = (int)nxy; p.R2 = 1; p.s1 = 1; p.s2 = 0; p.sm = nxy;
   }
-  p.cfg = tuned_cfg(*kcontig, p.n, (long long)p.R1 * p.R2);
+  p.cfg = tuned_cfg(*kcontig, p.n, (long long)p.R1 * p.R2, parity);
   return p;
 }
 
@@ -476,10 +482,10 @@ bool epi_ok(int axis, int epi, bool out_f64) {
 
 }  // namespace
 
-cudaError_t f32_autotune(const Geom& g, const DevAxis* ax) {
+cudaError_t f32_autotune(const Geom& g, const DevAxis* ax, bool parity) {
   // The three pass shapes of this grid, each timed on a synthetic forward pass
-  // by parity blocks with the same K extent, output length and access pattern
-  // and min(rows, TUNE_ROWS) rows, on scratch buffers of this device.
+  // of the form asked for with the same K extent, output length and access
+  // pattern and min(rows, TUNE_ROWS) rows, on scratch buffers of this device.
   struct Shape { bool kcontig; int n; long long rows; };
   const Shape shapes[3] = {{true, g.nx, (long long)g.ny * g.nz},
                            {false, g.ny, (long long)g.nx * g.nz},
@@ -488,7 +494,7 @@ cudaError_t f32_autotune(const Geom& g, const DevAxis* ax) {
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     for (int a = 0; a < 3; ++a)
-      if (!g_tune.count(tune_key(shapes[a].kcontig, shapes[a].n, shapes[a].rows))) todo.push_back(a);
+      if (!g_tune.count(tune_key(shapes[a].kcontig, shapes[a].n, shapes[a].rows, parity))) todo.push_back(a);
   }
   if (todo.empty()) return cudaSuccess;
   size_t need = 0;
@@ -509,18 +515,21 @@ cudaError_t f32_autotune(const Geom& g, const DevAxis* ax) {
     const Shape& sh = shapes[todo[q]];
     const long long r = sh.rows < TUNE_ROWS ? sh.rows : TUNE_ROWS;
     F32Pass p{};
-    p.in = in; p.out = out; p.W = ax[todo[q]].Wpf[0]; p.epi = EPI_STORE; p.n = sh.n;
+    p.in = in; p.out = out; p.W = parity ? ax[todo[q]].Wpf[0] : ax[todo[q]].Wf[0]; p.epi = EPI_STORE; p.n = sh.n;
     p.ne = ax[todo[q]].ne; p.no = ax[todo[q]].no;
     p.R1 = (int)r; p.R2 = 1; p.s2 = 0;
     if (sh.kcontig) { p.s1 = sh.n; p.sm = 1; }
     else { p.s1 = 1; p.sm = r; }
     int best = 0;
     float best_ms = 0.f;
+    auto pass = [&] {
+      return parity ? launch_f32<float, float, W_FWD>(p, sh.kcontig, s) : launch_f32<float, float, W_FULL>(p, sh.kcontig, s);
+    };
     for (int c = 0; c < F32_NCFG && err == cudaSuccess; ++c) {
       p.cfg = c;
-      err = launch_f32<float, float, W_FWD>(p, sh.kcontig, s);  // warm-up
+      err = pass();  // warm-up
       if (err == cudaSuccess) err = cudaEventRecord(e0, s);
-      for (int rep = 0; rep < 3 && err == cudaSuccess; ++rep) err = launch_f32<float, float, W_FWD>(p, sh.kcontig, s);
+      for (int rep = 0; rep < 3 && err == cudaSuccess; ++rep) err = pass();
       if (err == cudaSuccess) err = cudaEventRecord(e1, s);
       if (err == cudaSuccess) err = cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -529,7 +538,7 @@ cudaError_t f32_autotune(const Geom& g, const DevAxis* ax) {
     }
     if (err == cudaSuccess) {
       std::lock_guard<std::mutex> lk(g_tune_mu);
-      g_tune[tune_key(sh.kcontig, sh.n, sh.rows)] = best;
+      g_tune[tune_key(sh.kcontig, sh.n, sh.rows, parity)] = best;
     }
   }
   if (e0) cudaEventDestroy(e0);
@@ -545,13 +554,13 @@ void f32_set_config(int axis, const Geom& g, int cfg) {
   const int n = axis == 0 ? g.nx : (axis == 1 ? g.ny : g.nz);
   const long long rows = axis == 0 ? (long long)g.ny * g.nz : (axis == 1 ? (long long)g.nx * g.nz : (long long)g.nx * g.ny);
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tune[tune_key(kc, n, rows)] = cfg;
+  for (bool parity : {false, true}) g_tune[tune_key(kc, n, rows, parity)] = cfg;
 }
 
-int f32_config(int axis, const Geom& g) {
-  if (axis == 0) return tuned_cfg(true, g.nx, (long long)g.ny * g.nz);
-  if (axis == 1) return tuned_cfg(false, g.ny, (long long)g.nx * g.nz);
-  return tuned_cfg(false, g.nz, (long long)g.nx * g.ny);
+int f32_config(int axis, const Geom& g, bool parity) {
+  if (axis == 0) return tuned_cfg(true, g.nx, (long long)g.ny * g.nz, parity);
+  if (axis == 1) return tuned_cfg(false, g.ny, (long long)g.nx * g.nz, parity);
+  return tuned_cfg(false, g.nz, (long long)g.nx * g.ny, parity);
 }
 
 cudaError_t launch_mode_product_f32_grouped(int count, const Geom* geoms, int axis, const DevAxis* const* ax, int which,
