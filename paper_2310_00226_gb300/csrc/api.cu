@@ -289,7 +289,7 @@ sem3d_status solve_once_f64(sem3d_plan* p, const double* in, double* out, bool a
   double* B = reinterpret_cast<double*>(static_cast<char*>(p->ws) + align256(N * sizeof(double)));
   const Geom& g = p->g;
   const DevAxis* d = p->dev;
-  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 2, d, 0, in, A, EPI_STORE, p->num_sms, s));
+  LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 2, d, 0, in, A, EPI_HALF, p->num_sms, s));
   LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 1, d, 0, A, B, EPI_STORE, p->num_sms, s));
   LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 0, d, 0, B, A, EPI_DIV, p->num_sms, s));
   LAUNCH(p, K_F64, 1, s, launch_mode_product_f64(g, 2, d, 1, A, B, EPI_STORE, p->num_sms, s));
@@ -451,11 +451,9 @@ sem3d_status solve_once_fold(sem3d_plan* p, const FoldBuffers& b, cudaStream_t s
 int df_sweeps(const sem3d_plan* h);                // double-FP32 sweeps of a split-tier solve (defined below)
 bool use_fixed_residual(const sem3d_plan* h);      // FP64-accurate residuals in fixed point (defined below)
 
-// f -> S0, with f's exponent for the fixed-point residuals.
+// f -> S0, with f's exponent for the scale of the passes and the fixed-point residuals.
 sem3d_status fold_rhs(sem3d_plan* h, const FoldBuffers& b, const double* f, cudaStream_t s) {
-  const bool fixed = use_fixed_residual(h);
-  if (fixed) CUDA_TRY(cudaMemsetAsync(h->d_fix + 1, 0, sizeof(int), s));
-  LAUNCH(h, K_SPLIT, 1, s, launch_fold(b.g, f, nullptr, h->g.nx, b.S0, fixed ? h->d_fix + 1 : nullptr, s));
+  LAUNCH(h, K_SPLIT, 2, s, launch_fold(b.g, f, nullptr, h->g.nx, b.S0, h->d_fix + 1, h->num_sms, s));
   return SEM3D_OK;
 }
 
@@ -470,7 +468,8 @@ sem3d_status fold_update(sem3d_plan* h, const FoldBuffers& b, double* u, int sw,
   const DfBuffers D{b.D.hi, epi == EPI_DF_STORE ? nullptr : b.D.lo};
   const bool emax = !in_df && sw < h->sweeps && use_fixed_residual(h);  // a fixed-point residual of u follows
   if (emax) CUDA_TRY(cudaMemsetAsync(h->d_fix, 0, sizeof(int), s));
-  LAUNCH(h, K_SPLIT, 1, s, launch_unfold(b.g, b.delta, epi, sw == 1, u, D, h->g.Px, emax ? h->d_fix : nullptr, s));
+  LAUNCH(h, K_SPLIT, 1, s, launch_unfold(b.g, b.delta, epi, sw == 1, u, D, h->g.Px, h->d_fix + 1,
+                                         emax ? h->d_fix : nullptr, s));
   return SEM3D_OK;
 }
 
@@ -489,7 +488,7 @@ sem3d_status fold_residual(sem3d_plan* h, const FoldBuffers& b, const double* f,
   } else {
     LAUNCH(h, K_STENCIL, 1, s, launch_stencil_f32out(h->g, h->k, h->dev, u, f, b.r32, nullptr, s));
   }
-  LAUNCH(h, K_SPLIT, 1, s, launch_fold(b.g, nullptr, b.r32, h->g.Px, b.S0, nullptr, s));
+  LAUNCH(h, K_SPLIT, 1, s, launch_fold(b.g, nullptr, b.r32, h->g.Px, b.S0, h->d_fix + 1, h->num_sms, s));
   return SEM3D_OK;
 }
 
@@ -1734,7 +1733,7 @@ sem3d_status solve_once_f64_into(sem3d_plan* p, const double* in, double* out, b
                                  cudaStream_t s) {
   const Geom& g = p->g;
   const DevAxis* d = p->dev;
-  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 2, d, 0, in, A, EPI_STORE, p->num_sms, s));
+  LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 2, d, 0, in, A, EPI_HALF, p->num_sms, s));
   LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 1, d, 0, A, B, EPI_STORE, p->num_sms, s));
   LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 0, d, 0, B, A, EPI_DIV, p->num_sms, s));
   LAUNCH_COUNTED(p, 1, launch_mode_product_f64(g, 2, d, 1, A, B, EPI_STORE, p->num_sms, s));

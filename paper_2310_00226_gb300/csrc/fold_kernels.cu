@@ -11,10 +11,18 @@
 //            added to the solution at the 8 mirror images of a node.
 // A thread takes the 8 mirror images of one node (fold: of two neighbours, so
 // that the bf16 outputs go out in pairs).  Every stream is read and written in
-// runs of whole lines, forwards or backwards, and both kernels are bound by
+// runs of whole lines, forwards or backwards.  A sum of 8 values may exceed
+// FP32's range where the values do not: right-hand sides from 2^110 on, found by
+// the exponent that the fold records, are folded again at 2^-8, their residuals
+// and corrections scaled to match (powers of two: the same digits).  (Folding
+// everything at 1/8 would cost the other end of the range: the low bf16 part of
+// values below 1e-25.)  For all others that is one launch, 3 us, whose blocks
+// return at once.  Both kernels are bound by
 // HBM: at n = 999 fold 1.9 ms from FP64 (12 B per node, 6.3 TB/s) and 1.13 ms
 // from FP32, unfold 2.85 ms into FP64 and 2.9 ms into the double-FP32 pair
 // (20 B, 7 TB/s), 3.9 ms from the pair into FP64.
+#include <algorithm>
+
 #include "tc_common.cuh"
 
 namespace sem3d {
@@ -44,69 +52,90 @@ __device__ __forceinline__ unsigned int exp_of(double x) {
 }
 __device__ __forceinline__ unsigned int exp_of(float) { return 0; }
 
-template <typename TIN, bool EMAX>
-__global__ void __launch_bounds__(256) fold_split_kernel(const TIN* __restrict__ in, int pitch,
-                                                         __nv_bfloat16* __restrict__ hi,
-                                                         __nv_bfloat16* __restrict__ lo, FoldGeom g, int* emax) {
+// Right-hand sides whose largest biased FP64 exponent is at least this are scaled.
+constexpr int kFoldBig = 1023 + 110;
+constexpr float kFoldDown = 1.f / 256, kFoldUp = 256.f;
+
+// FOLD_F: f, its largest exponent to *fexp; FOLD_BIG: f at kFoldDown if its
+// exponent calls for it (else nothing); FOLD_R: a residual, scaled as f was.
+enum : int { FOLD_F, FOLD_BIG, FOLD_R };
+
+template <int WHAT, typename TIN>
+__device__ __forceinline__ void fold_nodes(const TIN* __restrict__ in, int pitch, __nv_bfloat16* __restrict__ hi,
+                                           __nv_bfloat16* __restrict__ lo, const FoldGeom& g, long long idx, float sc,
+                                           unsigned int& m) {
   const unsigned int cp = (unsigned int)g.Pe >> 1;
-  const long long total = (long long)cp * g.ne[1] * g.ne[2];
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned int m = 0;
-  if (idx < total) {
-    const int c = (int)(idx % cp);
-    const long long jl = idx / cp;
-    const int j = (int)(jl % g.ne[1]), l = (int)(jl / g.ne[1]);
-    const bool my = j < g.no[1], mz = l < g.no[2];  // has a mirror image along y / z
-    const int i0 = 2 * c;
-    // the lines (j,l), (j',l), (j,l'), (j',l'): values at i and at its mirror
-    // image (all loads issued before the conversions), then x-even / x-odd parts
-    TIN ra[4][2], rb[4][2];
-    float e[4][2], o[4][2];
+  const int c = (int)(idx % cp);
+  const long long jl = idx / cp;
+  const int j = (int)(jl % g.ne[1]), l = (int)(jl / g.ne[1]);
+  const bool my = j < g.no[1], mz = l < g.no[2];  // has a mirror image along y / z
+  const int i0 = 2 * c;
+  // the lines (j,l), (j',l), (j,l'), (j',l'): values at i and at its mirror
+  // image (all loads issued before the conversions), then x-even / x-odd parts
+  TIN ra[4][2], rb[4][2];
+  float e[4][2], o[4][2];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const bool ok = (!(q & 1) || my) && (!(q & 2) || mz);
-      const int jq = (q & 1) ? g.ny - 1 - j : j, lq = (q & 2) ? g.nz - 1 - l : l;
-      const TIN* row = in + ((long long)lq * g.ny + jq) * pitch;
+  for (int q = 0; q < 4; ++q) {
+    const bool ok = (!(q & 1) || my) && (!(q & 2) || mz);
+    const int jq = (q & 1) ? g.ny - 1 - j : j, lq = (q & 2) ? g.nz - 1 - l : l;
+    const TIN* row = in + ((long long)lq * g.ny + jq) * pitch;
 #pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const int i = i0 + p;
-        ra[q][p] = (ok && i < g.ne[0]) ? __ldg(row + i) : TIN(0);
-        rb[q][p] = (ok && i < g.no[0]) ? __ldg(row + g.nx - 1 - i) : TIN(0);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        if (EMAX) m = max(m, max(exp_of(ra[q][p]), exp_of(rb[q][p])));
-        const float a = to_f32(ra[q][p]), b = to_f32(rb[q][p]);
-        e[q][p] = a + b;
-        o[q][p] = i0 + p < g.no[0] ? a - b : 0.f;
-      }
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      if (x == 1 && i0 >= g.Po) break;
-      float v[4][2];  // (y even, z even), (y odd, z even), (y even, z odd), (y odd, z odd)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const float a0 = x ? o[0][p] : e[0][p], a1 = x ? o[1][p] : e[1][p];
-        const float a2 = x ? o[2][p] : e[2][p], a3 = x ? o[3][p] : e[3][p];
-        const float s0 = a0 + a1, d0 = a0 - a1, s1 = a2 + a3, d1 = a2 - a3;
-        v[0][p] = s0 + s1; v[1][p] = d0 + d1; v[2][p] = s0 - s1; v[3][p] = d0 - d1;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (((q & 1) && !my) || ((q & 2) && !mz)) continue;
-        const long long row = (long long)((q & 2) ? g.ne[2] + l : l) * g.ny + ((q & 1) ? g.ne[1] + j : j);
-        const long long at = row * g.Px + (x ? g.Pe : 0) + i0;
-        uint32_t h, w;
-        split_pair(v[q][0], v[q][1], h, w);
-        *reinterpret_cast<uint32_t*>(hi + at) = h;
-        *reinterpret_cast<uint32_t*>(lo + at) = w;
-      }
+    for (int p = 0; p < 2; ++p) {
+      const int i = i0 + p;
+      ra[q][p] = (ok && i < g.ne[0]) ? __ldg(row + i) : TIN(0);
+      rb[q][p] = (ok && i < g.no[0]) ? __ldg(row + g.nx - 1 - i) : TIN(0);
     }
   }
-  if (EMAX) block_max_exp(m, emax);
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      if (WHAT == FOLD_F) m = max(m, max(exp_of(ra[q][p]), exp_of(rb[q][p])));
+      float a = to_f32(ra[q][p]), b = to_f32(rb[q][p]);
+      if (WHAT != FOLD_F) { a *= sc; b *= sc; }
+      e[q][p] = a + b;
+      o[q][p] = i0 + p < g.no[0] ? a - b : 0.f;
+    }
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    if (x == 1 && i0 >= g.Po) break;
+    float v[4][2];  // (y even, z even), (y odd, z even), (y even, z odd), (y odd, z odd)
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const float a0 = x ? o[0][p] : e[0][p], a1 = x ? o[1][p] : e[1][p];
+      const float a2 = x ? o[2][p] : e[2][p], a3 = x ? o[3][p] : e[3][p];
+      const float s0 = a0 + a1, d0 = a0 - a1, s1 = a2 + a3, d1 = a2 - a3;
+      v[0][p] = s0 + s1; v[1][p] = d0 + d1; v[2][p] = s0 - s1; v[3][p] = d0 - d1;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (((q & 1) && !my) || ((q & 2) && !mz)) continue;
+      const long long row = (long long)((q & 2) ? g.ne[2] + l : l) * g.ny + ((q & 1) ? g.ne[1] + j : j);
+      const long long at = row * g.Px + (x ? g.Pe : 0) + i0;
+      uint32_t h, w;
+      split_pair(v[q][0], v[q][1], h, w);
+      *reinterpret_cast<uint32_t*>(hi + at) = h;
+      *reinterpret_cast<uint32_t*>(lo + at) = w;
+    }
+  }
+}
+
+template <int WHAT, typename TIN>
+__global__ void __launch_bounds__(256) fold_split_kernel(const TIN* __restrict__ in, int pitch,
+                                                         __nv_bfloat16* __restrict__ hi,
+                                                         __nv_bfloat16* __restrict__ lo, FoldGeom g, int* fexp) {
+  const long long total = (long long)((unsigned int)g.Pe >> 1) * g.ne[1] * g.ne[2];
+  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned int m = 0;
+  if (WHAT == FOLD_BIG) {  // a few blocks
+    if (*fexp < kFoldBig) return;
+    for (; idx < total; idx += (long long)gridDim.x * blockDim.x)
+      fold_nodes<WHAT>(in, pitch, hi, lo, g, idx, kFoldDown, m);
+  } else {
+    const float sc = WHAT == FOLD_R && __ldg(fexp) >= kFoldBig ? kFoldDown : 1.f;
+    if (idx < total) fold_nodes<WHAT>(in, pitch, hi, lo, g, idx, sc, m);
+    if (WHAT == FOLD_F) block_max_exp(m, fexp);
+  }
 }
 
 // What the correction is added to.  DF_*: the solution as a double-FP32 pair
@@ -115,9 +144,12 @@ enum : int { UP_F64 = 0, UP_F64_ACC, UP_DF, UP_DF_ACC, UP_DF_ACC_LOZ, UP_DF_F64,
 
 template <int MODE>
 __global__ void __launch_bounds__(256) unfold_update_kernel(const float* __restrict__ delta, FoldGeom g, double* u,
-                                                            float* dhi, float* dlo, int PxDf, int* emax) {
+                                                            float* dhi, float* dlo, int PxDf,
+                                                            const int* __restrict__ fexp,
+                                                            int* emax) {
   constexpr bool df = MODE >= UP_DF, reads = MODE != UP_F64 && MODE != UP_DF;
   constexpr bool loz = MODE == UP_DF_ACC_LOZ || MODE == UP_DF_F64_LOZ;
+  const float up = __ldg(fexp) >= kFoldBig ? kFoldUp : 1.f;
   const long long total = (long long)g.Pe * g.ne[1] * g.ne[2];
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned int m = 0;
@@ -163,6 +195,7 @@ __global__ void __launch_bounds__(256) unfold_update_kernel(const float* __restr
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       if (!ok[q]) continue;
+      v[q] *= up;  // here, where the reads above are on their way
       const int at = (q & 1) ? g.nx - 1 - i : i;
       const long long d = line[q >> 1] * PxDf + at, w = line[q >> 1] * g.nx + at;
       if (MODE == UP_F64 || MODE == UP_F64_ACC) {
@@ -217,23 +250,28 @@ FoldGeom fold_geom(const Geom& g) {
   return f;
 }
 
-cudaError_t launch_fold(const FoldGeom& g, const double* f64, const float* f32, int pitch, TcBuffers out, int* emax,
-                        cudaStream_t s) {
+cudaError_t launch_fold(const FoldGeom& g, const double* f64, const float* f32, int pitch, TcBuffers out, int* fexp,
+                        int num_sms, cudaStream_t s) {
   const long long total = (long long)(g.Pe / 2) * g.ne[1] * g.ne[2], blocks = (total + 255) / 256;
   if (blocks >= (1LL << 31)) return cudaErrorInvalidValue;
-  const unsigned b = (unsigned)blocks;
-  if (f32) fold_split_kernel<float, false><<<b, 256, 0, s>>>(f32, pitch, out.hi, out.lo, g, nullptr);
-  else if (emax) fold_split_kernel<double, true><<<b, 256, 0, s>>>(f64, pitch, out.hi, out.lo, g, emax);
-  else fold_split_kernel<double, false><<<b, 256, 0, s>>>(f64, pitch, out.hi, out.lo, g, nullptr);
+  const unsigned b = (unsigned)blocks, few = (unsigned)std::min<long long>(blocks, 8LL * num_sms);
+  if (f32) {
+    fold_split_kernel<FOLD_R><<<b, 256, 0, s>>>(f32, pitch, out.hi, out.lo, g, fexp);
+    return cudaGetLastError();
+  }
+  const cudaError_t e = cudaMemsetAsync(fexp, 0, sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  fold_split_kernel<FOLD_F><<<b, 256, 0, s>>>(f64, pitch, out.hi, out.lo, g, fexp);
+  fold_split_kernel<FOLD_BIG><<<few, 256, 0, s>>>(f64, pitch, out.hi, out.lo, g, fexp);
   return cudaGetLastError();
 }
 
 cudaError_t launch_unfold(const FoldGeom& g, const float* delta, int epi, bool lo_zero, double* u, DfBuffers df,
-                          int PxDf, int* emax, cudaStream_t s) {
+                          int PxDf, const int* fexp, int* emax, cudaStream_t s) {
   const long long total = (long long)g.Pe * g.ne[1] * g.ne[2], blocks = (total + 255) / 256;
   if (blocks >= (1LL << 31)) return cudaErrorInvalidValue;
   const unsigned b = (unsigned)blocks;
-  auto run = [&](auto kern) { kern<<<b, 256, 0, s>>>(delta, g, u, df.hi, df.lo, PxDf, emax); };
+  auto run = [&](auto kern) { kern<<<b, 256, 0, s>>>(delta, g, u, df.hi, df.lo, PxDf, fexp, emax); };
   switch (epi) {
     case EPI_STORE: run(unfold_update_kernel<UP_F64>); break;
     case EPI_ACCUM: run(unfold_update_kernel<UP_F64_ACC>); break;

@@ -178,6 +178,10 @@ __device__ __forceinline__ void f32_tile(const F32Pass& p, long long bx, int by,
       float u = to_f32(ra[it][0]);
       if constexpr (MODE != W_FULL) {
         float v = to_f32(ra[it][NP - 1]);
+        if (sizeof(TIN) == 8) {  // a right-hand side: halved, so that no sum of a mirrored pair overflows
+          u *= 0.5f;
+          v *= 0.5f;
+        }
         if (MODE == W_FWD) {
           const float d = t0 + kk < p.no ? u - v : 0.f;
           u = u + v;
@@ -283,8 +287,9 @@ __device__ __forceinline__ void f32_tile(const F32Pass& p, long long bx, int by,
             v[NP - 1][c] = e - d;
           } else if (KCONTIG && p.epi == EPI_DIV) {
             const double d = ly + lz + p.c;
-            if (o < p.ne) v[0][c] = v[0][c] / f64_to_f32_rn(p.lamx[o] + d);
-            if (pair) v[NP - 1][c] = v[NP - 1][c] / f64_to_f32_rn(p.lamx[p.ne + o] + d);
+            // of halved right-hand sides
+            if (o < p.ne) v[0][c] = v[0][c] / (0.5f * f64_to_f32_rn(p.lamx[o] + d));
+            if (pair) v[NP - 1][c] = v[NP - 1][c] / (0.5f * f64_to_f32_rn(p.lamx[p.ne + o] + d));
           }
         }
       }

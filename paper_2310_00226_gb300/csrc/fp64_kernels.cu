@@ -40,7 +40,18 @@ struct F64Pass {
   double c;
 };
 
-template <bool KCONTIG, bool FWD, int BM>
+// Half of x off the FP64 pipe and without a branch (one would keep the loads
+// from staying in flight): one off the exponent; below 2^-1021 the magnitude's
+// bits shifted, the last one dropped; infinities and NaN as they are.
+__device__ __forceinline__ double half_of(double x) {
+  const unsigned int h = (unsigned int)__double2hiint(x), w = (unsigned int)__double2loint(x);
+  const unsigned int m = h & 0x7FFFFFFFu, sign = h & 0x80000000u;
+  const bool tiny = m < 0x00200000u;
+  const unsigned int hi = tiny ? m >> 1 : m < 0x7FF00000u ? m - 0x00100000u : m;
+  return __hiloint2double((int)(sign | hi), (int)(tiny ? __funnelshift_r(w, m, 1) : w));
+}
+
+template <bool KCONTIG, bool FWD, bool HALF, int BM>
 __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
   constexpr int AF = BM / 16;                    // fragments of 8 rows per warp
   constexpr int LA = BM * F64_BK / 256;          // (even, odd) A pairs loaded per thread and chunk
@@ -73,6 +84,7 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
       if (abase[it] && t < p.ne) {
         u = abase[it][(long long)t * p.sm];
         if (t < p.no) v = abase[it][(long long)(FWD ? p.n - 1 - t : p.ne + t) * p.sm];
+        if (HALF) { u = half_of(u); v = half_of(v); }  // no sum of a mirrored pair overflows
       }
       // the middle node of an odd n (t = no) has no partner: v = 0 and the
       // odd block has no such column
@@ -137,7 +149,7 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
     if (p.epi == EPI_DIV) {
       const long long i = idx % p.nx, jl = idx / p.nx;
       const long long j = jl % p.ny, l = jl / p.ny;
-      p.out[idx] = v / (p.lamx[i] + p.lamy[j] + p.lamz[l] + p.c);
+      p.out[idx] = v / half_of(p.lamx[i] + p.lamy[j] + p.lamz[l] + p.c);  // of halved right-hand sides
     } else if (p.epi == EPI_ACCUM) {
       p.out[idx] += v;
     } else {
@@ -167,7 +179,7 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
   }
 }
 
-template <bool KCONTIG, bool FWD>
+template <bool KCONTIG, bool FWD, bool HALF = false>
 cudaError_t launch_f64(const F64Pass& p, int num_sms, cudaStream_t s) {
   // Rows per CTA: the CTAs of an SM share its FP64 pipe, so a pass takes as
   // long as the SM with the most rows; the largest tile within that minimum.
@@ -184,9 +196,9 @@ cudaError_t launch_f64(const F64Pass& p, int num_sms, cudaStream_t s) {
   const long long bx = (rows + best - 1) / best;
   if (bx >= (1LL << 31)) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)bx, (unsigned)nt);
-  if (best == 64) return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, 64>, grid, dim3(256), 0, s, p);
-  if (best == 32) return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, 32>, grid, dim3(256), 0, s, p);
-  return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, 16>, grid, dim3(256), 0, s, p);
+  if (best == 64) return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, HALF, 64>, grid, dim3(256), 0, s, p);
+  if (best == 32) return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, HALF, 32>, grid, dim3(256), 0, s, p);
+  return launch_pdl(mode_product_f64_kernel<KCONTIG, FWD, HALF, 16>, grid, dim3(256), 0, s, p);
 }
 
 // ------------------------------------------------------------------ stencil
@@ -505,6 +517,10 @@ cudaError_t launch_mode_product_f64(const Geom& g, int axis, const DevAxis* ax, 
     p.R1 = g.nx; p.R2 = g.nz; p.s1 = 1; p.s2 = nxy; p.sm = g.nx;
   } else {                 // rows = (i,j) plane, t = l
     p.R1 = (int)nxy; p.R2 = 1; p.s1 = 1; p.s2 = 0; p.sm = nxy;
+  }
+  if (epi == EPI_HALF) {  // the first pass of a solve
+    if (kcontig || which != 0) return cudaErrorInvalidValue;
+    return launch_f64<false, true, true>(p, num_sms, s);
   }
   if (which == 0) return kcontig ? launch_f64<true, true>(p, num_sms, s) : launch_f64<false, true>(p, num_sms, s);
   return kcontig ? launch_f64<true, false>(p, num_sms, s) : launch_f64<false, false>(p, num_sms, s);

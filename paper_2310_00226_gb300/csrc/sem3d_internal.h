@@ -206,7 +206,8 @@ enum Epi : int {
   EPI_ACCUM = 2,       // out += acc (FP64 outputs only)
   EPI_DF_STORE = 3,    // double-FP32 solution (hi, lo) = (acc, 0)            [z pass]
   EPI_DF_ACCUM = 4,    // (hi, lo) += acc                                     [z pass]
-  EPI_DF_ACCUM_F64 = 5 // FP64 out = (hi, lo) + acc                           [z pass]
+  EPI_DF_ACCUM_F64 = 5, // FP64 out = (hi, lo) + acc                          [z pass]
+  EPI_HALF = 6          // the input at half its value (see launch_mode_product_f64)
 };
 
 // Power-of-two scaling of the fp16 split arrays of the F16X3 tier, kept on
@@ -261,13 +262,17 @@ FoldGeom fold_geom(const Geom& g);
 // arrays with the parity blocks of T^{-1} (which = 0: nodes -> modes, even
 // modes first) or T (which = 1: modes -> nodes).  EPI_DIV divides by
 // lam_x + lam_y + lam_z + c, all three axes being in mode order.
+// A solve halves its right-hand side in the first pass (EPI_HALF) and its
+// division pass doubles: the sums of two mirrored values that the forward
+// passes form then stay in range wherever the values do, with the same digits.
 cudaError_t launch_mode_product_f64(const Geom& g, int axis, const DevAxis* ax, int which, const double* in,
                                     double* out, int epi, int num_sms, cudaStream_t s);
 // ---- FP32 CUDA-core kernels (fp32_kernels.cu)
 // One mode product in FP32 arithmetic with T^{-1} (which = 0) or T; `in` is
 // FP64 (first pass) or FP32, `out` FP64 (last pass, EPI_STORE or EPI_ACCUM) or
 // FP32; EPI_DIV in the x pass.  parity: by the parity blocks (modes, and the
-// eigenvalues of EPI_DIV, in mode order), else by the full matrices.
+// eigenvalues of EPI_DIV, in mode order), else by the full matrices.  With
+// parity, FP64 input is halved and EPI_DIV doubles (as in FP64, above).
 cudaError_t launch_mode_product_f32(const Geom& g, int axis, const DevAxis* ax, int which, bool parity, const void* in,
                                     bool in_f64, void* out, bool out_f64, int epi, cudaStream_t s);
 // Measure the FP32 kernel configurations on the three pass shapes of grid g, by
@@ -371,18 +376,20 @@ struct TcBuffers {
   __nv_bfloat16* lo;
 };
 // ---- parity form of the split arrays (fold_kernels.cu)
-// Right-hand side in node order (f64, pitch nx; or f32, rows of `pitch`) ->
-// split array in parity order.  emax (f64 only): as launch_split's.
-cudaError_t launch_fold(const FoldGeom& g, const double* f64, const float* f32, int pitch, TcBuffers out, int* emax,
-                        cudaStream_t s);
+// Right-hand side in node order -> split array in parity order: f64 (pitch nx;
+// two launches), whose largest biased exponent goes to *fexp and decides the
+// scale of the parity-order arrays until the next one; or f32, a residual (rows
+// of `pitch`; one launch) at that scale.
+cudaError_t launch_fold(const FoldGeom& g, const double* f64, const float* f32, int pitch, TcBuffers out, int* fexp,
+                        int num_sms, cudaStream_t s);
 // Add the correction delta (FP32, parity order) to the solution, as `epi`
 // says: EPI_STORE / EPI_ACCUM u, EPI_DF_STORE / EPI_DF_ACCUM the double-FP32
 // pair df (pitch PxDf; df.lo may be null for the store: then it is not
 // written, and the next update has to be told lo_zero), EPI_DF_ACCUM_F64 u
-// from the pair.  lo_zero: the pair's low parts are zero (not read).  emax: as
-// launch_split's, of the u written.
+// from the pair.  lo_zero: the pair's low parts are zero (not read).  fexp:
+// launch_fold's.  emax: as launch_split's, of the u written.
 cudaError_t launch_unfold(const FoldGeom& g, const float* delta, int epi, bool lo_zero, double* u, DfBuffers df,
-                          int PxDf, int* emax, cudaStream_t s);
+                          int PxDf, const int* fexp, int* emax, cudaStream_t s);
 // One pass in parity order: both blocks of T^{-1} (which = 0) or T along
 // `axis` as one CTA-pair launch (tc_pair_kernels.cu).  Writes the split array
 // `out` (EPI_STORE, or EPI_DIV with lambdas in mode order) or, with out32 (the
