@@ -440,9 +440,9 @@ def run_ours(args, rank: int, world: int, local_rank: int):
 
     # ---- roofline of the dominant kernel (tcgen05 BF16x3 mode product)
     tc_avg_ms = tc_ms / max(1, tc_n)
-    # 3 bf16 products per useful multiply-add; refined solves on 255 nodes an axis
-    # and more run their passes in parity order
-    parity = args.sweeps >= 2 and n >= 255
+    # 3 bf16 products per useful multiply-add; solves in parity order fold and
+    # unfold around every set of passes, the others convert f once
+    parity = sp_n > args.steps
     flops_per_launch = 3 * mode_flops(n, parity)
     achieved = flops_per_launch / (tc_avg_ms / 1e3) / 1e12
     peak = float(peaks.get("bf16_tflops_sustained", PEAKS_FALLBACK["bf16_tflops_sustained"]))

@@ -393,15 +393,22 @@ sem3d_status solve_once_bf16x3(sem3d_plan* p, TcBuffers S0, TcBuffers S1, double
 // Where it is used: split-bf16 solves with at least two refinement sweeps,
 // whose result no longer depends on how the correction solves round (a bare
 // solve's 1e-5 and one sweep's 1e-8 do, and keep the node-order passes), on
-// grids of at least 255 nodes along every axis.  Below, the passes are bound
-// by memory and latency instead of the tensor cores and the folding kernels
-// cost what is saved.  Refined solves, node order -> parity order: n = 127
-// 377 -> 421 us, 255 1647 -> 1644 (a group of 16 problems, most of them 255
-// and larger, 52.0 -> 51.3 ms), 383 5455 -> 5160, 511 12.6 -> 11.5 ms, 767
-// 49.7 -> 42.7 ms, 999 133.8 -> 102.8 ms; 511x63x255 978 -> 1007 us.
-constexpr int kFoldMin = 255;
+// grids of at least 255 nodes along every axis and more than 256 along one.
+// An axis of at most 256 is one output tile in either order, so parity order
+// saves it no pass over the data, and the folding kernels cost more than the
+// smaller products save.  Refined solves, k = 4, node order -> parity order in us:
+//   159^3 642 -> 640, 191^3 826 -> 853, 223^3 1128 -> 1202, 239^3 1330 -> 1406,
+//   255^3 1528 -> 1554, 263^3 2435 -> 2235, 287^3 2781 -> 2588, 383^3 5256 ->
+//   4972, 511^3 12.2 -> 11.2 ms, 767^3 47.5 -> 42.2, 999^3 135.5 -> 103.8;
+//   k = 1: 256^3 1239 -> 1283, 257^3 1899 -> 1620.
+// One axis longer, the others 255: 255x255x263 1709 -> 1621, 263x255x255 2005
+// -> 2051, 383 either way 1% faster, 511 within 2%.  An axis below 255 beside
+// longer ones: 599x599x191 7.12 -> 6.79 ms, 599x599x127 4.73 -> 4.59,
+// 127x599x599 4.51 -> 4.56, 255x255x127 837 -> 869 us (not taken).
+constexpr int kFoldMin = 255, kFoldLongest = 256;
 bool use_fold(const sem3d_plan* h) {
-  return h->prec == SEM3D_BF16X3 && h->sweeps >= 2 && std::min(h->g.nx, std::min(h->g.ny, h->g.nz)) >= kFoldMin;
+  return h->prec == SEM3D_BF16X3 && h->sweeps >= 2 && std::min(h->g.nx, std::min(h->g.ny, h->g.nz)) >= kFoldMin &&
+         std::max(h->g.nx, std::max(h->g.ny, h->g.nz)) > kFoldLongest;
 }
 
 // Its workspace, inside the node-order path's: two split arrays at the parity

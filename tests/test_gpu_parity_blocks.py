@@ -161,3 +161,24 @@ def test_double_fp32_residual_in_pairs(k, ne3):
         p.sync_check()
     ref = refined_solve(F, *axes, c, 1)
     assert np.abs(u.cpu().numpy() - ref).max() / np.abs(ref).max() <= max(1e-12, kappa(axes, c) * 2.0**-48)
+
+
+def test_parity_order_where_an_axis_has_more_than_one_tile():
+    # the orders launch different numbers of kernels per solve
+    from paper_2310_00226_gb300 import sem3d
+
+    def launches(n3):
+        f = torch.ones(n3[::-1], dtype=torch.float64, device="cuda")
+        u = torch.empty_like(f)
+        with sem3d.Plan(*n3, 1, (1.0, 1.0, 1.0), 1.0) as p:
+            p.set_precision("bf16x3", 3)
+            p.solve(f, u)
+            before = p.launch_count()
+            p.solve(f, u)
+            p.sync_check()
+            return p.launch_count() - before
+
+    node, parity = launches((254, 300, 300)), launches((300, 257, 255))
+    assert node != parity
+    assert launches((255, 256, 256)) == launches((255, 255, 255)) == node
+    assert launches((255, 255, 257)) == launches((257, 255, 255)) == launches((255, 257, 256)) == parity
