@@ -75,8 +75,9 @@ typedef enum {
  * T^-1 split into blocks acting on the even and the odd part of a field, which
  * is half the work.  In use for every FP64 product, for FP32 with two sweeps
  * or more, and for BF16X3 with two sweeps or more on at least 255 nodes along
- * every axis and more than 256 along one (results that do not depend on how a
- * correction solve rounds).
+ * every axis and more than 256 along one (there the blocks leave a refined
+ * result's error as it is; a bare solve's or one sweep's is the rounding of the
+ * products themselves, and stays that of the full matrices).
  * FP64 accuracy is recovered by iterative refinement (sem3d_set_precision). */
 typedef enum {
   SEM3D_FP64 = 0,

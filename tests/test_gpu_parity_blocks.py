@@ -182,3 +182,33 @@ def test_parity_order_where_an_axis_has_more_than_one_tile():
     assert node != parity
     assert launches((255, 256, 256)) == launches((255, 255, 255)) == node
     assert launches((255, 255, 257)) == launches((257, 255, 255)) == launches((255, 257, 256)) == parity
+
+
+# Two sweeps are the fewest that take parity order; with the mixed schedule the
+# first update then goes from the double-FP32 pair straight to FP64, without the
+# pair's low parts.  Bound: the error falls from the bare solve's e0 to one
+# sweep's e1 (both in node order, measured here) by e1 / e0, and the next sweep
+# may do up to four times worse: 4 e1^2 / e0, some 1e-11 (stale or missing low
+# parts would be 1e-8).
+@pytest.mark.parametrize("n3,k", [((271, 263, 299), 4), ((272, 258, 264), 1), ((257, 275, 260), 3)])
+def test_two_sweeps_in_parity_order(n3, k):
+    from paper_2310_00226_gb300 import sem3d
+    L, c = (1.0, 1.3, 0.8), 1.5
+    F = random_rhs(*n3, seed=k)
+    ref = refined_solve(F, *[sem_1d(k, (n + 1) // k, 0.0, Lb) for n, Lb in zip(n3, L)], c, 1)
+    f = torch.from_numpy(F).cuda()
+    u, v = torch.empty_like(f), torch.empty_like(f)
+    err = lambda: np.abs(u.cpu().numpy() - ref).max() / np.abs(ref).max()  # noqa: E731
+    with sem3d.Plan(*n3, k, L, c) as p:
+        e = []
+        for sweeps in (0, 1, 2):
+            u.fill_(float("nan"))
+            p.set_precision("bf16x3", sweeps)
+            p.solve(f, u)
+            p.sync_check()
+            e.append(err())
+        assert e[2] <= 4 * e[1] ** 2 / e[0], e
+        v.fill_(float("nan"))
+        sem3d.solve_batched([p], [f], [v])
+        p.sync_check()
+        assert torch.equal(u, v)
