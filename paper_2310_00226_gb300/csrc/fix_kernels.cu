@@ -155,13 +155,27 @@ __device__ __forceinline__ void fx1(long long& P2, long long& P1, int ch, int cl
   P1 += (long long)cl * uh;
 }
 
+// What the residual is written as: bf16 hi / lo, FP64 (pitch nx) or FP32, known
+// at compile time, or FIX_ANY: as the pointers say.  The kernels are at register
+// limits, and a branch costs the vector kernel 2.4% (n = 511, k = 4 1973 -> 2020
+// us).  FIX_ANY remains where it is the faster one: k = 5 but for bf16 (n = 384
+// FP64 1.73 ms against 1.90, FP32 1.59 against 1.69: 64 registers against 66) and
+// k = 1 to FP64 (n = 511 2.04 against 2.07 ms).
+enum : int { FIX_SPLIT, FIX_F64, FIX_F32, FIX_ANY };
+
+template <int OUT>
+__device__ __forceinline__ bool writes(const FixArgs& a, int what) {
+  if (OUT != FIX_ANY) return OUT == what;
+  return what == FIX_F64 ? a.out64 != nullptr : what == FIX_F32 ? a.out32 != nullptr : !a.out64 && !a.out32;
+}
+
 // Fixed-point residual for k in {1, 2, 4} with Dirichlet rows.  Layout as
 // the double-FP32 vector residual: a warp per (j, l) line, a lane per 4
 // consecutive nodes i = 4c .. 4c+3 (one int4 of Uh and one of Ul); since
 // 4 % k == 0 node 4c+p has local index (p+1) % k, so the x rows and their
 // folding are known at compile time.  The y and z rows depend on the warp's
 // (j, l) and are read from the term tables.
-template <int K>
+template <int K, int OUT>
 __global__ void __launch_bounds__(256, 4) stencil_fix4_kernel(FixArgs a, const __grid_constant__ FixCoef cf) {
   constexpr int BW = 2 * K + 1;
   const int lane = threadIdx.x & 31;
@@ -258,7 +272,7 @@ __global__ void __launch_bounds__(256, 4) stencil_fix4_kernel(FixArgs a, const _
         const long long T = P2[p] + ((P1[p] + ((long long)Q[p] << 3) + kHalf) >> kChunk);
         R[p] = (i0 + p < a.nx) ? f64_to_fixed(__ldg(frow + i0 + p), sF) - T : 0;
       }
-      if (a.out64) {  // FP64 r at pitch nx
+      if (writes<OUT>(a, FIX_F64)) {  // r at pitch nx
         double* orow = a.out64 + line * a.nx;
 #pragma unroll
         for (int p = 0; p < 4; ++p)
@@ -270,7 +284,7 @@ __global__ void __launch_bounds__(256, 4) stencil_fix4_kernel(FixArgs a, const _
       for (int p = 0; p < 4; ++p)  // pads stay zero
         r[p] = (i0 + p >= a.nx) ? 0.f : finite ? fixed_to_f32(R[p], X) : __int_as_float(0x7FC00000);
       const long long o = line * a.Px + i0;
-      if (a.out32) {
+      if (writes<OUT>(a, FIX_F32)) {
         *reinterpret_cast<float4*>(a.out32 + o) = make_float4(r[0], r[1], r[2], r[3]);
         continue;
       }
@@ -297,7 +311,7 @@ __global__ void __launch_bounds__(256, 4) stencil_fix4_kernel(FixArgs a, const _
 // from the term tables at its (j, l).  The thread of a line's last element
 // also writes the line's pad columns (zeros).  Same arithmetic as
 // stencil_fix4_kernel.
-template <int K>
+template <int K, int OUT>
 __global__ void __launch_bounds__(256) stencil_fix_elem_kernel(FixArgs a, const __grid_constant__ FixCoef cf,
                                                                int nex) {
   constexpr int BW = 2 * K + 1;
@@ -384,12 +398,12 @@ __global__ void __launch_bounds__(256) stencil_fix_elem_kernel(FixArgs a, const 
       if (i < 0) continue;
       const long long T = P2[q] + ((P1[q] + ((long long)Q[q] << 3) + kHalf) >> kChunk);
       const long long R = f64_to_fixed(__ldg(frow + i), sF) - T;
-      if (a.out64) {  // FP64 r at pitch nx
+      if (writes<OUT>(a, FIX_F64)) {  // r at pitch nx
         a.out64[jl * a.nx + i] = finite ? ldexp((double)R, X) : __longlong_as_double(0x7FF8000000000000LL);
         continue;
       }
       const float r = finite ? fixed_to_f32(R, X) : __int_as_float(0x7FC00000);
-      if (a.out32) {
+      if (writes<OUT>(a, FIX_F32)) {
         a.out32[row + i] = r;
         continue;
       }
@@ -397,7 +411,7 @@ __global__ void __launch_bounds__(256) stencil_fix_elem_kernel(FixArgs a, const 
       a.hi[row + i] = h16;
       a.lo[row + i] = __float2bfloat16_rn(r - __bfloat162float(h16));
     }
-    if (ex == nex - 1 && !a.out64 && !a.out32)
+    if (ex == nex - 1 && writes<OUT>(a, FIX_SPLIT))
       for (int i = a.nx; i < a.Px; ++i) {
         a.hi[row + i] = __float2bfloat16_rn(0.f);
         a.lo[row + i] = __float2bfloat16_rn(0.f);
@@ -411,7 +425,10 @@ cudaError_t launch_fix_elem(const FixArgs& a, const FixCoef& cf, cudaStream_t s)
   const long long total = (long long)nex * a.ny * a.nz;
   long long b = (total + 255) / 256;  // one thread per element and line, in order (see launch_fix4)
   if (b > 0x7FFFFFFFLL) b = 0x7FFFFFFFLL;
-  stencil_fix_elem_kernel<K><<<(unsigned)(b < 1 ? 1 : b), 256, 0, s>>>(a, cf, nex);
+  const unsigned g = (unsigned)(b < 1 ? 1 : b);
+  if (a.out64) stencil_fix_elem_kernel<K, K == 5 ? FIX_ANY : FIX_F64><<<g, 256, 0, s>>>(a, cf, nex);
+  else if (a.out32) stencil_fix_elem_kernel<K, K == 5 ? FIX_ANY : FIX_F32><<<g, 256, 0, s>>>(a, cf, nex);
+  else stencil_fix_elem_kernel<K, FIX_SPLIT><<<g, 256, 0, s>>>(a, cf, nex);
   return cudaGetLastError();
 }
 
@@ -422,7 +439,10 @@ cudaError_t launch_fix4(const FixArgs& a, const FixCoef& cf, cudaStream_t s) {
   const long long lines = (long long)a.ny * a.nz;
   long long blocks = (lines + 7) / 8;
   if (blocks > 0x7FFFFFFFLL) blocks = 0x7FFFFFFFLL;
-  stencil_fix4_kernel<K><<<(unsigned)(blocks < 1 ? 1 : blocks), 256, 0, s>>>(a, cf);
+  const unsigned g = (unsigned)(blocks < 1 ? 1 : blocks);
+  if (a.out64) stencil_fix4_kernel<K, K == 1 ? FIX_ANY : FIX_F64><<<g, 256, 0, s>>>(a, cf);
+  else if (a.out32) stencil_fix4_kernel<K, FIX_F32><<<g, 256, 0, s>>>(a, cf);
+  else stencil_fix4_kernel<K, FIX_SPLIT><<<g, 256, 0, s>>>(a, cf);
   return cudaGetLastError();
 }
 
