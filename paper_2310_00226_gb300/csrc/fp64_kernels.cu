@@ -40,8 +40,7 @@ struct F64Pass {
   double c;
 };
 
-// Half of x off the FP64 pipe and without a branch (one would keep the loads
-// from staying in flight): one off the exponent; below 2^-1021 the magnitude's
+// Half of x off the FP64 pipe, which bounds the passes: one off the exponent; below 2^-1021 the magnitude's
 // bits shifted, the last one dropped; infinities and NaN as they are.
 __device__ __forceinline__ double half_of(double x) {
   const unsigned int h = (unsigned int)__double2hiint(x), w = (unsigned int)__double2loint(x);
@@ -84,12 +83,11 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
       if (abase[it] && t < p.ne) {
         u = abase[it][(long long)t * p.sm];
         if (t < p.no) v = abase[it][(long long)(FWD ? p.n - 1 - t : p.ne + t) * p.sm];
-        if (HALF) { u = half_of(u); v = half_of(v); }  // no sum of a mirrored pair overflows
       }
       // the middle node of an odd n (t = no) has no partner: v = 0 and the
       // odd block has no such column
-      ra[it][0] = FWD ? u + v : u;
-      ra[it][1] = FWD ? (t < p.no ? u - v : 0.0) : v;
+      ra[it][0] = FWD && !HALF ? u + v : u;
+      ra[it][1] = FWD && !HALF ? (t < p.no ? u - v : 0.0) : v;
     }
 #pragma unroll
     for (int it = 0; it < LW; ++it) {
@@ -99,13 +97,19 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
       rw[it] = (o < m && t < m) ? __ldg(p.W + (par == 0 ? 0 : (long long)p.ne * p.ne) + (long long)o * m + t) : 0.0;
     }
   };
-  auto store = [&]() {
+  auto store = [&](int t0) {
 #pragma unroll
     for (int it = 0; it < LA; ++it) {
       const int e = tid + it * 256;
       const int kk = KCONTIG ? e % F64_BK : e / BM, r = KCONTIG ? e / F64_BK : e % BM;
-      As[0][kk][r] = ra[it][0];
-      As[1][kk][r] = ra[it][1];
+      if (HALF) {  // no sum of a mirrored pair overflows (here: the loads stay in flight)
+        const double u = half_of(ra[it][0]), v = half_of(ra[it][1]);
+        As[0][kk][r] = u + v;
+        As[1][kk][r] = t0 + kk < p.no ? u - v : 0.0;
+      } else {
+        As[0][kk][r] = ra[it][0];
+        As[1][kk][r] = ra[it][1];
+      }
     }
 #pragma unroll
     for (int it = 0; it < LW; ++it) {
@@ -123,7 +127,7 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
   pdl_wait();
   load(0);
   for (int t0 = 0; t0 < p.ne; t0 += F64_BK) {
-    store();
+    store(t0);
     __syncthreads();
     if (t0 + F64_BK < p.ne) load(t0 + F64_BK);
 #pragma unroll
@@ -146,7 +150,7 @@ __global__ void __launch_bounds__(256) mode_product_f64_kernel(F64Pass p) {
   // wc + 2*(lane%4) + {0,1} of both parities.
   auto put = [&](long long base, int o, double v) {
     const long long idx = base + (long long)o * p.sm;
-    if (p.epi == EPI_DIV) {
+    if (FWD && KCONTIG && p.epi == EPI_DIV) {
       const long long i = idx % p.nx, jl = idx / p.nx;
       const long long j = jl % p.ny, l = jl / p.ny;
       p.out[idx] = v / half_of(p.lamx[i] + p.lamy[j] + p.lamz[l] + p.c);  // of halved right-hand sides
@@ -518,6 +522,7 @@ cudaError_t launch_mode_product_f64(const Geom& g, int axis, const DevAxis* ax, 
   } else {                 // rows = (i,j) plane, t = l
     p.R1 = (int)nxy; p.R2 = 1; p.s1 = 1; p.s2 = 0; p.sm = nxy;
   }
+  if (epi == EPI_DIV && (axis != 0 || which != 0)) return cudaErrorInvalidValue;
   if (epi == EPI_HALF) {  // the first pass of a solve
     if (kcontig || which != 0) return cudaErrorInvalidValue;
     return launch_f64<false, true, true>(p, num_sms, s);
