@@ -113,9 +113,9 @@ typedef enum { SEM3D_BC_DIRICHLET = 0, SEM3D_BC_NEUMANN = 1 } sem3d_bc;
  * face; the unknowns are all n = Ne*k + 1 GLL nodes of each axis, so each n
  * must satisfy (n-1) % k == 0 and n > k, nodes run from 0 to L inclusive,
  * and c > 0 is required (lambda = 0 belongs to the constant mode).  Neumann
- * plans compute every refinement residual in FP64 with the per-row banded
- * operator (SEM3D_RESIDUAL_MIXED acts as SEM3D_RESIDUAL_FP64) and do not
- * support SEM3D_F16X3 (SEM3D_ERR_UNSUPPORTED). */
+ * plans compute every refinement residual in FP64 (by elements for k <= 8, with
+ * the per-row banded operator above; SEM3D_RESIDUAL_MIXED acts as
+ * SEM3D_RESIDUAL_FP64) and do not support SEM3D_F16X3 (SEM3D_ERR_UNSUPPORTED). */
 sem3d_status sem3d_setup_bc(int nx, int ny, int nz, int k, double Lx, double Ly, double Lz, double c, sem3d_bc bc,
                             sem3d_handle* out);
 

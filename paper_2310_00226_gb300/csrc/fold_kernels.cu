@@ -17,10 +17,11 @@
 // and corrections scaled to match (powers of two: the same digits).  (Folding
 // everything at 1/8 would cost the other end of the range: the low bf16 part of
 // values below 1e-25.)  For all others that is one launch, 3 us, whose blocks
-// return at once.  Both kernels are bound by
-// HBM: at n = 999 fold 1.9 ms from FP64 (12 B per node, 6.3 TB/s) and 1.13 ms
-// from FP32, unfold 2.85 ms into FP64 and 2.9 ms into the double-FP32 pair
-// (20 B, 7 TB/s), 3.9 ms from the pair into FP64.
+// return at once.  Both kernels are bound by HBM, the updates of the
+// double-FP32 pair by too few warps waiting for it (48 to 80 registers): at
+// n = 999 fold 1.9 ms from FP64 (12 B per node, 6.3 TB/s) and 1.14 ms from FP32
+// (8 B, 7.0), unfold 2.85 ms into FP64 (20 B, 7.0), 1.6 ms into the pair (8 B,
+// 5.0), 2.9 ms added to it (16 B, 5.6), 4.0 ms from the pair into FP64 (20 B, 5.0).
 #include <algorithm>
 
 #include "tc_common.cuh"

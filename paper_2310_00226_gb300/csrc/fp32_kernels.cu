@@ -4,7 +4,9 @@
 // transposes): C[row, o] = sum_t A[row, t] * W[o, t], rows enumerated by two
 // loops (p < R1 stride s1, q < R2 stride s2), axis stride sm.
 //
-// Bound by the FP32 pipe (74 TF/s).  A CTA of 256 threads computes a BM x BN
+// Bound by the shared-memory reads that feed the FP32 pipe, at two blocks of
+// 126 registers a thread (n = 383: pipe 53% busy, shared memory 70%; n = 767 with
+// full matrices 46 of 74 TF/s).  A CTA of 256 threads computes a BM x BN
 // output tile; each thread owns TM rows (in pairs of neighbours, so that a
 // packed f32x2 multiply-add serves two rows; the packed form has the scalar
 // one's lane rate for half the issue slots, which leaves room for the shared-
